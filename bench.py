@@ -36,13 +36,14 @@ POP_BYTES = {"fp64": 8, "fp32": 4, "fp16dev": 2}
 
 def kernels_per_step(nb, mpf, variant):
     """Kernel launches of one step of the library's graph: density + bulk collision (variant 0), the
-    fused pass (1), or the edge fix-up + accumulating collision (2); the closing kernel (fluid mass,
-    buffer flip); with bodies the tile pass of psi (variants 1 and 2), the collision of the cells
-    next to a solid, the force pass, repulsion (two or more bodies), body update, three advection
-    sweeps, kinetics (MPF on), flags and refill."""
-    k = (1 if variant == 1 else 2) + 1
+    fused pass (1), the edge fix-up + accumulating collision (2), or the moment pass (3); the closing
+    kernel (fluid mass, buffer flip); with bodies the tile pass of psi (variants 1 and 2) or the fill and
+    the close of the moment pass (3: it ends the step), the collision of the cells next to a solid, the force pass,
+    repulsion (two or more bodies), body update, three advection sweeps, kinetics (MPF on), flags and
+    refill."""
+    k = (1 if variant in (1, 3) else 2) + 1
     if nb:
-        k += (1 if variant in (1, 2) else 0) + 1 + 1 + (1 if nb > 1 else 0) + 1 + 3 + (1 if mpf else 0) + 2
+        k += {0: 0, 1: 1, 2: 1, 3: 1}[variant] + 1 + 1 + (1 if nb > 1 else 0) + 1 + 3 + (1 if mpf else 0) + 2
     return k
 
 
@@ -59,11 +60,11 @@ PROFILED_STEP = {
 
 
 def source_hash():
-    """sha1 prefix of the lattice-Boltzmann kernels' sources (lbm.cu and the shared device headers)."""
+    """sha1 prefix of the lattice-Boltzmann kernels' sources (lbm.cu, moments.cuh, the shared device headers)."""
     import hashlib
 
     h = hashlib.sha1()
-    for name in ("lbm.cu", "cbl_dev.cuh", "periodic.h", "weights.h"):
+    for name in ("lbm.cu", "moments.cuh", "cbl_dev.cuh", "periodic.h", "weights.h"):
         with open(os.path.join(ROOT, "paper_1902_10432_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:12]
@@ -77,8 +78,10 @@ def profiled_step_traffic(workload_name, prec, q=19):
     return PROFILED_STEP.get((workload_name, prec, q, source_hash()))
 
 
-def alg_bytes_per_cell(prec, q=19):
-    return 2 * q * POP_BYTES[prec] + 2
+def alg_bytes_per_cell(prec, q=19, variant=0):
+    """Bytes a step has to move per cell: the populations once in and once out and the flag, or with the
+    moment pass (3) density, momentum and psi once in and once out and the flag."""
+    return (40 if variant == 3 else 2 * q * POP_BYTES[prec]) + 2
 
 
 HBM_DATASHEET_GBS = 7900.0  # GB300 HBM3e nominal
@@ -278,6 +281,7 @@ def bench_batch(args, rank, world, local_rank):
     batch = cbl.Batch(sims)
     tile, tile_ms = autotune.tune_batch(batch, steps=3)
     binfo = batch.info()
+    variants = [3 if s.get_option("lbm_variant") == 3 else 0 for s in sims]  # the pass of each in the batch
     batch.step(args.warmup)
     batch.sync()
     ev0 = torch.cuda.Event(enable_timing=True)
@@ -311,9 +315,11 @@ def bench_batch(args, rank, world, local_rank):
             "sequential_mlups": cells * args.steps / seq_s / 1e6,
             "speedup_vs_sequential": seq_s / bat_s, "clocks": clk.summary(),
             # persistent mode: one launch for the bulk pass of all instances, then each instance's side
-            # chain (its step without the density and bulk collision kernels)
-            "gpu_launches": args.steps * ((1 + len(ws) * (kernels_per_step(2, 1, False) - 2)) if binfo["mode"] == 1
-                                          else sum(n * kernels_per_step(2, 1, 1 if json.loads(c).get("lbm_variant") == 1 else 0)
+            # chain (its step without the density and bulk collision kernels, or with the moment pass
+            # without that and the collision of the cells next to a solid)
+            "gpu_launches": args.steps * ((len(set(variants)) + sum(kernels_per_step(2, 1, v) - 2 for v in variants))
+                                          if binfo["mode"] == 1
+                                          else sum(n * kernels_per_step(2, 1, json.loads(c).get("lbm_variant", 0))
                                                    for c, n in choices.items()))}
     if rk.root:
         print(json.dumps(line), flush=True)
@@ -497,7 +503,7 @@ def bench_cuda(args, rank, world, local_rank):
 
     if rank == 0:
         peak, peak_kind = measured_peaks()
-        bpc = alg_bytes_per_cell(prec, args.q)
+        bpc = alg_bytes_per_cell(prec, args.q, variant)
         achieved = bpc * w.ncells / (t_kernel_ms * 1e-3) / 1e9
         step_achieved = bpc * w.ncells / (ms_med / args.steps * 1e-3) / 1e9
         step_traffic = profiled_step_traffic(w.name, prec, args.q)
@@ -516,7 +522,9 @@ def bench_cuda(args, rank, world, local_rank):
             "roofline": {"bound": "hbm", "kernel": {0: "bulk collision (k_collide: pull, force, BGK, store)",
                                                     1: "fused pass (k_fused: psi of the plane ahead, collision)",
                                                     2: "accumulating collision (k_collide_acc: collision and "
-                                                       "next step's density)"}[variant],
+                                                       "next step's density)",
+                                                    3: "moment pass (k_mom: force, collision, streaming; bound by "
+                                                       "instruction issue)"}[variant],
                          "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                          "traffic": profiled_traffic(w.name, prec, args.q), "peak_kind": peak_kind,
                          "peak_datasheet": HBM_DATASHEET_GBS, "alg_bytes_per_cell": bpc,
@@ -575,7 +583,7 @@ def main():
                     help="cap on warm-up plus timed steps (the workloads evolve with time)")
     ap.add_argument("--option", action="append", default=[],
                     help="execution option key=value for the timed simulation (cbl_set_option), repeatable")
-    ap.add_argument("--lbm-variant", type=int, default=None, choices=[0, 1, 2],
+    ap.add_argument("--lbm-variant", type=int, default=None, choices=[0, 1, 2, 3],
                     help="lattice-Boltzmann pass: 0 split density + collision, 1 fused, 2 accumulating "
                          "(default: the library's)")
     args = ap.parse_args()

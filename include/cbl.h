@@ -214,7 +214,7 @@ cbl_status cbl_info(cbl_ctx* ctx, int* nbodies, int64_t* ncells, int* device_err
 
 /* Phases of one step, in launch order, as reported by cbl_time_phases. */
 #define CBL_NPHASES 9
-/* 0 psi of the step: pull + density + psi (split pass), psi of the bodies' tiles (fused pass,
+/* 0 psi of the step: pull + density + psi (split pass), nothing (moment pass, "lbm_variant" 3), psi of the bodies' tiles (fused pass,
  * "lbm_variant" 1), the regions' edge cells and the tiles (accumulating pass, 2); 1 collision:
  * pull + force + collision + mass partials, bulk and next to a solid (the fused pass also computes
  * psi, the accumulating pass the next step's density); 2 solid-fluid force on the bodies (momentum
@@ -239,7 +239,7 @@ cbl_status cbl_kernel_times(cbl_ctx* ctx, int max, float* ms, int* count);
  *   "lbm_variant"  how each step computes the density and psi that the Shan-Chen force needs
  *                  (Sec. 3.2.3: psi of the post-streaming density at every neighbour):
  *                  0 = split pass: a density kernel pulls every cell, then the collision kernel
- *                  pulls it again (default);
+ *                  pulls it again (default where the moment pass is not);
  *                  1 = fused pass: one kernel marches along z, producer warps compute psi of the
  *                  plane ahead into shared memory, consumer warps collide;
  *                  2 = accumulating pass: the collision kernel also sums the next step's density
@@ -247,7 +247,14 @@ cbl_status cbl_kernel_times(cbl_ctx* ctx, int max, float* ms, int* count);
  *                  of 32 x acc_ty columns x acc_sz planes); the next step completes psi of the
  *                  regions' edge cells from the populations of their outside sources and of the
  *                  bodies' tiles from the populations. Each step pulls the populations once. A
- *                  batch (cbl_batch_*) runs its instances with the split pass;
+ *                  batch (cbl_batch_*) runs such instances with the split pass;
+ *                  3 = moment pass (default at tau = 1 with FP32 or binary16 storage on 2^19 cells or
+ *                  more; CBL_ERR_UNSUPPORTED at another tau or in FP64): at tau = 1 the post-collision
+ *                  populations are functions of density, momentum and force, so the cells away from a
+ *                  solid carry density and momentum (16 + 4 bytes per cell, two buffers, allocated at
+ *                  the first step; without room for them the split pass runs) and populations are
+ *                  stored next to the solids only. cbl_read_populations, cbl_save, cbl_move_bodies
+ *                  write out all populations first; binary16 storage rounds as before;
  *   "fused_ty"     y extent of a fused block's consumer tile: 4 or 8 (default);
  *   "fused_tz"     z extent of a fused block (0 = derived from the SM count);
  *   "acc_ty"       y extent of an accumulating region: 8 (default) or 16;
@@ -299,8 +306,10 @@ cbl_status cbl_lbm_step_noalloc(const float* f_in, float* f_out, int nx, int ny,
 /* Batches: advance many independent contexts (lattices of any size, each with its own bodies and
  * parameters) with one call; one captured CUDA graph holds one step of every instance.
  * Persistent mode (mode 1, the default when every instance has the same precision and velocity set
- * and uses the split pass): the step of all instances starts with ONE launch of a persistent kernel
+ * and uses the split or moment pass): the step of all instances starts with ONE launch of a persistent kernel
  * that computes psi and then the bulk collision of every cell of every instance (Sec. 3.2.1, 3.2.3):
+ * (for the instances on the moment pass, "lbm_variant" 3, a launch of its own: the cells next to a
+ * solid, the barrier, then the bulk);
  * its grid is as large as the GPU holds resident blocks, each block takes work items (a tile of one
  * instance; tile shape from "tile", picked by the project's autotuner) from a device queue, and the
  * two phases are separated by a grid barrier whose wait is bounded (option "spin_limit", clock64
@@ -320,7 +329,8 @@ cbl_status cbl_batch_step(cbl_batch* batch, int nsteps);
  * out since the last call (the error word is cleared). */
 cbl_status cbl_batch_sync(cbl_batch* batch);
 /* Batch options (synchronises, rebuilds the graphs): "mode" 0 or 1; "tile" 0..3, the persistent
- * kernel's tile of x * y * z cells: 32*4*1, 32*4*4 (default), 32*4*8, 64*2*4; "spin_limit" the
+ * kernel's tile of x * y * z cells: 32*4*1, 32*4*4 (default), 32*4*8, 64*2*4 (moment pass: columns of
+ * 16, 32, 64 or 24 planes); "spin_limit" the
  * barrier wait limit in clock64 cycles (0 makes every wait run out at once: a test of the timeout
  * path). CBL_ERR_UNSUPPORTED for mode 1 over mixed precisions or velocity sets. */
 cbl_status cbl_batch_set_option(cbl_batch* batch, const char* key, double value);

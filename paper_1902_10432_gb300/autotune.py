@@ -2,7 +2,8 @@
 tile shape of the persistent batch kernel for a batch.
 
 Candidates for one lattice: the split density + collision kernels with 128-thread blocks of x extent
-32, 64 or 128, the fused single pass, and the accumulating pass with regions 8 or 16 rows deep. For a batch (tune_batch): the persistent kernel's tile
+32, 64 or 128, the fused single pass, the accumulating pass with regions 8 or 16 rows deep, and at
+tau = 1 the moment pass. For a batch (tune_batch): the persistent kernel's tile
 shapes 32x4x1, 32x4x4, 32x4x8 and 64x2x4 cells. Each candidate is timed on the simulation it will run
 (three warm-up steps, then CUDA events around a few steps on the simulation's stream; the state
 advances, which does not matter for the choice); the fastest is applied and cached in a JSON file
@@ -23,6 +24,8 @@ def candidates(prec):
     c = [dict(lbm_variant=0, lbm_block_x=bx) for bx in (32, 64, 128)]
     c.append(dict(lbm_variant=1, lbm_block_x=32))
     c += [dict(lbm_variant=2, lbm_block_x=32, acc_ty=ty) for ty in (8, 16)]
+    if prec != "fp64":
+        c.append(dict(lbm_variant=3, lbm_block_x=32))  # only at tau = 1: left out elsewhere by tune()
     return c
 
 
@@ -32,8 +35,8 @@ def _key(sim):
     nx = sim.shape[2]
     ny = sim.shape[1]
     nz = sim.shape[0]
-    return "%dx%dx%d/%s/%s/%s" % (nx, ny, nz, sim.params["prec"], "bodies" if sim.nb else "fluid",
-                                  torch.cuda.get_device_name())
+    return "%dx%dx%d/%s/tau%g/%s/%s" % (nx, ny, nz, sim.params["prec"], sim.params["tau"],
+                                        "bodies" if sim.nb else "fluid", torch.cuda.get_device_name())
 
 
 def _load():
@@ -63,6 +66,8 @@ def tune(sim, steps=6, use_cache=True):
     best, best_ms = None, float("inf")
     s = sim.stream
     for cand in candidates(sim.params["prec"]):
+        if cand["lbm_variant"] == 3 and sim.params["tau"] != 1.0:
+            continue
         apply(sim, cand)
         sim.step(3)
         e0 = torch.cuda.Event(enable_timing=True)
@@ -88,6 +93,7 @@ def tune(sim, steps=6, use_cache=True):
     return best, results
 
 
+# of the split pass; the moment pass's columns of 32 x 8 cells have 16, 32, 64 and 24 planes
 BATCH_TILES = {0: (32, 4, 1), 1: (32, 4, 4), 2: (32, 4, 8), 3: (64, 2, 4)}
 
 

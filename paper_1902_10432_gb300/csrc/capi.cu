@@ -67,6 +67,13 @@ struct cbl_ctx {
   int acc_sz = 0;          // z extent in use
   int acc_attr_ty = 0;     // region depth whose kernel has its shared-memory limit set
   void *psi2 = nullptr, *rhop = nullptr;
+  // moment pass (lbm_variant 3, moments.cuh): -1 chosen by mom_rule, 0 off, 1 on
+  int mom_req = -1;
+  bool mom = false;        // the step graph runs the moment pass
+  bool mom_state = false;  // the state is in moments (populations complete only after mom_leave)
+  int mom_sz = 0;          // planes per block
+  MomDev md = {};
+  MomDev md_step() const { return mom ? md : MomDev{}; }
   bool psi_valid = false;  // psi of the current step is in place (else a whole-lattice density pass first)
   int fused_tz = 0;      // > 0: the density and the bulk collision run as one fused pass (k_fused)
   int fused_tz_req = 0;  // requested z extent of a fused block (0 = derived)
@@ -377,7 +384,7 @@ static cbl_status init_common(cbl_ctx* ctx, const double* rho_host, const double
     launch_rasterize(ctx->lat, ctx->db, nb, ctx->max_tile, ctx->arena, ctx->p.eta, ctx->s);
     launch_neighbour_lists(ctx->db, nb, ctx->lat, ctx->st, ctx->s);
     launch_flags(ctx->lat, ctx->db, nb, ctx->max_tile, ctx->arena, ctx->flags, ctx->p.solid_threshold, 1, ctx->st,
-                 ctx->s);
+                 MomDev{}, ctx->s);
     launch_body_props(ctx->lat, ctx->db, nb, ctx->max_tile, ctx->arena, ctx->scratch, ctx->s);
   }
   double* drho = (double*)dalloc(ctx, N * 8);
@@ -442,6 +449,16 @@ cbl_status cbl_init_fluid_fields(cbl_ctx* ctx, const double* rho_host, const dou
 // phases: 1 density (fused pass: psi over the bodies' tiles only), 2 bulk collision (fused pass:
 // with the density), 4 collision of the cells next to a solid
 static void enqueue_lbm(cbl_ctx* ctx, int phases, cudaStream_t s) {
+  if (ctx->mom) {
+    // moment pass: no density phase; the cells next to a solid collide first, the bulk pulls from them
+    if (phases & 4)
+      ctx->ops.mom_near(ctx->prec, ctx->lat, ctx->fa, ctx->fb, ctx->flags, ctx->psi, ctx->psi2, ctx->db, ctx->mass_part,
+                        ctx->st, ctx->diag_rho, ctx->diag_vel, ctx->pp, ctx->nbuf, ctx->blist, s);
+    if (phases & 2)
+      ctx->ops.mom(ctx->prec, ctx->lat, ctx->fa, ctx->fb, ctx->flags, ctx->psi, ctx->psi2, ctx->md, ctx->mass_part,
+                   ctx->st, ctx->diag_rho, ctx->diag_vel, ctx->pp, ctx->mom_sz, s);
+    return;
+  }
   if (ctx->acc_pass) {
     // accumulating pass: phase 1 completes psi of this step (the regions' edge cells, then the bodies'
     // tiles from the populations), phase 2 collides and sums the next step's density
@@ -487,6 +504,28 @@ static void enqueue_bulk(cbl_ctx* ctx, cudaStream_t s) {
   if (ctx->kev) cudaEventRecordWithFlags(ctx->kev_cap[1], s, cudaEventRecordExternal);
 }
 
+// New obstacle flags, cover refill, boundary-cell list; with the moment pass, the populations that a
+// flag change outside the stored bricks needs, and psi and moments around the changes.
+static void enqueue_refill(cbl_ctx* ctx, cudaStream_t s) {
+  const int nb = (int)ctx->hb.size();
+  if (ctx->mom)
+    ctx->ops.mom_fill(ctx->prec, ctx->lat, ctx->fa, ctx->fb, ctx->st, ctx->psi, ctx->psi2, ctx->md, ctx->pp, 1, s);
+  ctx->ops.refill(ctx->prec, ctx->lat, ctx->fa, ctx->fb, ctx->flags, ctx->db, nb, ctx->max_tile, ctx->st, ctx->blist,
+                  ctx->arena, ctx->p.member_threshold, ctx->mbox, 1, s);
+  if (ctx->mom)
+    ctx->ops.mom_close(ctx->prec, ctx->lat, ctx->fa, ctx->fb, ctx->st, ctx->flags, ctx->psi, ctx->psi2, ctx->md,
+                       ctx->blist, ctx->pp, 1, ctx->mass_part, s);  // and the step's end
+}
+// end of the step; the moment pass's last kernel does it where there are bodies
+static void enqueue_finish(cbl_ctx* ctx, cudaStream_t s) {
+  if (!ctx->mom || ctx->hb.empty()) launch_finish(ctx->mass_part, ctx->n_mass_part, ctx->st, s);
+}
+static void enqueue_flags_refill(cbl_ctx* ctx, cudaStream_t s) {
+  launch_flags(ctx->lat, ctx->db, (int)ctx->hb.size(), ctx->max_tile, ctx->arena, ctx->flags, ctx->p.solid_threshold, 0,
+               ctx->st, ctx->md_step(), s);
+  enqueue_refill(ctx, s);
+}
+
 // One step, enqueued for capture into a graph. With bodies, the collision of the cells next to a
 // solid, the solid-fluid force pass and the solid-solid repulsion run on a side branch beside the
 // bulk collision (they touch other cells, or only the phase fields, and add into the force
@@ -498,12 +537,6 @@ static void enqueue_step(cbl_ctx* ctx) {
                   ctx->Lmax, s);
     if (ctx->pp.mpf) launch_kinetics(ctx->lat, ctx->db, nb, ctx->max_tile, ctx->arena, ctx->volacc, ctx->pp, s);
   };
-  auto flags_refill = [&](cudaStream_t s) {
-    launch_flags(ctx->lat, ctx->db, nb, ctx->max_tile, ctx->arena, ctx->flags, ctx->p.solid_threshold, 0, ctx->st,
-                 s);
-    ctx->ops.refill(ctx->prec, ctx->lat, ctx->fa, ctx->fb, ctx->flags, ctx->db, nb, ctx->max_tile, ctx->st, ctx->blist,
-                  ctx->arena, ctx->p.member_threshold, ctx->mbox, 1, s);
-  };
   if (nb && ctx->branches) {
     // The bulk collision (every cell without a solid neighbour) runs beside the chain that needs only
     // the source populations, psi and the phase fields: collision of the cells next to a solid, force
@@ -511,12 +544,13 @@ static void enqueue_step(cbl_ctx* ctx) {
     // of small latency-bound kernels, so it runs on the high-priority side stream, whose blocks are
     // scheduled ahead of the bulk collision's queued ones. The flag update and the refill rewrite
     // what the bulk collision reads and writes, so they wait for both. With the fused pass, psi of the
-    // bodies' tiles (all that the side chain needs) is the side chain's first kernel.
-    if (!ctx->fused_tz) enqueue_lbm(ctx, 1, ctx->s);
+    // bodies' tiles (all that the side chain needs) is the side chain's first kernel. With the moment
+    // pass the collision of the cells next to a solid precedes the fork: the bulk pulls from them.
+    if (!ctx->fused_tz) enqueue_lbm(ctx, ctx->mom ? 4 : 1, ctx->s);
     cudaEventRecord(ctx->ev_fork, ctx->s);
     cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0);
     if (ctx->fused_tz) enqueue_lbm(ctx, 1, ctx->side);
-    enqueue_lbm(ctx, 4, ctx->side);
+    if (!ctx->mom) enqueue_lbm(ctx, 4, ctx->side);
     ctx->ops.boundary(ctx->prec, ctx->lat, ctx->fa, ctx->fb, ctx->flags, ctx->db, nb, ctx->acc, ctx->blist, ctx->st,
                     ctx->nbuf, ctx->pp.G, ctx->side);
     launch_repulsion(ctx->lat, ctx->db, nb, ctx->max_tile, ctx->arena, ctx->acc, ctx->pp, ctx->mbox, ctx->side);
@@ -526,11 +560,11 @@ static void enqueue_step(cbl_ctx* ctx) {
     cudaEventRecord(ctx->ev_join, ctx->side);
     enqueue_bulk(ctx, ctx->s);
     cudaStreamWaitEvent(ctx->s, ctx->ev_join, 0);
-    flags_refill(ctx->s);
+    enqueue_flags_refill(ctx, ctx->s);
   } else {
-    enqueue_lbm(ctx, 1, ctx->s);
+    enqueue_lbm(ctx, ctx->mom ? 4 : 1, ctx->s);
     enqueue_bulk(ctx, ctx->s);
-    enqueue_lbm(ctx, 4, ctx->s);
+    if (!ctx->mom) enqueue_lbm(ctx, 4, ctx->s);
     ctx->ops.boundary(ctx->prec, ctx->lat, ctx->fa, ctx->fb, ctx->flags, ctx->db, nb, ctx->acc, ctx->blist, ctx->st,
                     ctx->nbuf, ctx->pp.G, ctx->s);
     if (nb) {
@@ -538,17 +572,17 @@ static void enqueue_step(cbl_ctx* ctx) {
       launch_bodies(ctx->lat, ctx->db, nb, ctx->acc, ctx->last, ctx->volacc, ctx->st, ctx->rtab, ctx->Lmax,
                     ctx->mbox, ctx->fsum, ctx->s);
       phase_update(ctx->s);
-      flags_refill(ctx->s);
+      enqueue_flags_refill(ctx, ctx->s);
     }
   }
-  launch_finish(ctx->mass_part, ctx->n_mass_part, ctx->st, ctx->s);
+  enqueue_finish(ctx, ctx->s);
 }
 
 // The part of a step that follows the bulk lattice-Boltzmann pass in a persistent batch launch: the
 // collision of the cells next to a solid, the bodies' chain, flags and refill, the step's end.
 static void enqueue_side_chain(cbl_ctx* ctx) {
   const int nb = (int)ctx->hb.size();
-  enqueue_lbm(ctx, 4, ctx->s);
+  if (!ctx->mom) enqueue_lbm(ctx, 4, ctx->s);  // with the moment pass, in the persistent launch
   if (nb) {
     ctx->ops.boundary(ctx->prec, ctx->lat, ctx->fa, ctx->fb, ctx->flags, ctx->db, nb, ctx->acc, ctx->blist, ctx->st,
                       ctx->nbuf, ctx->pp.G, ctx->s);
@@ -558,12 +592,9 @@ static void enqueue_side_chain(cbl_ctx* ctx) {
     launch_advect(ctx->lat, ctx->db, nb, ctx->max_tile, ctx->arena, ctx->pp.mpf, ctx->volacc, ctx->st, ctx->rtab,
                   ctx->Lmax, ctx->s);
     if (ctx->pp.mpf) launch_kinetics(ctx->lat, ctx->db, nb, ctx->max_tile, ctx->arena, ctx->volacc, ctx->pp, ctx->s);
-    launch_flags(ctx->lat, ctx->db, nb, ctx->max_tile, ctx->arena, ctx->flags, ctx->p.solid_threshold, 0, ctx->st,
-                 ctx->s);
-    ctx->ops.refill(ctx->prec, ctx->lat, ctx->fa, ctx->fb, ctx->flags, ctx->db, nb, ctx->max_tile, ctx->st, ctx->blist,
-                    ctx->arena, ctx->p.member_threshold, ctx->mbox, 1, ctx->s);
+    enqueue_flags_refill(ctx, ctx->s);
   }
-  launch_finish(ctx->mass_part, ctx->n_mass_part, ctx->st, ctx->s);
+  enqueue_finish(ctx, ctx->s);
 }
 
 // Accumulating pass: its buffers, its kernel's shared-memory limit, its region depth, and psi of
@@ -597,13 +628,100 @@ static cbl_status acc_prepare(cbl_ctx* ctx) {
   return CBL_OK;
 }
 
+// Whether the step runs the moment pass: tau = 1 exactly (its identity), FP32 arithmetic (FP64 is
+// bound by its arithmetic, which the pass's ring cells do twice), and a lattice large enough.
+constexpr long long MOM_MIN_CELLS = 1LL << 19;
+static bool mom_rule(const cbl_ctx* ctx) {
+  if (ctx->fused_tz || ctx->acc_pass || ctx->mom_req == 0) return false;
+  if (ctx->prec == 0 || ctx->p.tau != 1.0) return false;
+  return ctx->mom_req == 1 || ctx->lat.N >= MOM_MIN_CELLS;
+}
+
+// complete populations from a state in moments, for whatever reads or changes them outside the step
+static cbl_status mom_leave(cbl_ctx* ctx, bool stay) {
+  if (!ctx->mom_state) return CBL_OK;
+  ctx->ops.mom_fill(ctx->prec, ctx->lat, ctx->fa, ctx->fb, ctx->st, ctx->psi, ctx->psi2, ctx->md, ctx->pp, 0, ctx->s);
+  CK(cudaGetLastError());
+  if (!stay) ctx->mom_state = false;
+  return CBL_OK;
+}
+
+// moments of a state in populations
+static cbl_status mom_enter(cbl_ctx* ctx) {
+  if (ctx->mom_state) return CBL_OK;
+  ctx->ops.mom_enter(ctx->prec, ctx->lat, ctx->fa, ctx->fb, ctx->st, ctx->flags, ctx->psi, ctx->psi2, ctx->md, ctx->pp,
+                     ctx->s);
+  ctx->ops.mom_close(ctx->prec, ctx->lat, ctx->fa, ctx->fb, ctx->st, ctx->flags, ctx->psi, ctx->psi2, ctx->md, ctx->blist,
+                     ctx->pp, 0, ctx->mass_part, ctx->s);
+  CK(cudaGetLastError());
+  ctx->mom_state = true;
+  return CBL_OK;
+}
+
+static void drop_graph(cbl_ctx* ctx) {
+  if (!ctx->gexec) return;
+  cudaStreamSynchronize(ctx->s);
+  cudaGraphExecDestroy(ctx->gexec);
+  cudaGraphDestroy(ctx->graph);
+  ctx->gexec = nullptr;
+  ctx->graph = nullptr;
+}
+
+// Before a step: the moment pass's buffers (without room for them the step stays with the split pass)
+// and, where the state is in populations, the moments.
+static cbl_status mom_prepare(cbl_ctx* ctx) {
+  bool use = mom_rule(ctx);
+  if (use && !ctx->md.M0) {
+    const size_t N = (size_t)ctx->lat.N;
+    MomDev& d = ctx->md;
+    d.nbx = (ctx->lat.nx + 7) / 8;
+    d.nby = (ctx->lat.ny + 7) / 8;
+    d.nbz = (ctx->lat.nz + 7) / 8;
+    const size_t bricks = (size_t)d.nbx * d.nby * d.nbz;
+    const size_t mark = ctx->allocs.size();
+    d.M0 = (float4*)dalloc(ctx, N * sizeof(float4));
+    d.M1 = d.M0 ? (float4*)dalloc(ctx, N * sizeof(float4)) : nullptr;
+    if (d.M1 && !ctx->psi2) ctx->psi2 = dalloc(ctx, N * 4);
+    unsigned char* small = d.M1 && ctx->psi2
+                               ? (unsigned char*)dalloc(ctx, 256 + 2 * bricks + 256 + sizeof(int) * (size_t)(ctx->arena_n / 3 + 1))
+                               : nullptr;
+    if (!small) {
+      for (size_t k = mark; k < ctx->allocs.size(); ++k) {
+        if (ctx->allocs[k] == ctx->psi2) ctx->psi2 = nullptr;
+        if (ctx->user_alloc) ctx->alloc.free(ctx->allocs[k], ctx->alloc.user);
+        else cudaFree(ctx->allocs[k]);
+      }
+      ctx->allocs.resize(mark);
+      cudaGetLastError();
+      d = MomDev{};
+      ctx->mom_req = 0;
+      use = false;
+    } else {
+      d.ms = (MomState*)small;
+      d.map0 = small + 256;
+      d.map1 = d.map0 + bricks;
+      d.events = (int*)(small + 256 + (2 * bricks + 255) / 256 * 256);
+      CK(cudaMemsetAsync(d.ms, 0, sizeof(MomState), ctx->s));
+      ctx->mom_sz = ctx->ops.mom_sz(ctx->lat, 1);
+      CK(ctx->ops.mom(ctx->prec, ctx->lat, ctx->fa, ctx->fb, ctx->flags, ctx->psi, ctx->psi2, d, ctx->mass_part, ctx->st,
+                      ctx->diag_rho, ctx->diag_vel, ctx->pp, 0, ctx->s));
+    }
+  }
+  if (use != ctx->mom) {
+    drop_graph(ctx);
+    ctx->mom = use;
+  }
+  return use ? mom_enter(ctx) : mom_leave(ctx, false);
+}
+
 cbl_status cbl_step(cbl_ctx* ctx, int nsteps) {
   if (!ctx) return fail(ctx, CBL_ERR_ARG, "NULL context");
   if (!ctx->ready) return fail(ctx, CBL_ERR_STATE, "cbl_step before cbl_init_fluid");
   if (nsteps < 0) return fail(ctx, CBL_ERR_ARG, "nsteps must be >= 0");
   if (nsteps == 0) return CBL_OK;
   {
-    const cbl_status sa = acc_prepare(ctx);
+    cbl_status sa = mom_prepare(ctx);
+    if (sa == CBL_OK) sa = acc_prepare(ctx);
     if (sa != CBL_OK) return sa;
   }
   if (!ctx->gexec) {
@@ -678,13 +796,14 @@ cbl_status cbl_time_phases(cbl_ctx* ctx, int nsteps, double* ms) {
   for (int k = 0; k <= CBL_NPHASES; ++k) CK(cudaEventCreate(&ev[k]));
   double acc[CBL_NPHASES] = {0};
   {
-    const cbl_status sa = acc_prepare(ctx);
+    cbl_status sa = mom_prepare(ctx);
+    if (sa == CBL_OK) sa = acc_prepare(ctx);
     if (sa != CBL_OK) return sa;
   }
   CK(cudaMemsetAsync(&ctx->st->diag, 0, sizeof(int), ctx->s));
   for (int it = 0; it < nsteps; ++it) {
     CK(cudaEventRecord(ev[0], ctx->s));
-    enqueue_lbm(ctx, 1, ctx->s);
+    if (!ctx->mom) enqueue_lbm(ctx, 1, ctx->s);
     CK(cudaEventRecord(ev[1], ctx->s));
     enqueue_lbm(ctx, 6, ctx->s);
     CK(cudaEventRecord(ev[2], ctx->s));
@@ -705,12 +824,10 @@ cbl_status cbl_time_phases(cbl_ctx* ctx, int nsteps, double* ms) {
     CK(cudaEventRecord(ev[7], ctx->s));
     if (nb)
       launch_flags(ctx->lat, ctx->db, nb, ctx->max_tile, ctx->arena, ctx->flags, ctx->p.solid_threshold, 0, ctx->st,
-                   ctx->s);
+                   ctx->md_step(), ctx->s);
     CK(cudaEventRecord(ev[8], ctx->s));
-    if (nb)
-      ctx->ops.refill(ctx->prec, ctx->lat, ctx->fa, ctx->fb, ctx->flags, ctx->db, nb, ctx->max_tile, ctx->st, ctx->blist,
-                    ctx->arena, ctx->p.member_threshold, ctx->mbox, 1, ctx->s);
-    launch_finish(ctx->mass_part, ctx->n_mass_part, ctx->st, ctx->s);
+    if (nb) enqueue_refill(ctx, ctx->s);
+    enqueue_finish(ctx, ctx->s);
     CK(cudaEventRecord(ev[9], ctx->s));
     CK(cudaGetLastError());
     CK(cudaEventSynchronize(ev[9]));
@@ -765,6 +882,8 @@ cbl_status cbl_read_populations(cbl_ctx* ctx, double* out, int on_device) {
   if (!ctx || !out) return fail(ctx, CBL_ERR_ARG, "NULL argument");
   if (!ctx->ready) return fail(ctx, CBL_ERR_STATE, "not initialised");
   const size_t bytes = (size_t)ctx->ops.q * ctx->lat.N * 8;
+  const cbl_status sm = mom_leave(ctx, true);
+  if (sm != CBL_OK) return sm;
   double* dst = out;
   if (!on_device) {
     if (!ctx->popbuf && !(ctx->popbuf = (double*)dalloc(ctx, bytes))) return fail(ctx, CBL_ERR_OOM, "population buffer");
@@ -888,7 +1007,11 @@ cbl_status cbl_move_bodies(cbl_ctx* ctx, const double* X, const double* Qn, cons
   for (int k = 0; k < 3 * nb; ++k)
     if ((V && !std::isfinite(V[k])) || (W && !std::isfinite(W[k])))
       return fail(ctx, CBL_ERR_ARG, "velocities must be finite");
-  ctx->psi_valid = false;  // flags and populations change
+  {
+    const cbl_status sm = mom_leave(ctx, false);  // flags and populations change
+    if (sm != CBL_OK) return sm;
+  }
+  ctx->psi_valid = false;
   std::vector<BodyDev> h0(nb), h(nb);
   CK(cudaMemcpyAsync(h0.data(), ctx->db, sizeof(BodyDev) * nb, cudaMemcpyDeviceToHost, ctx->s));
   CK(cudaStreamSynchronize(ctx->s));
@@ -972,7 +1095,7 @@ cbl_status cbl_move_bodies(cbl_ctx* ctx, const double* X, const double* Qn, cons
     CK(cudaMemsetAsync(&ctx->st->ncover, 0, sizeof(unsigned), ctx->s));
     CK(cudaMemsetAsync(&ctx->st->nbnd, 0, sizeof(unsigned), ctx->s));
     launch_flags(ctx->lat, ctx->db, nb, ctx->max_tile, ctx->arena, ctx->flags, ctx->p.solid_threshold, 0, ctx->st,
-                 ctx->s);
+                 MomDev{}, ctx->s);
     launch_clear_stale(ctx->lat, ctx->flags, ctx->s);
     reset_member_boxes(ctx);
     ctx->ops.refill(ctx->prec, ctx->lat, ctx->fa, ctx->fb, ctx->flags, ctx->db, nb, ctx->max_tile, ctx->st, ctx->blist,
@@ -1114,6 +1237,10 @@ static cbl_status copy_sync(cbl_ctx* ctx, void* dst, const void* src, size_t byt
 cbl_status cbl_save(cbl_ctx* ctx, const char* path) {
   if (!ctx || !path) return fail(ctx, CBL_ERR_ARG, "NULL argument");
   if (!ctx->ready) return fail(ctx, CBL_ERR_STATE, "cbl_save before cbl_init_fluid");
+  {
+    const cbl_status sm = mom_leave(ctx, true);
+    if (sm != CBL_OK) return sm;
+  }
   CK(cudaStreamSynchronize(ctx->s));
   FILE* f = std::fopen(path, "wb");
   if (!f) return fail(ctx, CBL_ERR_ARG, std::string("cannot open ") + path + " for writing");
@@ -1226,7 +1353,7 @@ cbl_status cbl_info(cbl_ctx* ctx, int* nbodies, int64_t* ncells, int* device_err
 cbl_status cbl_get_option(cbl_ctx* ctx, const char* key, double* value) {
   if (!ctx || !key || !value) return fail(ctx, CBL_ERR_ARG, "NULL argument");
   const std::string k(key);
-  if (k == "lbm_variant") *value = ctx->acc_pass ? 2 : (ctx->fused_tz ? 1 : 0);
+  if (k == "lbm_variant") *value = ctx->acc_pass ? 2 : (ctx->fused_tz ? 1 : (mom_rule(ctx) ? 3 : 0));
   else if (k == "acc_ty") *value = ctx->acc_ty;
   else if (k == "acc_sz") *value = ctx->acc_sz_req > 0 ? ctx->acc_sz_req : ctx->ops.acc_sz(ctx->lat, ctx->prec, ctx->acc_ty, 2);
   else if (k == "fused_ty") *value = ctx->fused_ty;
@@ -1250,9 +1377,12 @@ cbl_status cbl_set_option(cbl_ctx* ctx, const char* key, double value) {
   const std::string k(key);
   if (k == "lbm_variant") {
     const int v = (int)value;
-    if (v != 0 && v != 1 && v != 2) return fail(ctx, CBL_ERR_ARG, "lbm_variant must be 0, 1 or 2");
+    if (v < 0 || v > 3) return fail(ctx, CBL_ERR_ARG, "lbm_variant must be 0, 1, 2 or 3");
+    if (v == 3 && (ctx->prec == 0 || ctx->p.tau != 1.0))
+      return fail(ctx, CBL_ERR_UNSUPPORTED, "the moment pass needs tau = 1 and FP32 or binary16 storage");
     ctx->fused_tz = v == 1 ? fused_tz_of(ctx) : 0;
     ctx->acc_pass = v == 2;
+    ctx->mom_req = v == 3;
   } else if (k == "acc_ty") {
     const int v = (int)value;
     if (v != 8 && v != 16) return fail(ctx, CBL_ERR_ARG, "acc_ty must be 8 or 16");
@@ -1303,13 +1433,7 @@ cbl_status cbl_set_option(cbl_ctx* ctx, const char* key, double value) {
     return fail(ctx, CBL_ERR_ARG, "unknown option " + k);
   }
   ctx->psi_valid = false;
-  if (ctx->gexec) {
-    cudaStreamSynchronize(ctx->s);
-    cudaGraphExecDestroy(ctx->gexec);
-    cudaGraphDestroy(ctx->graph);
-    ctx->gexec = nullptr;
-    ctx->graph = nullptr;
-  }
+  drop_graph(ctx);
   return CBL_OK;
 }
 
@@ -1326,11 +1450,14 @@ struct cbl_batch {
   int mode = 0;        // 0: one fork/join branch with the whole step per instance; 1: persistent
   int tile_cfg = 1;    // tile shape of the persistent kernel (batch_tile)
   int cooperative = 1;
-  int grid = 0;
-  long long items = 0;
+  // instances on the split pass [0] and on the moment pass [1]: their number, work items, grid; the table
+  // holds those of the split pass first, and each group has its control block
+  int n[2] = {0, 0}, grid[2] = {0, 0}, sz = 0;
+  long long items[2] = {0, 0};
+  std::vector<char> mom;                // per context: 1 = on the moment pass
   long long spin_limit = 4000000000LL;  // clock64 cycles a block may wait at the grid barrier (~2 s)
   BatchInst* tab = nullptr;
-  BatchCtl* ctl = nullptr;
+  BatchCtl* ctl = nullptr;  // two
 };
 
 static cudaError_t batch_capture(cbl_batch* b, int diag, cudaGraph_t* g) {
@@ -1342,9 +1469,17 @@ static cudaError_t batch_capture(cbl_batch* b, int diag, cudaGraph_t* g) {
   if (b->mode == 1) {
     cbl_ctx* c0 = b->ctxs[0];
     for (cbl_ctx* c : b->ctxs) cudaMemsetAsync(&c->st->diag, diag, sizeof(int), b->s);
-    cudaMemsetAsync(b->ctl, 0, BATCH_CTL_RESET_BYTES, b->s);
-    el = c0->ops.batch_lbm(c0->prec, b->tile_cfg, b->tab, (int)b->ctxs.size(), b->items, b->ctl, b->grid,
-                           b->cooperative, b->s);
+    for (int k = 0; k < 2; ++k) {
+      if (!b->n[k]) continue;
+      cudaMemsetAsync(b->ctl + k, 0, BATCH_CTL_RESET_BYTES, b->s);
+      if (k)
+        el = c0->ops.batch_mom(c0->prec, b->tab + b->n[0], b->n[1], b->items[1], b->ctl + 1, b->grid[1], b->sz,
+                               b->cooperative, b->s);
+      else
+        el = c0->ops.batch_lbm(c0->prec, b->tile_cfg, b->tab, b->n[0], b->items[0], b->ctl, b->grid[0], b->cooperative,
+                               b->s);
+      if (el != cudaSuccess) break;
+    }
   }
   cudaEventRecord(b->events[0], b->s);
   for (size_t k = 0; k < b->ctxs.size(); ++k) {
@@ -1353,8 +1488,10 @@ static cudaError_t batch_capture(cbl_batch* b, int diag, cudaGraph_t* g) {
     cudaStreamWaitEvent(br, b->events[0], 0);
     cudaStream_t keep = c->s;
     const int keep_acc = c->acc_pass;
+    const bool keep_mom = c->mom;
     c->s = br;
-    c->acc_pass = 0;  // a batch runs its instances with the split or fused pass (one psi buffer)
+    c->acc_pass = 0;  // a batch runs these instances with the split pass (one psi buffer)
+    c->mom = b->mom[k];
     if (b->mode == 1) {
       enqueue_side_chain(c);
     } else {
@@ -1363,6 +1500,7 @@ static cudaError_t batch_capture(cbl_batch* b, int diag, cudaGraph_t* g) {
     }
     c->s = keep;
     c->acc_pass = keep_acc;
+    c->mom = keep_mom;
     cudaEventRecord(b->events[k + 1], br);
     cudaStreamWaitEvent(b->s, b->events[k + 1], 0);
   }
@@ -1381,47 +1519,88 @@ static void batch_drop_graphs(cbl_batch* b) {
   }
 }
 
+// which instances run the moment pass (those that do on their own; their buffers are allocated here)
+static cbl_status batch_kinds(cbl_batch* b) {
+  b->mom.assign(b->ctxs.size(), 0);
+  for (size_t k = 0; k < b->ctxs.size(); ++k) {
+    cbl_ctx* c = b->ctxs[k];
+    const cbl_status st = mom_prepare(c);
+    if (st != CBL_OK) return st;
+    b->mom[k] = c->mom_state;
+    if (cudaStreamSynchronize(c->s) != cudaSuccess) return CBL_ERR_CUDA;
+  }
+  return CBL_OK;
+}
+
+// Before a batch step: each instance's state in the form that its part of the graph steps (a move, a load
+// or a step of its own may have changed it).
+static cbl_status batch_states(cbl_batch* b) {
+  for (size_t k = 0; k < b->ctxs.size(); ++k) {
+    cbl_ctx* c = b->ctxs[k];
+    if (c->mom_state == (b->mom[k] != 0)) continue;
+    const cbl_status st = b->mom[k] ? mom_enter(c) : mom_leave(c, false);
+    if (st != CBL_OK) return st;
+    if (cudaStreamSynchronize(c->s) != cudaSuccess) return CBL_ERR_CUDA;
+  }
+  return CBL_OK;
+}
+
 // (re)build the instance table and both step graphs for the batch's mode and tile shape
 static cudaError_t batch_build(cbl_batch* b) {
   batch_drop_graphs(b);
+  if (batch_kinds(b) != CBL_OK) return cudaErrorUnknown;
+  b->n[0] = b->n[1] = 0;
   if (b->mode == 1) {
     cbl_ctx* c0 = b->ctxs[0];
-    int t[3];
-    c0->ops.batch_tile(b->tile_cfg, t);
-    std::vector<BatchInst> h(b->ctxs.size());
-    long long items = 0;
-    for (size_t k = 0; k < b->ctxs.size(); ++k) {
-      const cbl_ctx* c = b->ctxs[k];
-      BatchInst& I = h[k];
-      std::memset(&I, 0, sizeof(I));
-      I.lat = c->lat;
-      I.fa = c->fa;
-      I.fb = c->fb;
-      I.psi = c->psi;
-      I.flags = c->flags;
-      I.bodies = c->db;
-      I.mass_part = c->mass_part;
-      I.st = c->st;
-      I.diag_rho = c->diag_rho;
-      I.diag_vel = c->diag_vel;
-      I.pp = c->pp;
-      const int n[3] = {c->lat.nx, c->lat.ny, c->lat.nz};
-      for (int a = 0; a < 3; ++a) I.tiles[a] = (n[a] + t[a] - 1) / t[a];
-      I.item0 = items;
-      items += (long long)I.tiles[0] * I.tiles[1] * I.tiles[2];
+    std::vector<BatchInst> h;
+    for (int kind = 0; kind < 2; ++kind) {
+      int t[3];
+      c0->ops.batch_tile(b->tile_cfg, kind, t);
+      if (kind) b->sz = t[2];
+      long long items = 0;
+      for (size_t k = 0; k < b->ctxs.size(); ++k) {
+        const cbl_ctx* c = b->ctxs[k];
+        if ((b->mom[k] != 0) != (kind == 1)) continue;
+        BatchInst I;
+        std::memset(&I, 0, sizeof(I));
+        I.lat = c->lat;
+        I.fa = c->fa;
+        I.fb = c->fb;
+        I.psi = c->psi;
+        I.flags = c->flags;
+        I.bodies = c->db;
+        I.mass_part = c->mass_part;
+        I.st = c->st;
+        I.diag_rho = c->diag_rho;
+        I.diag_vel = c->diag_vel;
+        I.pp = c->pp;
+        I.psi2 = c->psi2;
+        I.nbuf = c->nbuf;
+        I.blist = c->blist;
+        if (kind) I.md = c->md;
+        const int n[3] = {c->lat.nx, c->lat.ny, c->lat.nz};
+        for (int a = 0; a < 3; ++a) I.tiles[a] = (n[a] + t[a] - 1) / t[a];
+        I.item0 = items;
+        items += (long long)I.tiles[0] * I.tiles[1] * I.tiles[2];
+        h.push_back(I);
+        ++b->n[kind];
+      }
+      b->items[kind] = items;
     }
-    b->items = items;
     cudaError_t e = cudaMemcpy(b->tab, h.data(), sizeof(BatchInst) * h.size(), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    b->grid = c0->ops.batch_blocks_per_sm(c0->prec, b->tile_cfg) * sms;
-    if (b->grid <= 0) return cudaErrorInvalidConfiguration;
-    BatchCtl ctl;
-    std::memset(&ctl, 0, sizeof(ctl));
-    ctl.spin_limit = b->spin_limit;
-    e = cudaMemcpy(b->ctl, &ctl, sizeof(ctl), cudaMemcpyHostToDevice);
+    for (int kind = 0; kind < 2; ++kind) {
+      if (!b->n[kind]) continue;
+      b->grid[kind] = sms * (kind ? c0->ops.batch_mom_blocks_per_sm(c0->prec) : c0->ops.batch_blocks_per_sm(c0->prec, b->tile_cfg));
+      if (b->grid[kind] <= 0) return cudaErrorInvalidConfiguration;
+    }
+    BatchCtl ctl[2];
+    std::memset(ctl, 0, sizeof(ctl));
+    ctl[0].spin_limit = ctl[1].spin_limit = b->spin_limit;
+    e = cudaMemcpy(b->ctl, ctl, sizeof(ctl), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return e;
   }
   for (int d = 0; d < 2; ++d) {
@@ -1466,7 +1645,7 @@ cbl_status cbl_batch_create(cbl_ctx* const* ctxs, int n, void* stream, cbl_batch
   for (int k = 0; k < n; ++k) ok &= cudaStreamCreateWithFlags(&b->branches[k], cudaStreamNonBlocking) == cudaSuccess;
   for (int k = 0; k <= n; ++k) ok &= cudaEventCreateWithFlags(&b->events[k], cudaEventDisableTiming) == cudaSuccess;
   ok &= cudaMalloc(&b->tab, sizeof(BatchInst) * n) == cudaSuccess;
-  ok &= cudaMalloc(&b->ctl, sizeof(BatchCtl)) == cudaSuccess;
+  ok &= cudaMalloc(&b->ctl, 2 * sizeof(BatchCtl)) == cudaSuccess;
   if (ok && batch_build(b) != cudaSuccess && b->mode == 1) {
     // a cooperative kernel that cannot be captured: the same launch, plain (the grid is sized to be
     // resident, and the barrier's wait is bounded either way)
@@ -1514,14 +1693,15 @@ cbl_status cbl_batch_info(cbl_batch* b, int* mode, int* tile, long long* items, 
   if (!b) return fail(nullptr, CBL_ERR_ARG, "NULL batch");
   if (mode) *mode = b->mode;
   if (tile) *tile = b->tile_cfg;
-  if (items) *items = b->items;
-  if (grid) *grid = b->grid;
+  if (items) *items = b->items[0] + b->items[1];
+  if (grid) *grid = std::max(b->grid[0], b->grid[1]);
   return CBL_OK;
 }
 
 cbl_status cbl_batch_step(cbl_batch* b, int nsteps) {
   if (!b) return fail(nullptr, CBL_ERR_ARG, "NULL batch");
   if (nsteps < 0) return fail(nullptr, CBL_ERR_ARG, "nsteps must be >= 0");
+  if (batch_states(b) != CBL_OK) return fail(nullptr, CBL_ERR_CUDA, "state of an instance");
   for (int k = 0; k < nsteps; ++k)
     if (cudaGraphLaunch(b->gexec[k == nsteps - 1 ? 1 : 0], b->s) != cudaSuccess)
       return fail(nullptr, CBL_ERR_CUDA, "batch graph launch failed");
@@ -1537,12 +1717,12 @@ cbl_status cbl_batch_sync(cbl_batch* b) {
   if (!b) return fail(nullptr, CBL_ERR_ARG, "NULL batch");
   if (cudaStreamSynchronize(b->s) != cudaSuccess) return fail(nullptr, CBL_ERR_CUDA, "sync");
   if (b->mode == 1) {
-    int err = 0;
-    if (cudaMemcpy(&err, &b->ctl->err, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
+    BatchCtl ctl[2];
+    if (cudaMemcpy(ctl, b->ctl, sizeof(ctl), cudaMemcpyDeviceToHost) != cudaSuccess)
       return fail(nullptr, CBL_ERR_CUDA, "sync");
-    if (err) {
+    if (ctl[0].err || ctl[1].err) {
       const int zero = 0;
-      cudaMemcpy(&b->ctl->err, &zero, sizeof(int), cudaMemcpyHostToDevice);
+      for (int k = 0; k < 2; ++k) cudaMemcpy(&b->ctl[k].err, &zero, sizeof(int), cudaMemcpyHostToDevice);
       return fail(nullptr, CBL_ERR_TIMEOUT, "a grid-barrier wait of the persistent batch kernel ran out");
     }
   }

@@ -151,6 +151,30 @@ struct PhysParams {
   float tau_f, G_f, rho0_f, ext_f[3];
 };
 
+// End of a step, by one block of T threads: the fluid mass (fixed-order sum of the collision's partials,
+// which are cleared) and the population buffer flip. The bulk collision may run beside the body
+// update, so neither can happen earlier.
+template <int T>
+__device__ __forceinline__ void finish_step(double* mass_part, unsigned n_mass_part, StepState* st) {
+  __shared__ double red[T];
+  double sm = 0.0;
+  for (unsigned k = threadIdx.x; k < n_mass_part; k += T) {
+    sm += mass_part[k];
+    mass_part[k] = 0.0;
+  }
+  red[threadIdx.x] = sm;
+  __syncthreads();
+  for (int w = T / 2; w > 0; w >>= 1) {
+    if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
+    st->last_mass = red[0];
+    st->parity ^= 1;
+    st->psi_skip = 0;
+  }
+}
+
 inline void fill_float_params(PhysParams& p) {
   p.tau_f = (float)p.tau;
   p.G_f = (float)p.G;
@@ -173,6 +197,49 @@ __device__ __forceinline__ long long dbits(double v) { return __double_as_longlo
 
 // wrapi, mimg, wrapd: periodic wraps with a fixed operation count (periodic.h)
 
+// ---- moment pass (moments.cuh) -----------------------------------------------------------------
+// Per-step state of the moment pass: obstacle flags that changed in this step's flag update (cells in
+// `events`), and whether one changed where populations are not stored.
+struct MomState {
+  unsigned nevent;
+  int full;
+  unsigned done;  // blocks of the step's last kernel that are through
+};
+// Buffers of the moment pass, indexed by the parity of the step they belong to: moments (rho, m) of
+// every cell, and a byte per brick of 8 x 8 x 8 cells in which populations are stored.
+struct MomDev {
+  float4 *M0, *M1;
+  unsigned char *map0, *map1;
+  int nbx, nby, nbz;  // bricks per axis
+  int* events;        // NULL: the step does not run the moment pass
+  MomState* ms;
+  // (selected, not indexed: an index into a kernel parameter would copy it to local memory)
+  __device__ float4* M(int q) const { return q ? M1 : M0; }
+  __device__ unsigned char* map(int q) const { return q ? map1 : map0; }
+  __device__ unsigned brick(int bx, int by, int bz) const { return (unsigned)(bx + nbx * (by + nby * bz)); }
+  __device__ unsigned bricks() const { return (unsigned)(nbx * nby * nbz); }
+};
+
+// Bricks along one axis that the cells within r (<= 4) of cell g of a periodic side n touch: at most
+// two of 8 cells, and at the periodic seam, where the last brick may be short, those beside it.
+constexpr int BRICK_SPAN = 5;
+__device__ __forceinline__ int brick_span(int g, int r, int n, int b[BRICK_SPAN]) {
+  int cnt = 0;
+  auto add = [&](int v) {
+    for (int k = 0; k < cnt; ++k)
+      if (b[k] == v) return;
+    b[cnt++] = v;
+  };
+  add(wrapi_near(g - r, n) >> 3);
+  add(g >> 3);
+  add(wrapi_near(g + r, n) >> 3);
+  if (g - r < 0 || g + r >= n) {
+    add((n - 1) >> 3);
+    add(0);
+  }
+  return cnt;
+}
+
 // ---- batches of independent lattices -----------------------------------------------------------
 // One instance of a batch, as the persistent lattice-Boltzmann kernel sees it (a device-resident
 // table, one entry per instance): its lattice and buffers, and where its work items start. A work
@@ -189,6 +256,10 @@ struct BatchInst {
   PhysParams pp;
   int tiles[3];    // tiles per axis
   int pad;
+  // moment pass: its second psi buffer and buffers, the cells next to a solid and their side buffer
+  void *psi2, *nbuf;
+  const int* blist;
+  MomDev md;
   long long item0;  // first work item of this instance
 };
 
@@ -226,6 +297,22 @@ extern thread_local int g_launch_share;
                        void* psi_b, const BodyDev* bodies, double* mass_part, unsigned blocks,        \
                        StepState* st, double* diag_rho, double* diag_vel, const PhysParams& pp,       \
                        void* nbuf, const int* blist, cudaStream_t s, int phases);                     \
+  int mom_sz(const Lat& lat, int share);                                                             \
+  cudaError_t launch_mom(int prec, const Lat& lat, void* fa, void* fb, const uint16_t* flags, void* psi_a, \
+                         void* psi_b, const MomDev& md, double* mass_part, StepState* st,            \
+                         double* diag_rho, double* diag_vel, const PhysParams& pp, int sz, cudaStream_t s); \
+  void launch_mom_near(int prec, const Lat& lat, void* fa, void* fb, const uint16_t* flags, void* psi_a, \
+                       void* psi_b, const BodyDev* bodies, double* mass_part, StepState* st,         \
+                       double* diag_rho, double* diag_vel, const PhysParams& pp, void* nbuf,         \
+                       const int* blist, cudaStream_t s);                                             \
+  void launch_mom_enter(int prec, const Lat& lat, const void* fa, const void* fb, const StepState* st, \
+                        const uint16_t* flags, void* psi_a, void* psi_b, const MomDev& md,           \
+                        const PhysParams& pp, cudaStream_t s);                                        \
+  void launch_mom_fill(int prec, const Lat& lat, void* fa, void* fb, const StepState* st, const void* psi_a, \
+                       const void* psi_b, const MomDev& md, const PhysParams& pp, int next, cudaStream_t s); \
+  void launch_mom_close(int prec, const Lat& lat, const void* fa, const void* fb, StepState* st,     \
+                        const uint16_t* flags, void* psi_a, void* psi_b, const MomDev& md,           \
+                        const int* blist, const PhysParams& pp, int next, double* mass_part, cudaStream_t s); \
   int acc_sz(const Lat& lat, int prec, int ty, int waves);                                          \
   cudaError_t launch_lbm_acc(int prec, const Lat& lat, void* fa, void* fb, const uint16_t* flags,    \
                              void* psi_a, void* psi_b, void* rhop, const BodyDev* bodies,           \
@@ -255,7 +342,10 @@ extern thread_local int g_launch_share;
   void launch_refill(int prec, const Lat& lat, void* fa, void* fb, uint16_t* flags, const BodyDev* bodies, \
                      int nb, int max_tile, StepState* st, int* blist, const double* arena,           \
                      double member_thr, int* mbox, int next, cudaStream_t s);                        \
-  void batch_tile(int cfg, int* t);                                                                   \
+  void batch_tile(int cfg, int mom, int* t);                                                          \
+  int batch_mom_blocks_per_sm(int prec);                                                              \
+  cudaError_t launch_batch_mom(int prec, const BatchInst* tab, int ninst, long long items, BatchCtl* ctl, \
+                               int grid, int sz, int cooperative, cudaStream_t s);                   \
   int batch_blocks_per_sm(int prec, int cfg);                                                         \
   cudaError_t launch_batch_lbm(int prec, int cfg, const BatchInst* tab, int ninst, long long items,  \
                                BatchCtl* ctl, int grid, int cooperative, cudaStream_t s);
@@ -271,6 +361,12 @@ struct LbmOps {
   int q;
   decltype(&q19::set_fp16_weights) set_fp16_weights;
   decltype(&q19::launch_lbm_step) lbm_step;
+  decltype(&q19::mom_sz) mom_sz;
+  decltype(&q19::launch_mom) mom;
+  decltype(&q19::launch_mom_near) mom_near;
+  decltype(&q19::launch_mom_enter) mom_enter;
+  decltype(&q19::launch_mom_fill) mom_fill;
+  decltype(&q19::launch_mom_close) mom_close;
   decltype(&q19::acc_sz) acc_sz;
   decltype(&q19::launch_lbm_acc) lbm_acc;
   decltype(&q19::launch_psi_fixup) psi_fixup;
@@ -283,16 +379,19 @@ struct LbmOps {
   decltype(&q19::launch_init_fluid) init_fluid;
   decltype(&q19::launch_refill) refill;
   decltype(&q19::batch_tile) batch_tile;
+  decltype(&q19::batch_mom_blocks_per_sm) batch_mom_blocks_per_sm;
+  decltype(&q19::launch_batch_mom) batch_mom;
   decltype(&q19::batch_blocks_per_sm) batch_blocks_per_sm;
   decltype(&q19::launch_batch_lbm) batch_lbm;
 };
 inline LbmOps lbm_ops(int q) {
 #define CBL_OPS(ns) \
-  LbmOps { q, &ns::set_fp16_weights, &ns::launch_lbm_step, &ns::acc_sz, &ns::launch_lbm_acc,                     \
+  LbmOps { q, &ns::set_fp16_weights, &ns::launch_lbm_step, &ns::mom_sz, &ns::launch_mom, &ns::launch_mom_near,   \
+           &ns::launch_mom_enter, &ns::launch_mom_fill, &ns::launch_mom_close, &ns::acc_sz, &ns::launch_lbm_acc,   \
            &ns::launch_psi_fixup, &ns::fused_tz, &ns::launch_lbm_fused,                                             \
            &ns::launch_density_tiles, &ns::launch_boundary,                                                             \
            &ns::launch_read_populations, &ns::launch_zero_solid, &ns::launch_init_fluid, &ns::launch_refill,        \
-           &ns::batch_tile, &ns::batch_blocks_per_sm, &ns::launch_batch_lbm }
+           &ns::batch_tile, &ns::batch_mom_blocks_per_sm, &ns::launch_batch_mom, &ns::batch_blocks_per_sm, &ns::launch_batch_lbm }
   return q == 27 ? CBL_OPS(q27) : CBL_OPS(q19);
 #undef CBL_OPS
 }
@@ -305,7 +404,7 @@ void launch_rasterize(const Lat& lat, BodyDev* bodies, int nb, int max_tile, dou
                       double eta, cudaStream_t s);
 void launch_neighbour_lists(BodyDev* bodies, int nb, const Lat& lat, StepState* st, cudaStream_t s);
 void launch_flags(const Lat& lat, BodyDev* bodies, int nb, int max_tile, double* arena, uint16_t* flags,
-                  double threshold, int init, StepState* st, cudaStream_t s);
+                  double threshold, int init, StepState* st, const MomDev& md, cudaStream_t s);
 void launch_body_props(const Lat& lat, BodyDev* bodies, int nb, int max_tile, double* arena,
                        double* scratch, cudaStream_t s);
 void launch_repulsion(const Lat& lat, const BodyDev* bodies, int nb, int max_tile, const double* arena, double* acc,

@@ -30,6 +30,7 @@
 #include <algorithm>
 #include <climits>
 #include <cmath>
+#include <type_traits>
 #include "../../include/cbl.h"
 #include "cbl_dev.cuh"
 
@@ -67,6 +68,8 @@ template <>
 struct St<float> {
   using R = float;
   __device__ static R ld(const float* p, size_t k, int) { return __ldg(p + k); }
+  // plain load: of a buffer that the same kernel writes elsewhere
+  __device__ static R ldv(const float* p, size_t k, int) { return p[k]; }
   __device__ static void st(float* p, size_t k, int, R v) { p[k] = v; }
   __device__ static R rt(R v, int) { return v; }
 };
@@ -75,6 +78,7 @@ struct St<__half> {
   using R = float;
   // f = h + w_hat: zero populations (solid cells) are stored exactly as h = -w_hat.
   __device__ static R ld(const __half* p, size_t k, int i) { return __half2float(__ldg(p + k)) + c_wh[i]; }
+  __device__ static R ldv(const __half* p, size_t k, int i) { return __half2float(p[k]) + c_wh[i]; }
   __device__ static R from_raw(unsigned short h, int i) { return __half2float(__ushort_as_half(h)) + c_wh[i]; }
   __device__ static void st(__half* p, size_t k, int i, R v) { p[k] = __float2half_rn(v - c_wh[i]); }
   // the value a later load of the stored population returns
@@ -549,8 +553,45 @@ __global__ void __launch_bounds__(128, CollideMinBlocks<S>::value) k_collide(S* 
   add_mass_slot(mass_part, my_mass, blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z));
 }
 
-// Collision of the fluid cells next to a solid (the boundary-cell list built by the refill pass).
-template <typename S>
+// Collision of the fluid cells next to a solid (the boundary-cell list built by the refill pass), entries
+// first, first + stride, ... Returns the sum of their densities.
+// WET: solid neighbours' psi comes from their owner (the moment pass keeps no psi of solid cells).
+template <typename S, bool WET>
+__device__ __forceinline__ typename St<S>::R near_cells(S* __restrict__ fa, S* __restrict__ fb,
+                                                        const uint16_t* __restrict__ flags,
+                                                        const typename St<S>::R* __restrict__ psi_a,
+                                                        const typename St<S>::R* __restrict__ psi_b,
+                                                        const BodyDev* __restrict__ bodies,
+                                                        const StepState* __restrict__ st,
+                                                        double* __restrict__ diag_rho, double* __restrict__ diag_vel,
+                                                        const int* __restrict__ blist, const Lat& lat,
+                                                        const PhysParams& pp, RhoPsi<typename St<S>::R>* __restrict__ nbuf,
+                                                        unsigned first, unsigned stride) {
+  using R = typename St<S>::R;
+  const R* __restrict__ psi = (psi_b && st->parity) ? psi_b : psi_a;
+  const int diag = st->diag;
+  const S* __restrict__ src = st->parity ? fb : fa;
+  S* __restrict__ dst = st->parity ? fa : fb;
+  const unsigned count = st->nbnd;
+  R mass = 0;
+  for (unsigned k = first; k < count; k += stride) {
+    const long long n = blist[k];
+    const Cell c = cell_of(n, lat);
+    auto psi_at = [&](int i) -> R {
+      if (i == 0) return psi[n];
+      const long long k2 = nbr(c, lat, i, +1);
+      if constexpr (WET) {
+        const uint16_t fl = __ldg(flags + k2);
+        if (fl & F_SOLID) return par<R>(bodies[fl & F_OWNER].psi_wet, bodies[fl & F_OWNER].psi_wet_f);
+      }
+      return psi[k2];
+    };
+    mass += collide_fluid<S, true>(src, dst, flags, psi_at, bodies, diag, diag_rho, diag_vel, lat, pp, nbuf, c, n);
+  }
+  return mass;
+}
+
+template <typename S, bool WET = false>
 __global__ void __launch_bounds__(128) k_collide_near(S* __restrict__ fa, S* __restrict__ fb,
                                                       const uint16_t* __restrict__ flags,
                                                       const typename St<S>::R* __restrict__ psi_a,
@@ -561,20 +602,10 @@ __global__ void __launch_bounds__(128) k_collide_near(S* __restrict__ fa, S* __r
                                                       double* __restrict__ diag_rho, double* __restrict__ diag_vel,
                                                       const int* __restrict__ blist, Lat lat, PhysParams pp,
                                                       RhoPsi<typename St<S>::R>* __restrict__ nbuf) {
-  using R = typename St<S>::R;
-  const R* __restrict__ psi = (psi_b && st->parity) ? psi_b : psi_a;
-  const int diag = st->diag;
-  const S* __restrict__ src = st->parity ? fb : fa;
-  S* __restrict__ dst = st->parity ? fa : fb;
-  const unsigned count = st->nbnd;
-  R my_mass = 0;
-  for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < count; k += gridDim.x * blockDim.x) {
-    const long long n = blist[k];
-    const Cell c = cell_of(n, lat);
-    auto psi_at = [&](int i) -> R { return i ? psi[nbr(c, lat, i, +1)] : psi[n]; };
-    my_mass += collide_fluid<S, true>(src, dst, flags, psi_at, bodies, diag, diag_rho, diag_vel, lat, pp, nbuf, c, n);
-  }
-  add_mass_slot(mass_part, my_mass, blockIdx.x * 7u + 3u);
+  const typename St<S>::R mass =
+      near_cells<S, WET>(fa, fb, flags, psi_a, psi_b, bodies, st, diag_rho, diag_vel, blist, lat, pp, nbuf,
+                         blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+  add_mass_slot(mass_part, mass, blockIdx.x * 7u + 3u);
 }
 
 // ---- accumulating pass (lbm_variant 2) ---------------------------------------------------------
@@ -1040,6 +1071,19 @@ __device__ __forceinline__ bool grid_barrier(BatchCtl* ctl) {
   return s_ok != 0;
 }
 
+// the instance whose items contain this one (item0 ascends with the instance index)
+__device__ __forceinline__ int batch_instance(const BatchInst* __restrict__ tab, int ninst, long long item) {
+  int lo = 0, hi = ninst - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (tab[mid].item0 <= item) lo = mid;
+    else hi = mid - 1;
+  }
+  return lo;
+}
+
+#include "moments.cuh"
+
 template <typename S, int TX, int TY, int TZ>
 __global__ void __launch_bounds__(TX * TY, CollideMinBlocks<S>::value)
     k_batch_lbm(const BatchInst* __restrict__ tab, int ninst, long long items, BatchCtl* ctl) {
@@ -1053,14 +1097,7 @@ __global__ void __launch_bounds__(TX * TY, CollideMinBlocks<S>::value)
       const long long item = s_item;
       __syncthreads();  // s_item is written again in the next round
       if (item >= items) break;
-      // the instance whose items contain this one (item0 ascends with the instance index)
-      int lo = 0, hi = ninst - 1;
-      while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (tab[mid].item0 <= item) lo = mid;
-        else hi = mid - 1;
-      }
-      const BatchInst& I = tab[lo];
+      const BatchInst& I = tab[batch_instance(tab, ninst, item)];
       const Lat lat = I.lat;
       const long long k = item - I.item0;
       const int bx = (int)(k % I.tiles[0]), by = (int)((k / I.tiles[0]) % I.tiles[1]),
@@ -1605,6 +1642,107 @@ void launch_lbm_step(int prec, const Lat& lat, void* fa, void* fb, const uint16_
                        diag_vel, pp, nbuf, blist, s, phases);
 }
 
+// Moment pass: columns of 32 x MOM_TY cells. D3Q19: 8 rows, 107 KB of shared memory, two blocks per SM;
+// D3Q27's 26 directions leave room for two blocks at 4 rows.
+constexpr int MOM_TY = Q == 19 ? 8 : 4, MOM_MINB = 2;
+
+// Planes per block. A block computes sz + 2 planes (two are only pulled from), so the resident blocks
+// share blocks x (sz + 2) planes, and the last ones end half a block's march apart on average.
+// Measured on 256^3 (us per step): 335 at 256 planes, 307 at 64, 301 at 37, 308 at 32, 325 at 16;
+// on 96^3: 78 at 96, 33 at 32, 29 at 8.
+int mom_sz(const Lat& lat, int share) {
+  const long long cols = (long long)((lat.nx + 31) / 32) * ((lat.ny + MOM_TY - 1) / MOM_TY);
+  const double slots = std::max(1.0, (double)MOM_MINB * sm_count() / std::max(1, share));
+  int best = lat.nz;
+  double best_cost = 1e300;
+  for (int sz = lat.nz; sz >= 1; --sz) {
+    const int chunks = (lat.nz + sz - 1) / sz;
+    const double march = std::max(1.0, cols * chunks / slots);
+    const double cost = march * (lat.nz / (double)chunks + 2.0) + 0.5 * (sz + 2);
+    if (cost < best_cost) {
+      best_cost = cost;
+      best = sz;
+    }
+  }
+  return best;
+}
+
+// sz = 0: set the kernel's dynamic shared-memory limit (outside any stream capture) and return
+template <typename S>
+static cudaError_t mom_t(const Lat& lat, void* fa, void* fb, const uint16_t* flags, void* psi_a, void* psi_b,
+                         const MomDev& md, double* mass_part, StepState* st, double* diag_rho, double* diag_vel,
+                         const PhysParams& pp, int sz, cudaStream_t s) {
+  using T = MomTile<MOM_TY>;
+  if (sz <= 0)
+    return cudaFuncSetAttribute(k_mom<S, MOM_TY, MOM_MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::smem);
+  const dim3 grid((lat.nx + 31) / 32, (lat.ny + MOM_TY - 1) / MOM_TY, (lat.nz + sz - 1) / sz);
+  const MomArgs<S> a{(S*)fa, (S*)fb, flags, (float*)psi_a, (float*)psi_b, md, mass_part, st, diag_rho, diag_vel};
+  k_mom<S, MOM_TY, MOM_MINB><<<grid, T::NT, T::smem, s>>>(a, lat, pp, sz);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_mom(int prec, const Lat& lat, void* fa, void* fb, const uint16_t* flags, void* psi_a, void* psi_b,
+                       const MomDev& md, double* mass_part, StepState* st, double* diag_rho, double* diag_vel,
+                       const PhysParams& pp, int sz, cudaStream_t s) {
+  if (prec == 1) return mom_t<float>(lat, fa, fb, flags, psi_a, psi_b, md, mass_part, st, diag_rho, diag_vel, pp, sz, s);
+  return mom_t<__half>(lat, fa, fb, flags, psi_a, psi_b, md, mass_part, st, diag_rho, diag_vel, pp, sz, s);
+}
+
+template <typename S>
+static void mom_near_t(const Lat& lat, void* fa, void* fb, const uint16_t* flags, void* psi_a, void* psi_b,
+                       const BodyDev* bodies, double* mass_part, StepState* st, double* diag_rho, double* diag_vel,
+                       const PhysParams& pp, void* nbuf, const int* blist, cudaStream_t s) {
+  k_collide_near<S, true><<<std::max(1, 2 * sm_count() / g_launch_share), 128, 0, s>>>(
+      (S*)fa, (S*)fb, flags, (const float*)psi_a, (const float*)psi_b, bodies, mass_part, st, diag_rho, diag_vel, blist,
+      lat, pp, (RhoPsi<float>*)nbuf);
+}
+
+void launch_mom_near(int prec, const Lat& lat, void* fa, void* fb, const uint16_t* flags, void* psi_a, void* psi_b,
+                     const BodyDev* bodies, double* mass_part, StepState* st, double* diag_rho, double* diag_vel,
+                     const PhysParams& pp, void* nbuf, const int* blist, cudaStream_t s) {
+  if (!blist) return;
+  if (prec == 1) mom_near_t<float>(lat, fa, fb, flags, psi_a, psi_b, bodies, mass_part, st, diag_rho, diag_vel, pp, nbuf, blist, s);
+  else mom_near_t<__half>(lat, fa, fb, flags, psi_a, psi_b, bodies, mass_part, st, diag_rho, diag_vel, pp, nbuf, blist, s);
+}
+
+void launch_mom_enter(int prec, const Lat& lat, const void* fa, const void* fb, const StepState* st,
+                      const uint16_t* flags, void* psi_a, void* psi_b, const MomDev& md, const PhysParams& pp,
+                      cudaStream_t s) {
+  const dim3 grid((lat.nx + 31) / 32, (lat.ny + 3) / 4, lat.nz);
+  if (prec == 1)
+    k_mom_enter<float><<<grid, 128, 0, s>>>((const float*)fa, (const float*)fb, st, flags, (float*)psi_a, (float*)psi_b,
+                                            md, lat, pp.rho0_f);
+  else
+    k_mom_enter<__half><<<grid, 128, 0, s>>>((const __half*)fa, (const __half*)fb, st, flags, (float*)psi_a,
+                                             (float*)psi_b, md, lat, pp.rho0_f);
+}
+
+void launch_mom_fill(int prec, const Lat& lat, void* fa, void* fb, const StepState* st, const void* psi_a,
+                     const void* psi_b, const MomDev& md, const PhysParams& pp, int next, cudaStream_t s) {
+  // inside a step the launch is a test of one word in nearly every step: one block per SM
+  const unsigned grid = (unsigned)std::min(
+      (lat.N + 255) / 256, next ? std::max(1LL, (long long)sm_count() / g_launch_share) : 16LL * sm_count());
+  if (prec == 1)
+    k_mom_fill<float><<<grid, 256, 0, s>>>((float*)fa, (float*)fb, st, (const float*)psi_a, (const float*)psi_b, md, lat,
+                                           pp, next);
+  else
+    k_mom_fill<__half><<<grid, 256, 0, s>>>((__half*)fa, (__half*)fb, st, (const float*)psi_a, (const float*)psi_b, md,
+                                            lat, pp, next);
+}
+
+void launch_mom_close(int prec, const Lat& lat, const void* fa, const void* fb, StepState* st, const uint16_t* flags,
+                      void* psi_a, void* psi_b, const MomDev& md, const int* blist, const PhysParams& pp, int next,
+                      double* mass_part, cudaStream_t s) {
+  if (!blist) return;
+  const unsigned grid = (unsigned)std::max(1, 4 * sm_count() / g_launch_share);
+  if (prec == 1)
+    k_mom_close<float><<<grid, 128, 0, s>>>((const float*)fa, (const float*)fb, st, flags, (float*)psi_a, (float*)psi_b,
+                                            md, blist, lat, pp.rho0_f, next, mass_part);
+  else
+    k_mom_close<__half><<<grid, 128, 0, s>>>((const __half*)fa, (const __half*)fb, st, flags, (float*)psi_a,
+                                             (float*)psi_b, md, blist, lat, pp.rho0_f, next, mass_part);
+}
+
 // Accumulating pass: blocks of 32 x ty threads (ty = 8 or 16) marching sz planes. Resident blocks
 // per SM asked of the compiler: 64 registers per thread for FP32 storage, 80 for binary16, 128 for
 // FP64.
@@ -1738,11 +1876,54 @@ void launch_refill(int prec, const Lat& lat, void* fa, void* fb, uint16_t* flags
                                         mbox, next);
 }
 
-// Tile shapes of the persistent batch kernel (x, y, z cells; 128 threads per block).
-void batch_tile(int cfg, int* t) {
+// Tile shapes of the persistent batch kernels (x, y, z cells): of the split pass (128 threads per block),
+// and of the moment pass (columns of 32 x MOM_TY cells, by their number of planes).
+void batch_tile(int cfg, int mom, int* t) {
   static const int T[BATCH_TILE_CFGS][3] = {{32, 4, 1}, {32, 4, 4}, {32, 4, 8}, {64, 2, 4}};
+  static const int Z[BATCH_TILE_CFGS] = {16, 32, 64, 24};
   const int k = cfg < 0 || cfg >= BATCH_TILE_CFGS ? 1 : cfg;
   for (int a = 0; a < 3; ++a) t[a] = T[k][a];
+  if (mom) {
+    t[0] = 32;
+    t[1] = MOM_TY;
+    t[2] = Z[k];
+  }
+}
+
+template <typename S>
+static cudaError_t batch_mom_t(const BatchInst* tab, int ninst, long long items, BatchCtl* ctl, int grid, int sz, int coop,
+                               cudaStream_t s) {
+  using T = MomTile<MOM_TY>;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(T::NT);
+  cfg.dynamicSmemBytes = T::smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = coop ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, k_batch_mom<S, MOM_TY, MOM_MINB>, tab, ninst, items, ctl, sz);
+}
+
+template <typename S>
+static int batch_mom_occ() {
+  using T = MomTile<MOM_TY>;
+  int nb = 0;
+  if (cudaFuncSetAttribute(k_batch_mom<S, MOM_TY, MOM_MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::smem) ==
+      cudaSuccess)
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_batch_mom<S, MOM_TY, MOM_MINB>, T::NT, T::smem);
+  return nb;
+}
+
+// resident blocks per SM of the moment pass's batch kernel (and its shared-memory limit set)
+int batch_mom_blocks_per_sm(int prec) { return prec == 1 ? batch_mom_occ<float>() : batch_mom_occ<__half>(); }
+
+cudaError_t launch_batch_mom(int prec, const BatchInst* tab, int ninst, long long items, BatchCtl* ctl, int grid, int sz,
+                             int cooperative, cudaStream_t s) {
+  return prec == 1 ? batch_mom_t<float>(tab, ninst, items, ctl, grid, sz, cooperative, s)
+                   : batch_mom_t<__half>(tab, ninst, items, ctl, grid, sz, cooperative, s);
 }
 
 template <typename S, int TX, int TY, int TZ>

@@ -173,8 +173,29 @@ __global__ void k_neighbour_lists(BodyDev* bodies, int nb, Lat lat, StepState* s
 }
 
 // ---- flags --------------------------------------------------------------------------------------
+
+// A cell's obstacle flag changed: the moment pass has to pull its surroundings again from the populations
+// (k_mom_close), which needs those within 3 cells of it stored; where the bricks do not say so, all of
+// them are written first (k_mom_fill).
+__device__ __noinline__ void flag_event(const MomDev& md, const StepState* st, const TileCell& c, long long n,
+                                        const Lat& lat) {
+  md.events[atomicAdd(&md.ms->nevent, 1u)] = (int)n;
+  int b[3][BRICK_SPAN], nbk[3];
+  nbk[0] = brick_span(c.gx, 3, lat.nx, b[0]);
+  nbk[1] = brick_span(c.gy, 3, lat.ny, b[1]);
+  nbk[2] = brick_span(c.gz, 3, lat.nz, b[2]);
+  const unsigned char* map = md.map(st->parity);
+  bool all = true;
+  for (int iz = 0; iz < nbk[2]; ++iz)
+    for (int iy = 0; iy < nbk[1]; ++iy)
+      for (int ix = 0; ix < nbk[0]; ++ix) all &= map[md.brick(b[0][ix], b[1][iy], b[2][iz])] != 0;
+  if (!all) md.ms->full = 1;
+}
+
+// EV: record the changes (moment pass)
+template <bool EV>
 __global__ void k_flags(BodyDev* bodies, double* arena, uint16_t* flags, Lat lat, double thr, int init,
-                        StepState* st) {
+                        StepState* st, MomDev md) {
   const int self = blockIdx.y;
   const BodyDev& b = bodies[self];
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -210,6 +231,7 @@ __global__ void k_flags(BodyDev* bodies, double* arena, uint16_t* flags, Lat lat
         atomicAdd(&st->ncover, 1u);
       }
     }
+    if (EV && ((flags[n_cell] ^ nf) & F_SOLID)) flag_event(md, st, c, n_cell, lat);
     flags[n_cell] = nf;
     return;
   }
@@ -262,6 +284,7 @@ __global__ void k_flags(BodyDev* bodies, double* arena, uint16_t* flags, Lat lat
       atomicAdd(&st->ncover, 1u);
     }
   }
+  if (EV && ((old ^ nf) & F_SOLID)) flag_event(md, st, c, n, lat);
   flags[n] = nf;
 }
 
@@ -594,27 +617,8 @@ __global__ void __launch_bounds__(256) k_bodies(BodyDev* bodies, int nb, double*
   }
 }
 
-// End of a step: the fluid mass (fixed-order sum of the collision's per-block partials, which are
-// cleared) and the population buffer flip. The bulk collision may run beside the body update, so
-// neither can happen earlier.
 __global__ void __launch_bounds__(256) k_finish(double* mass_part, unsigned n_mass_part, StepState* st) {
-  __shared__ double red[256];
-  double sm = 0.0;
-  for (unsigned k = threadIdx.x; k < n_mass_part; k += blockDim.x) {
-    sm += mass_part[k];
-    mass_part[k] = 0.0;
-  }
-  red[threadIdx.x] = sm;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    st->last_mass = red[0];
-    st->parity ^= 1;
-    st->psi_skip = 0;
-  }
+  finish_step<256>(mass_part, n_mass_part, st);
 }
 
 // ---- advection ---------------------------------------------------------------------------------
@@ -1080,8 +1084,10 @@ void launch_neighbour_lists(BodyDev* bodies, int nb, const Lat& lat, StepState* 
   if (nb) k_neighbour_lists<<<1, 256, 0, s>>>(bodies, nb, lat, st);
 }
 void launch_flags(const Lat& lat, BodyDev* bodies, int nb, int max_tile, double* arena, uint16_t* flags,
-                  double threshold, int init, StepState* st, cudaStream_t s) {
-  if (nb) k_flags<<<tile_grid(max_tile, nb), 256, 0, s>>>(bodies, arena, flags, lat, threshold, init, st);
+                  double threshold, int init, StepState* st, const MomDev& md, cudaStream_t s) {
+  if (!nb) return;
+  if (md.events) k_flags<true><<<tile_grid(max_tile, nb), 256, 0, s>>>(bodies, arena, flags, lat, threshold, init, st, md);
+  else k_flags<false><<<tile_grid(max_tile, nb), 256, 0, s>>>(bodies, arena, flags, lat, threshold, init, st, md);
 }
 void launch_body_props(const Lat& lat, BodyDev* bodies, int nb, int max_tile, double* arena, double* scratch,
                        cudaStream_t s) {

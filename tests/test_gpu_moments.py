@@ -1,0 +1,174 @@
+"""The moment pass of the bulk fluid (lbm_variant 3: at tau = 1 the cells away from a solid are carried
+as density and momentum, their populations formed where they are pulled) against the split pass
+(lbm_variant 0), through the C ABI.
+
+Both evaluate the same post-collision values from the same density, momentum and force, in another
+association, so they agree to rounding: FP32 within 2e-5 of the largest density and 20 times that of
+the largest velocity (the bounds of the accumulating pass), binary16 storage within its own rounding.
+Sides smaller than a block's column, sides that are no multiple of it or of the 8-cell bricks, and both
+velocity sets cover the edges; free, held and thrown spheres the cells where populations are stored.
+"""
+import os
+import tempfile
+
+import numpy as np
+import pytest
+
+from paper_1902_10432_gb300 import cbl, workloads
+
+pytestmark = pytest.mark.gpu
+
+TOL = {"fp32": 2e-5, "fp16dev": 2e-2}
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import __graft_entry__
+    import torch
+
+    __graft_entry__.build()
+    assert torch.cuda.is_available()
+
+
+def _sim(nx, ny, nz, variant, **kw):
+    s = cbl.Sim(nx, ny, nz, **kw)
+    s.set_option("lbm_variant", variant)
+    assert s.get_option("lbm_variant") == variant
+    return s
+
+
+def _rel(a, b):
+    # a cell that a thrown body uncovers starts empty, and its velocity may overflow: on both sides alike
+    fine = np.isfinite(b)
+    assert np.array_equal(fine, np.isfinite(a))
+    a, b = a[fine], b[fine]
+    return float(np.abs(a - b).max() / max(np.abs(b).max(), 1e-300))
+
+
+def _close(a, b, tol, vtol=20):
+    sa, sb = a.flags()[0], b.flags()[0]
+    assert (sa != sb).sum() == 0
+    (ra, va, pa), (rb, vb, pb) = a.fields(), b.fields()
+    assert _rel(rb, ra) < tol and _rel(vb, va) < vtol * tol, (_rel(rb, ra), _rel(vb, va))
+    assert np.abs(pa - pb).max() < tol
+    fa, fb = a.populations(), b.populations()
+    assert _rel(fb, fa) < tol, _rel(fb, fa)
+    assert a.info()["device_error"] == b.info()["device_error"]
+    if a.info()["device_error"] == 0:
+        assert abs(b.total_mass() - a.total_mass()) < 0.05 * tol * a.total_mass()
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp16dev"])
+@pytest.mark.parametrize("q", [19, 27])
+@pytest.mark.parametrize("dims", [(4, 5, 6), (37, 29, 23), (64, 16, 40), (70, 33, 17), (33, 8, 9)])
+def test_no_bodies_against_split(prec, q, dims):
+    nx, ny, nz = dims
+    rng = np.random.default_rng(nx * 131 + nz)
+    rho = 0.12 + 1.77 * (rng.random((nz, ny, nx)) > 0.55)
+    u = 0.02 * rng.standard_normal((nz, ny, nx, 3))
+    sims = [_sim(nx, ny, nz, v, prec=prec, q=q, ext_force=(1e-4, -2e-4, 5e-5)) for v in (0, 3)]
+    for s in sims:
+        s.init_fluid_fields(rho, u)
+        s.step(5)
+        s.step(7)
+    _close(*sims, TOL[prec])
+
+
+def _spheres(variant, prec="fp32", **kw):
+    w = workloads.small_spheres(prec=prec, mobility=2e-3)
+    s = _sim(w.nx, w.ny, w.nz, variant, **dict(w.params, **kw))
+    workloads.build(s, w)
+    return s
+
+
+@pytest.mark.parametrize("q", [19, 27])
+def test_free_spheres_against_split(q):
+    # light spheres: cells covered and uncovered, the list of cells next to a solid changing every step
+    a, b = (_spheres(v, q=q) for v in (0, 3))
+    for _ in range(4):
+        a.step(25)
+        b.step(25)
+        _close(a, b, 1e-5, 10)
+        assert np.abs(a.bodies()["X"] - b.bodies()["X"]).max() < 1e-6
+    Fa, Fb = a.body_forces()[0], b.body_forces()[0]
+    assert _rel(Fb, Fa) < 1e-4
+
+
+def test_binary16_spheres_against_split():
+    a, b = (_spheres(v, "fp16dev") for v in (0, 3))
+    a.step(10)
+    b.step(10)
+    _close(a, b, TOL["fp16dev"])
+
+
+def test_thrown_sphere_against_split():
+    # seven cells in a step: flags change where no population is stored, so all of them are written first
+    sims = [_spheres(v) for v in (0, 3)]
+    for s in sims:
+        s.step(3)
+        s.set_body_velocities(V=np.array([[0.0, 0.0, -7.0], [0.3, 0.0, 0.0]]))
+        s.step(1)
+        s.set_body_velocities(V=np.zeros((2, 3)))
+        s.step(2)
+    _close(*sims, 1e-4, 20)
+
+
+def test_move_save_load_and_variant_switch():
+    sims = []
+    with tempfile.TemporaryDirectory() as d:
+        for v in (0, 3):
+            s = _spheres(v)
+            s.step(20)
+            f = s.populations()
+            s.step(0)
+            assert np.array_equal(f, s.populations())  # reading changes nothing
+            X = s.bodies()["X"].copy()
+            X[0, 2] -= 0.4
+            s.move_bodies(X)
+            s.step(10)
+            s.set_option("lbm_variant", 3 - v)
+            s.step(7)
+            s.set_option("lbm_variant", v)
+            s.step(3)
+            path = os.path.join(d, "v%d.ckpt" % v)
+            s.save(path)
+            s.step(15)
+            w = workloads.small_spheres(prec="fp32", mobility=2e-3)
+            r = _sim(w.nx, w.ny, w.nz, v, **w.params)
+            for b in w.bodies:
+                bk = dict(b)
+                r.add_body(bk.pop("shape"), **bk)
+            r.load(path)
+            r.step(15)
+            # the resumed run is the uninterrupted one up to the order of FP64 atomic sums
+            assert _rel(r.fields()[0], s.fields()[0]) < 1e-9
+            sims.append(r)
+    _close(*sims, 1e-5, 20)
+
+
+def test_batch_after_moment_steps():
+    a, b = _spheres(0), _spheres(3)
+    c, d = _spheres(0), _spheres(3)
+    a.step(25)
+    b.step(12)
+    batch = cbl.Batch([b, d])
+    batch.step(13)
+    batch.sync()
+    batch.close()
+    c.step(33)
+    d.step(20)
+    _close(a, b, 1e-5, 20)
+    _close(c, d, 1e-5, 20)
+
+
+def test_phase_timing_and_refused_parameters():
+    a, b = _spheres(0), _spheres(3)
+    a.step(9)
+    b.time_phases(4)
+    b.step(5)
+    _close(a, b, 1e-5, 20)
+    for kw in (dict(tau=1.1), dict(prec="fp64")):
+        s = cbl.Sim(16, 16, 16, **dict(dict(prec="fp32"), **kw))
+        with pytest.raises(cbl.CblError):
+            s.set_option("lbm_variant", 3)
+        assert s.get_option("lbm_variant") == 0
