@@ -36,15 +36,23 @@ POP_BYTES = {"fp64": 8, "fp32": 4, "fp16dev": 2}
 
 def kernels_per_step(nb, mpf, variant):
     """Kernel launches of one step of the library's graph: density + bulk collision (variant 0), the
-    fused pass (1), the edge fix-up + accumulating collision (2), or the moment pass (3); the closing
-    kernel (fluid mass, buffer flip); with bodies the tile pass of psi (variants 1 and 2) or the fill and
-    the close of the moment pass (3: it ends the step), the collision of the cells next to a solid, the force pass,
-    repulsion (two or more bodies), body update, three advection sweeps, kinetics (MPF on), flags and
-    refill."""
-    k = (1 if variant in (1, 3) else 2) + 1
-    if nb:
-        k += {0: 0, 1: 1, 2: 1, 3: 1}[variant] + 1 + 1 + (1 if nb > 1 else 0) + 1 + 3 + (1 if mpf else 0) + 2
-    return k
+    fused pass (1), the edge fix-up + accumulating collision (2), or the moment pass (3); without bodies the
+    closing kernel (fluid mass, buffer flip). With bodies their last kernel closes the step: the tile pass
+    of psi (variants 1 and 2) or the fill and the close of the moment pass (3), the collision of the
+    cells next to a solid, the force pass, repulsion (two or more bodies), body update, three advection
+    sweeps, kinetics (MPF on), flags and refill."""
+    k = 1 if variant in (1, 3) else 2
+    if not nb:
+        return k + 1
+    return k + {0: 0, 1: 1, 2: 1, 3: 2}[variant] + 1 + 1 + (1 if nb > 1 else 0) + 1 + 3 + (1 if mpf else 0) + 2
+
+
+def batch_kernels_per_step(variants):
+    """Kernel launches of one step of a persistent batch of pairs: its start, a bulk launch per kind of pass,
+    the collision of the cells next to a solid (split pass) or the fill and the close (moment pass), and one
+    launch over all instances for each kernel of the bodies."""
+    split, mom = any(v != 3 for v in variants), any(v == 3 for v in variants)
+    return 1 + 2 * split + 3 * mom + 9
 
 
 # DRAM bytes per launch of the bulk collision, and per step of the whole step graph, from one-pass
@@ -314,10 +322,7 @@ def bench_batch(args, rank, world, local_rank):
                        "parallelism": "instances sharded over %d GPUs" % world if world > 1 else "single GPU"},
             "sequential_mlups": cells * args.steps / seq_s / 1e6,
             "speedup_vs_sequential": seq_s / bat_s, "clocks": clk.summary(),
-            # persistent mode: one launch for the bulk pass of all instances, then each instance's side
-            # chain (its step without the density and bulk collision kernels, or with the moment pass
-            # without that and the collision of the cells next to a solid)
-            "gpu_launches": args.steps * ((len(set(variants)) + sum(kernels_per_step(2, 1, v) - 2 for v in variants))
+            "gpu_launches": args.steps * (batch_kernels_per_step(variants)
                                           if binfo["mode"] == 1
                                           else sum(n * kernels_per_step(2, 1, json.loads(c).get("lbm_variant", 0))
                                                    for c, n in choices.items()))}

@@ -315,12 +315,12 @@ cbl_status cbl_lbm_step_noalloc(const float* f_in, float* f_out, int nx, int ny,
  * two phases are separated by a grid barrier whose wait is bounded (option "spin_limit", clock64
  * cycles, default ~2 s): a block that waits longer sets an error word and returns, and
  * cbl_batch_sync then returns CBL_ERR_TIMEOUT (that step's results are not valid; the contexts stay
- * usable). Each instance's remaining work (the cells next to a solid, the bodies, the phase fields,
- * flags and refill) follows on its own graph branch. Mode 0: one fork/join branch per instance with
+ * usable). The remaining work (the cells next to a solid, the bodies, the phase fields, flags and
+ * refill) follows with one launch per kernel over all instances and bodies. Mode 0: one fork/join branch per instance with
  * its whole step. The contexts must be initialised (cbl_init_fluid), live on the current device
  * and outlive the batch; while in a batch they must not be stepped on their own. `stream` (may be
  * NULL: the library creates one) orders the batch's work. The batch itself allocates its instance
- * table and control block with cudaMalloc (a few kB). */
+ * tables and control blocks with cudaMalloc (a few kB). */
 typedef struct cbl_batch cbl_batch;
 cbl_status cbl_batch_create(cbl_ctx* const* ctxs, int n, void* stream, cbl_batch** out);
 /* Advance every instance nsteps steps (asynchronous); the fields of the last step are kept. */

@@ -73,7 +73,9 @@ struct cbl_ctx {
   bool mom_state = false;  // the state is in moments (populations complete only after mom_leave)
   int mom_sz = 0;          // planes per block
   MomDev md = {};
-  MomDev md_step() const { return mom ? md : MomDev{}; }
+  ChainState* cs = nullptr;
+  int* events = nullptr;  // cells whose obstacle flag changed in a flag update (capacity: the tiles)
+  int max_xy = 0, max_z = 0;  // largest tile extents: cells per plane, planes
   bool psi_valid = false;  // psi of the current step is in place (else a whole-lattice density pass first)
   int fused_tz = 0;      // > 0: the density and the bulk collision run as one fused pass (k_fused)
   int fused_tz_req = 0;  // requested z extent of a fused block (0 = derived)
@@ -217,12 +219,15 @@ cbl_status cbl_create(const cbl_params* params, const cbl_allocator* alloc, cbl_
   // psi of the split and fused passes (the accumulating pass adds a second buffer when chosen)
   ctx->psi = dalloc(ctx, N * (ctx->prec == 0 ? 8 : 4));
   ctx->nbuf = dalloc(ctx, N * 2 * (ctx->prec == 0 ? 8 : 4));
-  ctx->flags = (uint16_t*)dalloc(ctx, N * 2);
+  ctx->flags = (uint16_t*)dalloc(ctx, (N + 1) / 2 * 4);  // whole 32-bit words (atomics on half words)
   ctx->diag_rho = (double*)dalloc(ctx, N * 8);
   ctx->diag_vel = (double*)dalloc(ctx, N * 24);
   ctx->n_mass_part = MASS_SLOTS;
   ctx->mass_part = (double*)dalloc(ctx, (size_t)ctx->n_mass_part * 8);
-  ctx->st = (StepState*)dalloc(ctx, sizeof(StepState));
+  // step state and, 256 bytes on, the chain's counters
+  static_assert(sizeof(StepState) <= 256, "chain counters behind the step state");
+  ctx->st = (StepState*)dalloc(ctx, 256 + sizeof(ChainState));
+  if (ctx->st) ctx->cs = (ChainState*)((char*)ctx->st + 256);
   if (!ctx->fa || !ctx->fb || !ctx->psi || !ctx->nbuf || !ctx->flags || !ctx->diag_rho || !ctx->diag_vel ||
       !ctx->mass_part || !ctx->st) {
     dfree_all(ctx);
@@ -233,8 +238,9 @@ cbl_status cbl_create(const cbl_params* params, const cbl_allocator* alloc, cbl_
     delete ctx;
     return fail(nullptr, CBL_ERR_OOM, "device allocation failed");
   }
-  cudaMemsetAsync(ctx->flags, 0, N * 2, ctx->s);
+  cudaMemsetAsync(ctx->flags, 0, (N + 1) / 2 * 4, ctx->s);
   cudaMemsetAsync(ctx->st, 0, sizeof(StepState), ctx->s);
+  cudaMemsetAsync(ctx->cs, 0, sizeof(ChainState), ctx->s);
   cudaMemsetAsync(ctx->mass_part, 0, (size_t)ctx->n_mass_part * 8, ctx->s);
   ctx->ops.set_fp16_weights(ctx->s);
   set_repulsion_offsets(p.rc, p.e0, p.nrep, ctx->s);
@@ -328,6 +334,8 @@ cbl_status cbl_add_body(cbl_ctx* ctx, const cbl_body* body, int* body_id) {
   b.off = ctx->arena_n;
   ctx->arena_n += 3 * sz;
   if (sz > ctx->max_tile) ctx->max_tile = (int)sz;
+  ctx->max_xy = std::max(ctx->max_xy, b.L[0] * b.L[1]);
+  ctx->max_z = std::max(ctx->max_z, b.L[2]);
   ctx->hb.push_back(b);
   if (body_id) *body_id = (int)ctx->hb.size() - 1;
   return CBL_OK;
@@ -353,10 +361,58 @@ static cbl_status alloc_bodies(cbl_ctx* ctx) {
   ctx->rtab = (double*)dalloc(ctx, sizeof(double) * 3 * (size_t)ctx->Lmax * nb);
   ctx->mbox = (int*)dalloc(ctx, sizeof(int) * MBOX_N * nb);
   ctx->blist = (int*)dalloc(ctx, sizeof(int) * (size_t)(ctx->arena_n / 3));
+  ctx->events = (int*)dalloc(ctx, sizeof(int) * (size_t)(ctx->arena_n / 3));
   if (!ctx->db || !ctx->arena || !ctx->acc || !ctx->last || !ctx->volacc || !ctx->fsum || !ctx->scratch || !ctx->blist ||
-      !ctx->rtab || !ctx->mbox)
+      !ctx->events || !ctx->rtab || !ctx->mbox)
     return fail(ctx, CBL_ERR_OOM, "device allocation failed (bodies)");
   return CBL_OK;
+}
+
+// what the kernels of the bodies' chain need of a context
+static TileSet tile_set_of(const cbl_ctx* ctx, bool mom) {
+  TileSet t;
+  std::memset(&t, 0, sizeof(t));
+  t.lat = ctx->lat;
+  t.bodies = ctx->db;
+  t.nb = (int)ctx->hb.size();
+  t.Lmax = ctx->Lmax;
+  t.arena = ctx->arena;
+  t.acc = ctx->acc;
+  t.last = ctx->last;
+  t.volacc = ctx->volacc;
+  t.fsum = ctx->fsum;
+  t.rtab = ctx->rtab;
+  t.mbox = ctx->mbox;
+  t.blist = ctx->blist;
+  t.events = ctx->events;
+  t.flags = ctx->flags;
+  t.st = ctx->st;
+  t.cs = ctx->cs;
+  t.fa = ctx->fa;
+  t.fb = ctx->fb;
+  t.nbuf = ctx->nbuf;
+  t.mass_part = ctx->mass_part;
+  t.mom = mom;
+  t.md = ctx->md;
+  t.mpf = ctx->pp.mpf;
+  t.rep = t.nb > 1 && ctx->pp.e0 != 0.0;
+  t.Rc = (int)std::ceil(ctx->pp.rc);
+  t.G = ctx->pp.G;
+  t.G_f = ctx->pp.G_f;
+  t.rc = ctx->pp.rc;
+  t.solid_thr = ctx->p.solid_threshold;
+  t.member_thr = ctx->p.member_threshold;
+  t.kin = kin_params(ctx->pp);
+  return t;
+}
+static ChainLaunch chain_of(const cbl_ctx* ctx, bool mom) {
+  ChainLaunch c;
+  c.one = tile_set_of(ctx, mom);
+  c.bodies = (int)ctx->hb.size();
+  c.max_xy = ctx->max_xy;
+  c.max_z = ctx->max_z;
+  c.share = g_launch_share;
+  return c;
 }
 
 // initial density from a liquid mask on the device (NULL mask: vapour everywhere)
@@ -383,8 +439,7 @@ static cbl_status init_common(cbl_ctx* ctx, const double* rho_host, const double
     CK(cudaMemsetAsync(ctx->fsum, 0, sizeof(double) * 6 * nb, ctx->s));
     launch_rasterize(ctx->lat, ctx->db, nb, ctx->max_tile, ctx->arena, ctx->p.eta, ctx->s);
     launch_neighbour_lists(ctx->db, nb, ctx->lat, ctx->st, ctx->s);
-    launch_flags(ctx->lat, ctx->db, nb, ctx->max_tile, ctx->arena, ctx->flags, ctx->p.solid_threshold, 1, ctx->st,
-                 MomDev{}, ctx->s);
+    launch_flags(chain_of(ctx, false), 1, ctx->s);
     launch_body_props(ctx->lat, ctx->db, nb, ctx->max_tile, ctx->arena, ctx->scratch, ctx->s);
   }
   double* drho = (double*)dalloc(ctx, N * 8);
@@ -402,8 +457,8 @@ static cbl_status init_common(cbl_ctx* ctx, const double* rho_host, const double
   ctx->ops.init_fluid(ctx->prec, ctx->lat, ctx->fa, ctx->flags, drho, du, ctx->s);
   // first boundary-cell list (no cover events yet, so the pass only scans) and member boxes
   reset_member_boxes(ctx);
-  ctx->ops.refill(ctx->prec, ctx->lat, ctx->fa, ctx->fb, ctx->flags, ctx->db, nb, ctx->max_tile, ctx->st, ctx->blist,
-                ctx->arena, ctx->p.member_threshold, ctx->mbox, 0, ctx->s);
+  ctx->ops.near_refill(ctx->prec, chain_of(ctx, false), 0, ctx->s);
+  launch_commit(ctx->st, ctx->cs, ctx->s);
   CK(cudaMemsetAsync(ctx->diag_rho, 0, N * 8, ctx->s));
   CK(cudaMemsetAsync(ctx->diag_vel, 0, N * 24, ctx->s));
   CK(cudaGetLastError());
@@ -507,23 +562,29 @@ static void enqueue_bulk(cbl_ctx* ctx, cudaStream_t s) {
 // New obstacle flags, cover refill, boundary-cell list; with the moment pass, the populations that a
 // flag change outside the stored bricks needs, and psi and moments around the changes.
 static void enqueue_refill(cbl_ctx* ctx, cudaStream_t s) {
-  const int nb = (int)ctx->hb.size();
   if (ctx->mom)
-    ctx->ops.mom_fill(ctx->prec, ctx->lat, ctx->fa, ctx->fb, ctx->st, ctx->psi, ctx->psi2, ctx->md, ctx->pp, 1, s);
-  ctx->ops.refill(ctx->prec, ctx->lat, ctx->fa, ctx->fb, ctx->flags, ctx->db, nb, ctx->max_tile, ctx->st, ctx->blist,
-                  ctx->arena, ctx->p.member_threshold, ctx->mbox, 1, s);
+    ctx->ops.mom_fill(ctx->prec, ctx->lat, ctx->fa, ctx->fb, ctx->st, ctx->psi, ctx->psi2, ctx->md, ctx->cs, ctx->pp, 1, s);
+  ctx->ops.near_refill(ctx->prec, chain_of(ctx, ctx->mom), 1, s);
   if (ctx->mom)
     ctx->ops.mom_close(ctx->prec, ctx->lat, ctx->fa, ctx->fb, ctx->st, ctx->flags, ctx->psi, ctx->psi2, ctx->md,
-                       ctx->blist, ctx->pp, 1, ctx->mass_part, s);  // and the step's end
+                       ctx->events, ctx->cs, ctx->blist, ctx->pp, 1, ctx->mass_part, s);  // and the step's end
 }
-// end of the step; the moment pass's last kernel does it where there are bodies
+// end of the step; the refill (or the moment pass's close) does it where there are bodies
 static void enqueue_finish(cbl_ctx* ctx, cudaStream_t s) {
-  if (!ctx->mom || ctx->hb.empty()) launch_finish(ctx->mass_part, ctx->n_mass_part, ctx->st, s);
+  if (ctx->hb.empty()) launch_finish(ctx->mass_part, ctx->n_mass_part, ctx->st, ctx->cs, s);
 }
 static void enqueue_flags_refill(cbl_ctx* ctx, cudaStream_t s) {
-  launch_flags(ctx->lat, ctx->db, (int)ctx->hb.size(), ctx->max_tile, ctx->arena, ctx->flags, ctx->p.solid_threshold, 0,
-               ctx->st, ctx->md_step(), s);
+  launch_flags(chain_of(ctx, ctx->mom), 0, s);
   enqueue_refill(ctx, s);
+}
+// solid-fluid force, repulsion, body update, advection and kinetics
+static void enqueue_bodies(cbl_ctx* ctx, cudaStream_t s) {
+  const ChainLaunch c = chain_of(ctx, ctx->mom);
+  ctx->ops.boundary(ctx->prec, c, s);
+  if (c.one.rep) launch_repulsion(c, s);
+  launch_bodies(c, s);
+  launch_advect(c, s);
+  if (ctx->pp.mpf) launch_kinetics(c, s);
 }
 
 // One step, enqueued for capture into a graph. With bodies, the collision of the cells next to a
@@ -532,11 +593,6 @@ static void enqueue_flags_refill(cbl_ctx* ctx, cudaStream_t s) {
 // accumulators with atomics); the body update joins both.
 static void enqueue_step(cbl_ctx* ctx) {
   const int nb = (int)ctx->hb.size();
-  auto phase_update = [&](cudaStream_t s) {
-    launch_advect(ctx->lat, ctx->db, nb, ctx->max_tile, ctx->arena, ctx->pp.mpf, ctx->volacc, ctx->st, ctx->rtab,
-                  ctx->Lmax, s);
-    if (ctx->pp.mpf) launch_kinetics(ctx->lat, ctx->db, nb, ctx->max_tile, ctx->arena, ctx->volacc, ctx->pp, s);
-  };
   if (nb && ctx->branches) {
     // The bulk collision (every cell without a solid neighbour) runs beside the chain that needs only
     // the source populations, psi and the phase fields: collision of the cells next to a solid, force
@@ -551,12 +607,7 @@ static void enqueue_step(cbl_ctx* ctx) {
     cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0);
     if (ctx->fused_tz) enqueue_lbm(ctx, 1, ctx->side);
     if (!ctx->mom) enqueue_lbm(ctx, 4, ctx->side);
-    ctx->ops.boundary(ctx->prec, ctx->lat, ctx->fa, ctx->fb, ctx->flags, ctx->db, nb, ctx->acc, ctx->blist, ctx->st,
-                    ctx->nbuf, ctx->pp.G, ctx->side);
-    launch_repulsion(ctx->lat, ctx->db, nb, ctx->max_tile, ctx->arena, ctx->acc, ctx->pp, ctx->mbox, ctx->side);
-    launch_bodies(ctx->lat, ctx->db, nb, ctx->acc, ctx->last, ctx->volacc, ctx->st, ctx->rtab, ctx->Lmax, ctx->mbox, ctx->fsum,
-                  ctx->side);
-    phase_update(ctx->side);
+    enqueue_bodies(ctx, ctx->side);
     cudaEventRecord(ctx->ev_join, ctx->side);
     enqueue_bulk(ctx, ctx->s);
     cudaStreamWaitEvent(ctx->s, ctx->ev_join, 0);
@@ -565,34 +616,10 @@ static void enqueue_step(cbl_ctx* ctx) {
     enqueue_lbm(ctx, ctx->mom ? 4 : 1, ctx->s);
     enqueue_bulk(ctx, ctx->s);
     if (!ctx->mom) enqueue_lbm(ctx, 4, ctx->s);
-    ctx->ops.boundary(ctx->prec, ctx->lat, ctx->fa, ctx->fb, ctx->flags, ctx->db, nb, ctx->acc, ctx->blist, ctx->st,
-                    ctx->nbuf, ctx->pp.G, ctx->s);
     if (nb) {
-      launch_repulsion(ctx->lat, ctx->db, nb, ctx->max_tile, ctx->arena, ctx->acc, ctx->pp, ctx->mbox, ctx->s);
-      launch_bodies(ctx->lat, ctx->db, nb, ctx->acc, ctx->last, ctx->volacc, ctx->st, ctx->rtab, ctx->Lmax,
-                    ctx->mbox, ctx->fsum, ctx->s);
-      phase_update(ctx->s);
+      enqueue_bodies(ctx, ctx->s);
       enqueue_flags_refill(ctx, ctx->s);
     }
-  }
-  enqueue_finish(ctx, ctx->s);
-}
-
-// The part of a step that follows the bulk lattice-Boltzmann pass in a persistent batch launch: the
-// collision of the cells next to a solid, the bodies' chain, flags and refill, the step's end.
-static void enqueue_side_chain(cbl_ctx* ctx) {
-  const int nb = (int)ctx->hb.size();
-  if (!ctx->mom) enqueue_lbm(ctx, 4, ctx->s);  // with the moment pass, in the persistent launch
-  if (nb) {
-    ctx->ops.boundary(ctx->prec, ctx->lat, ctx->fa, ctx->fb, ctx->flags, ctx->db, nb, ctx->acc, ctx->blist, ctx->st,
-                      ctx->nbuf, ctx->pp.G, ctx->s);
-    launch_repulsion(ctx->lat, ctx->db, nb, ctx->max_tile, ctx->arena, ctx->acc, ctx->pp, ctx->mbox, ctx->s);
-    launch_bodies(ctx->lat, ctx->db, nb, ctx->acc, ctx->last, ctx->volacc, ctx->st, ctx->rtab, ctx->Lmax, ctx->mbox, ctx->fsum,
-                  ctx->s);
-    launch_advect(ctx->lat, ctx->db, nb, ctx->max_tile, ctx->arena, ctx->pp.mpf, ctx->volacc, ctx->st, ctx->rtab,
-                  ctx->Lmax, ctx->s);
-    if (ctx->pp.mpf) launch_kinetics(ctx->lat, ctx->db, nb, ctx->max_tile, ctx->arena, ctx->volacc, ctx->pp, ctx->s);
-    enqueue_flags_refill(ctx, ctx->s);
   }
   enqueue_finish(ctx, ctx->s);
 }
@@ -640,7 +667,7 @@ static bool mom_rule(const cbl_ctx* ctx) {
 // complete populations from a state in moments, for whatever reads or changes them outside the step
 static cbl_status mom_leave(cbl_ctx* ctx, bool stay) {
   if (!ctx->mom_state) return CBL_OK;
-  ctx->ops.mom_fill(ctx->prec, ctx->lat, ctx->fa, ctx->fb, ctx->st, ctx->psi, ctx->psi2, ctx->md, ctx->pp, 0, ctx->s);
+  ctx->ops.mom_fill(ctx->prec, ctx->lat, ctx->fa, ctx->fb, ctx->st, ctx->psi, ctx->psi2, ctx->md, ctx->cs, ctx->pp, 0, ctx->s);
   CK(cudaGetLastError());
   if (!stay) ctx->mom_state = false;
   return CBL_OK;
@@ -651,8 +678,8 @@ static cbl_status mom_enter(cbl_ctx* ctx) {
   if (ctx->mom_state) return CBL_OK;
   ctx->ops.mom_enter(ctx->prec, ctx->lat, ctx->fa, ctx->fb, ctx->st, ctx->flags, ctx->psi, ctx->psi2, ctx->md, ctx->pp,
                      ctx->s);
-  ctx->ops.mom_close(ctx->prec, ctx->lat, ctx->fa, ctx->fb, ctx->st, ctx->flags, ctx->psi, ctx->psi2, ctx->md, ctx->blist,
-                     ctx->pp, 0, ctx->mass_part, ctx->s);
+  ctx->ops.mom_close(ctx->prec, ctx->lat, ctx->fa, ctx->fb, ctx->st, ctx->flags, ctx->psi, ctx->psi2, ctx->md, ctx->events,
+                     ctx->cs, ctx->blist, ctx->pp, 0, ctx->mass_part, ctx->s);
   CK(cudaGetLastError());
   ctx->mom_state = true;
   return CBL_OK;
@@ -674,16 +701,16 @@ static cbl_status mom_prepare(cbl_ctx* ctx) {
   if (use && !ctx->md.M0) {
     const size_t N = (size_t)ctx->lat.N;
     MomDev& d = ctx->md;
-    d.nbx = (ctx->lat.nx + 7) / 8;
-    d.nby = (ctx->lat.ny + 7) / 8;
-    d.nbz = (ctx->lat.nz + 7) / 8;
+    d.nbx = (ctx->lat.nx - 1 >> BRICK_BITS) + 1;
+    d.nby = (ctx->lat.ny - 1 >> BRICK_BITS) + 1;
+    d.nbz = (ctx->lat.nz - 1 >> BRICK_BITS) + 1;
     const size_t bricks = (size_t)d.nbx * d.nby * d.nbz;
     const size_t mark = ctx->allocs.size();
     d.M0 = (float4*)dalloc(ctx, N * sizeof(float4));
     d.M1 = d.M0 ? (float4*)dalloc(ctx, N * sizeof(float4)) : nullptr;
     if (d.M1 && !ctx->psi2) ctx->psi2 = dalloc(ctx, N * 4);
     unsigned char* small = d.M1 && ctx->psi2
-                               ? (unsigned char*)dalloc(ctx, 256 + 2 * bricks + 256 + sizeof(int) * (size_t)(ctx->arena_n / 3 + 1))
+                               ? (unsigned char*)dalloc(ctx, 2 * bricks)
                                : nullptr;
     if (!small) {
       for (size_t k = mark; k < ctx->allocs.size(); ++k) {
@@ -697,11 +724,8 @@ static cbl_status mom_prepare(cbl_ctx* ctx) {
       ctx->mom_req = 0;
       use = false;
     } else {
-      d.ms = (MomState*)small;
-      d.map0 = small + 256;
+      d.map0 = small;
       d.map1 = d.map0 + bricks;
-      d.events = (int*)(small + 256 + (2 * bricks + 255) / 256 * 256);
-      CK(cudaMemsetAsync(d.ms, 0, sizeof(MomState), ctx->s));
       ctx->mom_sz = ctx->ops.mom_sz(ctx->lat, 1);
       CK(ctx->ops.mom(ctx->prec, ctx->lat, ctx->fa, ctx->fb, ctx->flags, ctx->psi, ctx->psi2, d, ctx->mass_part, ctx->st,
                       ctx->diag_rho, ctx->diag_vel, ctx->pp, 0, ctx->s));
@@ -807,24 +831,18 @@ cbl_status cbl_time_phases(cbl_ctx* ctx, int nsteps, double* ms) {
     CK(cudaEventRecord(ev[1], ctx->s));
     enqueue_lbm(ctx, 6, ctx->s);
     CK(cudaEventRecord(ev[2], ctx->s));
-    ctx->ops.boundary(ctx->prec, ctx->lat, ctx->fa, ctx->fb, ctx->flags, ctx->db, nb, ctx->acc, ctx->blist, ctx->st,
-                    ctx->nbuf, ctx->pp.G, ctx->s);
+    const ChainLaunch c = chain_of(ctx, ctx->mom);
+    ctx->ops.boundary(ctx->prec, c, ctx->s);
     CK(cudaEventRecord(ev[3], ctx->s));
-    if (nb) launch_repulsion(ctx->lat, ctx->db, nb, ctx->max_tile, ctx->arena, ctx->acc, ctx->pp, ctx->mbox, ctx->s);
+    if (c.one.rep) launch_repulsion(c, ctx->s);
     CK(cudaEventRecord(ev[4], ctx->s));
-    launch_bodies(ctx->lat, ctx->db, nb, ctx->acc, ctx->last, ctx->volacc, ctx->st, ctx->rtab, ctx->Lmax, ctx->mbox, ctx->fsum,
-                  ctx->s);
+    launch_bodies(c, ctx->s);
     CK(cudaEventRecord(ev[5], ctx->s));
-    if (nb)
-      launch_advect(ctx->lat, ctx->db, nb, ctx->max_tile, ctx->arena, ctx->pp.mpf, ctx->volacc, ctx->st, ctx->rtab,
-                    ctx->Lmax, ctx->s);
+    launch_advect(c, ctx->s);
     CK(cudaEventRecord(ev[6], ctx->s));
-    if (nb && ctx->pp.mpf)
-      launch_kinetics(ctx->lat, ctx->db, nb, ctx->max_tile, ctx->arena, ctx->volacc, ctx->pp, ctx->s);
+    if (ctx->pp.mpf) launch_kinetics(c, ctx->s);
     CK(cudaEventRecord(ev[7], ctx->s));
-    if (nb)
-      launch_flags(ctx->lat, ctx->db, nb, ctx->max_tile, ctx->arena, ctx->flags, ctx->p.solid_threshold, 0, ctx->st,
-                   ctx->md_step(), ctx->s);
+    launch_flags(c, 0, ctx->s);
     CK(cudaEventRecord(ev[8], ctx->s));
     if (nb) enqueue_refill(ctx, ctx->s);
     enqueue_finish(ctx, ctx->s);
@@ -1091,15 +1109,15 @@ cbl_status cbl_move_bodies(cbl_ctx* ctx, const double* X, const double* Qn, cons
     CK(cudaMemcpyAsync(ctx->db, h.data(), sizeof(BodyDev) * nb, cudaMemcpyHostToDevice, ctx->s));
     launch_rasterize(ctx->lat, ctx->db, nb, ctx->max_tile, ctx->arena, ctx->p.eta, ctx->s);
     launch_neighbour_lists(ctx->db, nb, ctx->lat, ctx->st, ctx->s);
-    // cover events are counted by the flag pass; the boundary list is rebuilt by the refill pass
+    // cover events are counted by the flag pass; the boundary list is rebuilt by the refill pass, and its
+    // near-solid bits went with the flags under the tiles
     CK(cudaMemsetAsync(&ctx->st->ncover, 0, sizeof(unsigned), ctx->s));
     CK(cudaMemsetAsync(&ctx->st->nbnd, 0, sizeof(unsigned), ctx->s));
-    launch_flags(ctx->lat, ctx->db, nb, ctx->max_tile, ctx->arena, ctx->flags, ctx->p.solid_threshold, 0, ctx->st,
-                 MomDev{}, ctx->s);
+    launch_flags(chain_of(ctx, false), 0, ctx->s);
     launch_clear_stale(ctx->lat, ctx->flags, ctx->s);
     reset_member_boxes(ctx);
-    ctx->ops.refill(ctx->prec, ctx->lat, ctx->fa, ctx->fb, ctx->flags, ctx->db, nb, ctx->max_tile, ctx->st, ctx->blist,
-                  ctx->arena, ctx->p.member_threshold, ctx->mbox, 0, ctx->s);
+    ctx->ops.near_refill(ctx->prec, chain_of(ctx, false), 0, ctx->s);
+    launch_commit(ctx->st, ctx->cs, ctx->s);
     CK(cudaGetLastError());
     // the host copy h (and the device memcpy source) must outlive the copy
     CK(cudaStreamSynchronize(ctx->s));
@@ -1316,6 +1334,9 @@ cbl_status cbl_load(cbl_ctx* ctx, const char* path) {
   if (st != CBL_OK) return st;
   if (!ok) return fail(ctx, CBL_ERR_ARG, std::string(path) + " is truncated");
   CK(cudaMemsetAsync(ctx->mass_part, 0, (size_t)ctx->n_mass_part * 8, ctx->s));
+  CK(cudaMemsetAsync(ctx->cs, 0, sizeof(ChainState), ctx->s));
+  launch_clear_cover(ctx->lat, ctx->flags, ctx->s);  // of the last flag update before the save: used up
+  CK(cudaGetLastError());
   if (nb) CK(cudaMemsetAsync(ctx->fsum, 0, sizeof(double) * 6 * nb, ctx->s));  // running sums start anew
   ctx->fsum_steps = 0;
   CK(cudaStreamSynchronize(ctx->s));
@@ -1453,56 +1474,80 @@ struct cbl_batch {
   // instances on the split pass [0] and on the moment pass [1]: their number, work items, grid; the table
   // holds those of the split pass first, and each group has its control block
   int n[2] = {0, 0}, grid[2] = {0, 0}, sz = 0;
-  long long items[2] = {0, 0};
+  long long items_n[2] = {0, 0};
   std::vector<char> mom;                // per context: 1 = on the moment pass
   long long spin_limit = 4000000000LL;  // clock64 cycles a block may wait at the grid barrier (~2 s)
   BatchInst* tab = nullptr;
   BatchCtl* ctl = nullptr;  // two
+  // the bodies' chain of every instance, a launch per kernel: contexts and their bodies (device)
+  TileSet* sets = nullptr;
+  int2* items = nullptr;
+  ChainLaunch chain;
 };
+
+// Persistent mode: the bulk pass of every instance in one launch (or two, split and moment pass), then the
+// bodies' chain of every instance with one launch per kernel: a batch of 64 pairs of spheres has 13 launches
+// per step instead of 750 on 64 branches (7.5 ms per step; each is too short to fill the GPU and waits
+// for its turn).
+static cudaError_t batch_enqueue(cbl_batch* b, int diag) {
+  cbl_ctx* c0 = b->ctxs[0];
+  const LbmOps& ops = c0->ops;
+  cudaStream_t s = b->s;
+  ops.batch_begin(b->tab, (int)b->ctxs.size(), b->ctl, diag, s);
+  const BatchInst* const mom = b->tab + b->n[0];
+  for (int k = 0; k < 2; ++k) {
+    if (!b->n[k]) continue;
+    const cudaError_t e =
+        k ? ops.batch_mom(c0->prec, mom, b->n[1], b->items_n[1], b->ctl + 1, b->grid[1], b->sz, b->cooperative, s)
+          : ops.batch_lbm(c0->prec, b->tile_cfg, b->tab, b->n[0], b->items_n[0], b->ctl, b->grid[0], b->cooperative, s);
+    if (e != cudaSuccess) return e;
+  }
+  const ChainLaunch& c = b->chain;
+  if (c.bodies) {
+    if (b->n[0]) ops.batch_near(c0->prec, b->tab, b->n[0], s);
+    ops.boundary(c0->prec, c, s);
+    launch_repulsion(c, s);
+    launch_bodies(c, s);
+    launch_advect(c, s);
+    launch_kinetics(c, s);
+    launch_flags(c, 0, s);
+    if (b->n[1]) ops.batch_fill(c0->prec, mom, b->n[1], s);
+    ops.near_refill(c0->prec, c, 1, s);
+    if (b->n[1]) ops.batch_close(c0->prec, mom, b->n[1], s);
+  }
+  for (size_t k = 0; k < b->ctxs.size(); ++k)
+    if (b->ctxs[k]->hb.empty()) launch_finish(b->ctxs[k]->mass_part, b->ctxs[k]->n_mass_part, b->ctxs[k]->st, b->ctxs[k]->cs, s);
+  return cudaSuccess;
+}
 
 static cudaError_t batch_capture(cbl_batch* b, int diag, cudaGraph_t* g) {
   cudaError_t e = cudaStreamBeginCapture(b->s, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return e;
-  // the instances' kernels run side by side: each sizes its device-sized grids for its share
-  LaunchShare share((int)std::min<size_t>(b->ctxs.size(), 64));
   cudaError_t el = cudaSuccess;
   if (b->mode == 1) {
-    cbl_ctx* c0 = b->ctxs[0];
-    for (cbl_ctx* c : b->ctxs) cudaMemsetAsync(&c->st->diag, diag, sizeof(int), b->s);
-    for (int k = 0; k < 2; ++k) {
-      if (!b->n[k]) continue;
-      cudaMemsetAsync(b->ctl + k, 0, BATCH_CTL_RESET_BYTES, b->s);
-      if (k)
-        el = c0->ops.batch_mom(c0->prec, b->tab + b->n[0], b->n[1], b->items[1], b->ctl + 1, b->grid[1], b->sz,
-                               b->cooperative, b->s);
-      else
-        el = c0->ops.batch_lbm(c0->prec, b->tile_cfg, b->tab, b->n[0], b->items[0], b->ctl, b->grid[0], b->cooperative,
-                               b->s);
-      if (el != cudaSuccess) break;
-    }
-  }
-  cudaEventRecord(b->events[0], b->s);
-  for (size_t k = 0; k < b->ctxs.size(); ++k) {
-    cbl_ctx* c = b->ctxs[k];
-    cudaStream_t br = b->branches[k];
-    cudaStreamWaitEvent(br, b->events[0], 0);
-    cudaStream_t keep = c->s;
-    const int keep_acc = c->acc_pass;
-    const bool keep_mom = c->mom;
-    c->s = br;
-    c->acc_pass = 0;  // a batch runs these instances with the split pass (one psi buffer)
-    c->mom = b->mom[k];
-    if (b->mode == 1) {
-      enqueue_side_chain(c);
-    } else {
+    el = batch_enqueue(b, diag);
+  } else {
+    // the instances' kernels run side by side: each sizes its device-sized grids for its share
+    LaunchShare share((int)std::min<size_t>(b->ctxs.size(), 64));
+    cudaEventRecord(b->events[0], b->s);
+    for (size_t k = 0; k < b->ctxs.size(); ++k) {
+      cbl_ctx* c = b->ctxs[k];
+      cudaStream_t br = b->branches[k];
+      cudaStreamWaitEvent(br, b->events[0], 0);
+      cudaStream_t keep = c->s;
+      const int keep_acc = c->acc_pass;
+      const bool keep_mom = c->mom;
+      c->s = br;
+      c->acc_pass = 0;  // a batch runs these instances with the split pass (one psi buffer)
+      c->mom = b->mom[k];
       cudaMemsetAsync(&c->st->diag, diag, sizeof(int), br);
       enqueue_step(c);
+      c->s = keep;
+      c->acc_pass = keep_acc;
+      c->mom = keep_mom;
+      cudaEventRecord(b->events[k + 1], br);
+      cudaStreamWaitEvent(b->s, b->events[k + 1], 0);
     }
-    c->s = keep;
-    c->acc_pass = keep_acc;
-    c->mom = keep_mom;
-    cudaEventRecord(b->events[k + 1], br);
-    cudaStreamWaitEvent(b->s, b->events[k + 1], 0);
   }
   cudaError_t e1 = cudaGetLastError();
   cudaError_t e2 = cudaStreamEndCapture(b->s, g);
@@ -1577,6 +1622,8 @@ static cudaError_t batch_build(cbl_batch* b) {
         I.psi2 = c->psi2;
         I.nbuf = c->nbuf;
         I.blist = c->blist;
+        I.events = c->events;
+        I.cs = c->cs;
         if (kind) I.md = c->md;
         const int n[3] = {c->lat.nx, c->lat.ny, c->lat.nz};
         for (int a = 0; a < 3; ++a) I.tiles[a] = (n[a] + t[a] - 1) / t[a];
@@ -1585,9 +1632,28 @@ static cudaError_t batch_build(cbl_batch* b) {
         h.push_back(I);
         ++b->n[kind];
       }
-      b->items[kind] = items;
+      b->items_n[kind] = items;
     }
     cudaError_t e = cudaMemcpy(b->tab, h.data(), sizeof(BatchInst) * h.size(), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) return e;
+    std::vector<TileSet> sets;
+    std::vector<int2> items;
+    ChainLaunch& ch = b->chain;
+    ch = ChainLaunch{};
+    for (size_t k = 0; k < b->ctxs.size(); ++k) {
+      const cbl_ctx* c = b->ctxs[k];
+      sets.push_back(tile_set_of(c, b->mom[k] != 0));
+      for (int q = 0; q < (int)c->hb.size(); ++q) items.push_back(make_int2((int)k, q));
+      ch.max_xy = std::max(ch.max_xy, c->max_xy);
+      ch.max_z = std::max(ch.max_z, c->max_z);
+    }
+    ch.bodies = (int)items.size();
+    ch.inst = ch.share = (int)sets.size();
+    ch.sets = b->sets;
+    ch.items = b->items;
+    e = cudaMemcpy(b->sets, sets.data(), sizeof(TileSet) * sets.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess && ch.bodies)
+      e = cudaMemcpy(b->items, items.data(), sizeof(int2) * items.size(), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
@@ -1646,6 +1712,10 @@ cbl_status cbl_batch_create(cbl_ctx* const* ctxs, int n, void* stream, cbl_batch
   for (int k = 0; k <= n; ++k) ok &= cudaEventCreateWithFlags(&b->events[k], cudaEventDisableTiming) == cudaSuccess;
   ok &= cudaMalloc(&b->tab, sizeof(BatchInst) * n) == cudaSuccess;
   ok &= cudaMalloc(&b->ctl, 2 * sizeof(BatchCtl)) == cudaSuccess;
+  size_t bodies = 1;
+  for (int k = 0; k < n; ++k) bodies += ctxs[k]->hb.size();
+  ok &= cudaMalloc(&b->sets, sizeof(TileSet) * n) == cudaSuccess;
+  ok &= cudaMalloc(&b->items, sizeof(int2) * bodies) == cudaSuccess;
   if (ok && batch_build(b) != cudaSuccess && b->mode == 1) {
     // a cooperative kernel that cannot be captured: the same launch, plain (the grid is sized to be
     // resident, and the barrier's wait is bounded either way)
@@ -1693,7 +1763,7 @@ cbl_status cbl_batch_info(cbl_batch* b, int* mode, int* tile, long long* items, 
   if (!b) return fail(nullptr, CBL_ERR_ARG, "NULL batch");
   if (mode) *mode = b->mode;
   if (tile) *tile = b->tile_cfg;
-  if (items) *items = b->items[0] + b->items[1];
+  if (items) *items = b->items_n[0] + b->items_n[1];
   if (grid) *grid = std::max(b->grid[0], b->grid[1]);
   return CBL_OK;
 }
@@ -1739,6 +1809,8 @@ cbl_status cbl_batch_destroy(cbl_batch* b) {
     if (e) cudaEventDestroy(e);
   if (b->tab) cudaFree(b->tab);
   if (b->ctl) cudaFree(b->ctl);
+  if (b->sets) cudaFree(b->sets);
+  if (b->items) cudaFree(b->items);
   if (b->own_stream) cudaStreamDestroy(b->s);
   delete b;
   return CBL_OK;

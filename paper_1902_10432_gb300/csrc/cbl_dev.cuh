@@ -138,6 +138,17 @@ struct StepState {
   unsigned ncover;   // nodes covered in this step's flag update
 };
 
+// Counters of one step: obstacle flags that changed in its flag update (cells in `events`), and in the last
+// one (nprev: their cover bits are cleared by the body update of this step); entries of the
+// boundary list that is being built (the list of the step to come; StepState::nbnd counts the current
+// one); moment pass: whether a flag changed where populations are not stored, and the blocks of the
+// step's last kernel that are through.
+struct ChainState {
+  unsigned nevent, nprev, nnew;
+  int full;
+  unsigned done;
+};
+
 struct PhysParams {
   double tau, G, rho0;
   double ext[3];
@@ -154,8 +165,9 @@ struct PhysParams {
 // End of a step, by one block of T threads: the fluid mass (fixed-order sum of the collision's partials,
 // which are cleared) and the population buffer flip. The bulk collision may run beside the body
 // update, so neither can happen earlier.
+// The boundary list that the refill built becomes the current one.
 template <int T>
-__device__ __forceinline__ void finish_step(double* mass_part, unsigned n_mass_part, StepState* st) {
+__device__ __forceinline__ void finish_step(double* mass_part, unsigned n_mass_part, StepState* st, ChainState* cs) {
   __shared__ double red[T];
   double sm = 0.0;
   for (unsigned k = threadIdx.x; k < n_mass_part; k += T) {
@@ -172,6 +184,11 @@ __device__ __forceinline__ void finish_step(double* mass_part, unsigned n_mass_p
     st->last_mass = red[0];
     st->parity ^= 1;
     st->psi_skip = 0;
+    st->nbnd = cs->nnew;
+    cs->nnew = 0;
+    cs->nprev = cs->nevent;
+    cs->nevent = 0;
+    cs->full = 0;
   }
 }
 
@@ -198,21 +215,12 @@ __device__ __forceinline__ long long dbits(double v) { return __double_as_longlo
 // wrapi, mimg, wrapd: periodic wraps with a fixed operation count (periodic.h)
 
 // ---- moment pass (moments.cuh) -----------------------------------------------------------------
-// Per-step state of the moment pass: obstacle flags that changed in this step's flag update (cells in
-// `events`), and whether one changed where populations are not stored.
-struct MomState {
-  unsigned nevent;
-  int full;
-  unsigned done;  // blocks of the step's last kernel that are through
-};
 // Buffers of the moment pass, indexed by the parity of the step they belong to: moments (rho, m) of
-// every cell, and a byte per brick of 8 x 8 x 8 cells in which populations are stored.
+// every cell, and a byte per brick in which populations are stored.
 struct MomDev {
   float4 *M0, *M1;
   unsigned char *map0, *map1;
   int nbx, nby, nbz;  // bricks per axis
-  int* events;        // NULL: the step does not run the moment pass
-  MomState* ms;
   // (selected, not indexed: an index into a kernel parameter would copy it to local memory)
   __device__ float4* M(int q) const { return q ? M1 : M0; }
   __device__ unsigned char* map(int q) const { return q ? map1 : map0; }
@@ -220,8 +228,57 @@ struct MomDev {
   __device__ unsigned bricks() const { return (unsigned)(nbx * nby * nbz); }
 };
 
-// Bricks along one axis that the cells within r (<= 4) of cell g of a periodic side n touch: at most
-// two of 8 cells, and at the periodic seam, where the last brick may be short, those beside it.
+// Kinetics constants evaluated once on the host with the expressions the kernel would use per cell (IEEE
+// division is correctly rounded on both sides, so the values are identical): pi^2 / eta^2 and M / N for
+// every possible number of active phases N (an FP64 division costs many FP64-pipe instructions, and
+// GB300 issues FP64 at 1/64 of the FP32 rate).
+constexpr int MAXACT = 8;
+struct KinParams {
+  double k2, s_sf, s_ss;
+  double mobN[MAXACT + 2];
+};
+
+// What the kernels of the bodies' chain need of one context: a kernel argument for a single context, an
+// entry of a device table for a batch.
+struct TileSet {
+  Lat lat;
+  BodyDev* bodies;
+  int nb, Lmax;
+  double *arena, *acc, *last, *volacc, *fsum, *rtab;
+  int *mbox, *blist, *events;
+  uint16_t* flags;
+  StepState* st;
+  ChainState* cs;
+  void *fa, *fb, *nbuf;
+  double* mass_part;
+  int mom;  // the step runs the moment pass
+  MomDev md;
+  int mpf, rep, Rc;  // kinetics on, repulsion on
+  float G_f;
+  double G, rc, solid_thr, member_thr;
+  KinParams kin;
+};
+
+// A launch over the tiles of a context, or of all contexts of a batch (sets: device table; items: context and
+// body of every body; inst: contexts). Extents are those of the largest tile.
+struct ChainLaunch {
+  TileSet one;
+  const TileSet* sets = nullptr;
+  const int2* items = nullptr;
+  int bodies = 0, inst = 1;
+  int max_xy = 0, max_z = 0;
+  int share = 1;  // contexts that the launch serves at once (sizes the grids whose work is known on the device)
+};
+
+// Bricks of 4 cells a side in which the moment pass stores populations: those within BRICK_REACH cells of a cell
+// next to a solid. A covered cell is one of these, and what it touches (k_mom_close) is pulled from
+// within 3 cells; an uncovered cell is next to one, and what it touches is pulled from within 2.
+// Around a sphere of R = 24 these hold 75 700 fluid cells (R = 12: 23 600); bricks of 8 held 119 300 (29 600),
+// and need no fewer marks.
+constexpr int BRICK_BITS = 2, BRICK_REACH = 3;
+
+// Bricks along one axis that the cells within r (<= BRICK_REACH) of cell g of a periodic side n touch: at most
+// three, and at the periodic seam, where the last brick may be short, those beside it.
 constexpr int BRICK_SPAN = 5;
 __device__ __forceinline__ int brick_span(int g, int r, int n, int b[BRICK_SPAN]) {
   int cnt = 0;
@@ -230,11 +287,11 @@ __device__ __forceinline__ int brick_span(int g, int r, int n, int b[BRICK_SPAN]
       if (b[k] == v) return;
     b[cnt++] = v;
   };
-  add(wrapi_near(g - r, n) >> 3);
-  add(g >> 3);
-  add(wrapi_near(g + r, n) >> 3);
+  add(wrapi_near(g - r, n) >> BRICK_BITS);
+  add(g >> BRICK_BITS);
+  add(wrapi_near(g + r, n) >> BRICK_BITS);
   if (g - r < 0 || g + r >= n) {
-    add((n - 1) >> 3);
+    add((n - 1) >> BRICK_BITS);
     add(0);
   }
   return cnt;
@@ -258,7 +315,8 @@ struct BatchInst {
   int pad;
   // moment pass: its second psi buffer and buffers, the cells next to a solid and their side buffer
   void *psi2, *nbuf;
-  const int* blist;
+  const int *blist, *events;
+  ChainState* cs;
   MomDev md;
   long long item0;  // first work item of this instance
 };
@@ -266,14 +324,13 @@ struct BatchInst {
 // Control block of the persistent kernel. queue[p]: next work item of phase p; arrive / gen: the
 // grid barrier between the phases (arrivals of this generation, generation count); spin_limit: the
 // longest a block waits at the barrier, in clock64 cycles, before it sets err bit 0 and returns.
-// The first 20 bytes (queues and arrivals) are cleared before every launch.
+// Queues and arrivals are cleared before every launch (k_batch_begin).
 struct BatchCtl {
   unsigned long long queue[2];
   unsigned arrive, gen;
   long long spin_limit;
   int err, pad;
 };
-constexpr size_t BATCH_CTL_RESET_BYTES = 2 * sizeof(unsigned long long) + sizeof(unsigned);
 constexpr int BATCH_TILE_CFGS = 4;  // tile shapes of the persistent kernel (see batch_tile)
 
 // Share of the GPU that the kernels launched by this host thread may assume (1 = all of it). The
@@ -305,14 +362,16 @@ extern thread_local int g_launch_share;
                        void* psi_b, const BodyDev* bodies, double* mass_part, StepState* st,         \
                        double* diag_rho, double* diag_vel, const PhysParams& pp, void* nbuf,         \
                        const int* blist, cudaStream_t s);                                             \
-  void launch_mom_enter(int prec, const Lat& lat, const void* fa, const void* fb, const StepState* st, \
+  void launch_mom_enter(int prec, const Lat& lat, void* fa, void* fb, const StepState* st, \
                         const uint16_t* flags, void* psi_a, void* psi_b, const MomDev& md,           \
                         const PhysParams& pp, cudaStream_t s);                                        \
   void launch_mom_fill(int prec, const Lat& lat, void* fa, void* fb, const StepState* st, const void* psi_a, \
-                       const void* psi_b, const MomDev& md, const PhysParams& pp, int next, cudaStream_t s); \
-  void launch_mom_close(int prec, const Lat& lat, const void* fa, const void* fb, StepState* st,     \
+                       const void* psi_b, const MomDev& md, ChainState* cs, const PhysParams& pp, int next,  \
+                       cudaStream_t s);                                                               \
+  void launch_mom_close(int prec, const Lat& lat, void* fa, void* fb, StepState* st,     \
                         const uint16_t* flags, void* psi_a, void* psi_b, const MomDev& md,           \
-                        const int* blist, const PhysParams& pp, int next, double* mass_part, cudaStream_t s); \
+                        const int* events, ChainState* cs, const int* blist, const PhysParams& pp, int next,  \
+                        double* mass_part, cudaStream_t s);                                           \
   int acc_sz(const Lat& lat, int prec, int ty, int waves);                                          \
   cudaError_t launch_lbm_acc(int prec, const Lat& lat, void* fa, void* fb, const uint16_t* flags,    \
                              void* psi_a, void* psi_b, void* rhop, const BodyDev* bodies,           \
@@ -329,9 +388,7 @@ extern thread_local int g_launch_share;
                             const StepState* st, const uint16_t* flags, const BodyDev* bodies, int nb, \
                             int max_tile, void* psi, void* psi_b, const PhysParams& pp,              \
                             cudaStream_t s);                                                         \
-  void launch_boundary(int prec, const Lat& lat, const void* fa, const void* fb, const uint16_t* flags, \
-                       const BodyDev* bodies, int nb, double* acc, const int* blist, const StepState* st, \
-                       const void* nbuf, double G, cudaStream_t s);                                   \
+  void launch_boundary(int prec, const ChainLaunch& c, cudaStream_t s);                               \
   void launch_read_populations(int prec, const Lat& lat, const void* fa, const void* fb,             \
                                const StepState* st, const uint16_t* flags, double* out, cudaStream_t s); \
   void launch_zero_solid(int prec, const Lat& lat, void* fa, void* fb, const StepState* st,          \
@@ -339,10 +396,12 @@ extern thread_local int g_launch_share;
                          cudaStream_t s);                                                             \
   void launch_init_fluid(int prec, const Lat& lat, void* fa, const uint16_t* flags, const double* rho, \
                          const double* u, cudaStream_t s);                                            \
-  void launch_refill(int prec, const Lat& lat, void* fa, void* fb, uint16_t* flags, const BodyDev* bodies, \
-                     int nb, int max_tile, StepState* st, int* blist, const double* arena,           \
-                     double member_thr, int* mbox, int next, cudaStream_t s);                        \
+  void launch_near_refill(int prec, const ChainLaunch& c, int next, cudaStream_t s);                  \
   void batch_tile(int cfg, int mom, int* t);                                                          \
+  void launch_batch_begin(const BatchInst* tab, int ninst, BatchCtl* ctl, int diag, cudaStream_t s);  \
+  void launch_batch_near(int prec, const BatchInst* tab, int ninst, cudaStream_t s);                 \
+  void launch_batch_fill(int prec, const BatchInst* tab, int ninst, cudaStream_t s);                 \
+  void launch_batch_close(int prec, const BatchInst* tab, int ninst, cudaStream_t s);                \
   int batch_mom_blocks_per_sm(int prec);                                                              \
   cudaError_t launch_batch_mom(int prec, const BatchInst* tab, int ninst, long long items, BatchCtl* ctl, \
                                int grid, int sz, int cooperative, cudaStream_t s);                   \
@@ -377,8 +436,12 @@ struct LbmOps {
   decltype(&q19::launch_read_populations) read_populations;
   decltype(&q19::launch_zero_solid) zero_solid;
   decltype(&q19::launch_init_fluid) init_fluid;
-  decltype(&q19::launch_refill) refill;
+  decltype(&q19::launch_near_refill) near_refill;
   decltype(&q19::batch_tile) batch_tile;
+  decltype(&q19::launch_batch_begin) batch_begin;
+  decltype(&q19::launch_batch_near) batch_near;
+  decltype(&q19::launch_batch_fill) batch_fill;
+  decltype(&q19::launch_batch_close) batch_close;
   decltype(&q19::batch_mom_blocks_per_sm) batch_mom_blocks_per_sm;
   decltype(&q19::launch_batch_mom) batch_mom;
   decltype(&q19::batch_blocks_per_sm) batch_blocks_per_sm;
@@ -390,8 +453,9 @@ inline LbmOps lbm_ops(int q) {
            &ns::launch_mom_enter, &ns::launch_mom_fill, &ns::launch_mom_close, &ns::acc_sz, &ns::launch_lbm_acc,   \
            &ns::launch_psi_fixup, &ns::fused_tz, &ns::launch_lbm_fused,                                             \
            &ns::launch_density_tiles, &ns::launch_boundary,                                                             \
-           &ns::launch_read_populations, &ns::launch_zero_solid, &ns::launch_init_fluid, &ns::launch_refill,        \
-           &ns::batch_tile, &ns::batch_mom_blocks_per_sm, &ns::launch_batch_mom, &ns::batch_blocks_per_sm, &ns::launch_batch_lbm }
+           &ns::launch_read_populations, &ns::launch_zero_solid, &ns::launch_init_fluid, &ns::launch_near_refill,        \
+           &ns::batch_tile, &ns::launch_batch_begin, &ns::launch_batch_near, &ns::launch_batch_fill, &ns::launch_batch_close,                     \
+           &ns::batch_mom_blocks_per_sm, &ns::launch_batch_mom, &ns::batch_blocks_per_sm, &ns::launch_batch_lbm }
   return q == 27 ? CBL_OPS(q27) : CBL_OPS(q19);
 #undef CBL_OPS
 }
@@ -399,24 +463,22 @@ inline LbmOps lbm_ops(int q) {
 void launch_clear_tile_flags(const Lat& lat, const BodyDev* bodies, int nb, int max_tile, uint16_t* flags,
                              cudaStream_t s);
 void launch_clear_stale(const Lat& lat, uint16_t* flags, cudaStream_t s);
+void launch_clear_cover(const Lat& lat, uint16_t* flags, cudaStream_t s);
 void launch_reset_member_boxes(int* mbox, int nb, cudaStream_t s);
 void launch_rasterize(const Lat& lat, BodyDev* bodies, int nb, int max_tile, double* arena,
                       double eta, cudaStream_t s);
 void launch_neighbour_lists(BodyDev* bodies, int nb, const Lat& lat, StepState* st, cudaStream_t s);
-void launch_flags(const Lat& lat, BodyDev* bodies, int nb, int max_tile, double* arena, uint16_t* flags,
-                  double threshold, int init, StepState* st, const MomDev& md, cudaStream_t s);
+void launch_flags(const ChainLaunch& c, int init, cudaStream_t s);
+void launch_commit(StepState* st, ChainState* cs, cudaStream_t s);
 void launch_body_props(const Lat& lat, BodyDev* bodies, int nb, int max_tile, double* arena,
                        double* scratch, cudaStream_t s);
-void launch_repulsion(const Lat& lat, const BodyDev* bodies, int nb, int max_tile, const double* arena, double* acc,
-                      const PhysParams& pp, const int* mbox, cudaStream_t s);
-void launch_bodies(const Lat& lat, BodyDev* bodies, int nb, double* acc, double* last, double* volacc,
-                   StepState* st, double* rtab, int Lmax, int* mbox, double* fsum, cudaStream_t s);
-void launch_finish(double* mass_part, unsigned n_mass_part, StepState* st, cudaStream_t s);
-void launch_advect(const Lat& lat, const BodyDev* bodies, int nb, int max_tile, double* arena, int mpf, double* volacc,
-                   StepState* st, const double* rtab, int Lmax, cudaStream_t s);
+void launch_repulsion(const ChainLaunch& c, cudaStream_t s);
+void launch_bodies(const ChainLaunch& c, cudaStream_t s);
+void launch_finish(double* mass_part, unsigned n_mass_part, StepState* st, ChainState* cs, cudaStream_t s);
+void launch_advect(const ChainLaunch& c, cudaStream_t s);
 void set_repulsion_offsets(double rc, double e0, int nrep, cudaStream_t s);
-void launch_kinetics(const Lat& lat, const BodyDev* bodies, int nb, int max_tile, double* arena,
-                     const double* volacc, const PhysParams& pp, cudaStream_t s);
+void launch_kinetics(const ChainLaunch& c, cudaStream_t s);
+KinParams kin_params(const PhysParams& pp);
 void launch_phi_dense(const Lat& lat, const BodyDev* bodies, int nb, int max_tile, const double* arena,
                       int body, double* out, cudaStream_t s);
 

@@ -32,7 +32,7 @@
 #include <cmath>
 #include <type_traits>
 #include "../../include/cbl.h"
-#include "cbl_dev.cuh"
+#include "tile.cuh"
 
 #ifndef CBL_Q
 #define CBL_Q 19
@@ -61,6 +61,7 @@ template <>
 struct St<double> {
   using R = double;
   __device__ static R ld(const double* p, size_t k, int) { return __ldg(p + k); }
+  __device__ static R ldv(const double* p, size_t k, int) { return p[k]; }
   __device__ static void st(double* p, size_t k, int, R v) { p[k] = v; }
   __device__ static R rt(R v, int) { return v; }
 };
@@ -296,18 +297,27 @@ __device__ __forceinline__ R mimg1(R d, int n) {
   return d;
 }
 
-// moving-wall term of solid link i at fluid cell c: g_i = 2 rho w_i c_i.u_B(x - c_i/2) / c_s^2
+// moving-wall term of solid link c_i = (cx, cy, cz), weight w, at fluid cell c: g_i = 2 rho w_i c_i.u_B(x - c_i/2) / c_s^2
 template <typename R>
-__device__ __forceinline__ R wall_term(const BodyDev& b, const Cell& c, const Lat& lat, int i, R rho) {
-  const R mx = (R)c.x - (R)0.5 * (R)cx_of(i), my = (R)c.y - (R)0.5 * (R)cy_of(i), mz = (R)c.z - (R)0.5 * (R)cz_of(i);
+__device__ __forceinline__ R wall_term_at(const BodyDev& b, const Cell& c, const Lat& lat, R cx, R cy, R cz, R w, R rho) {
+  const R mx = (R)c.x - (R)0.5 * cx, my = (R)c.y - (R)0.5 * cy, mz = (R)c.z - (R)0.5 * cz;
   const R ax = mimg1<R>(mx - par<R>(b.X[0], b.Xf[0]), lat.nx), ay = mimg1<R>(my - par<R>(b.X[1], b.Xf[1]), lat.ny),
           az = mimg1<R>(mz - par<R>(b.X[2], b.Xf[2]), lat.nz);
   const R wx = par<R>(b.W[0], b.Wf[0]), wy = par<R>(b.W[1], b.Wf[1]), wz = par<R>(b.W[2], b.Wf[2]);
   const R ux = par<R>(b.V[0], b.Vf[0]) + (wy * az - wz * ay);
   const R uy = par<R>(b.V[1], b.Vf[1]) + (wz * ax - wx * az);
   const R uz = par<R>(b.V[2], b.Vf[2]) + (wx * ay - wy * ax);
-  const R cu = (R)cx_of(i) * ux + (R)cy_of(i) * uy + (R)cz_of(i) * uz;
-  return (R)2 * rho * (R)w_of(i) * cu * (R)3;
+  const R cu = cx * ux + cy * uy + cz * uz;
+  return (R)2 * rho * w * cu * (R)3;
+}
+// w_i for a direction known only at run time (selected after the conversion)
+template <typename R>
+__device__ __forceinline__ R w_run(int i) {
+  return i <= 6 ? (R)w_of(1) : (i <= 18 ? (R)w_of(7) : (R)w_of(Q - 1));
+}
+template <typename R>
+__device__ __forceinline__ R wall_term(const BodyDev& b, const Cell& c, const Lat& lat, int i, R rho) {
+  return wall_term_at<R>(b, c, lat, (R)cx_of(i), (R)cy_of(i), (R)cz_of(i), (R)w_of(i), rho);
 }
 
 // Resident 128-thread blocks per SM requested for the bulk collision kernel: for FP32 occupancy
@@ -809,21 +819,6 @@ __global__ void __launch_bounds__(256) k_psi_fixup(const S* __restrict__ fa, con
   }
 }
 
-// the cell (gx, gy, gz) lies in the tile of a body with a lower id than `self` (so that a pass over
-// the tiles visits every cell once)
-__device__ __forceinline__ bool covered_by_lower(const BodyDev* bodies, const BodyDev& b, int self, int gx, int gy,
-                                                 int gz, const Lat& lat) {
-  for (int k = 0; k < b.nnb; ++k) {
-    int o = b.nbl[k];
-    if (o >= self) break;
-    const BodyDev& ob = bodies[o];
-    if (wrapi_near(gx - ob.o[0], lat.nx) < ob.L[0] && wrapi_near(gy - ob.o[1], lat.ny) < ob.L[1] &&
-        wrapi_near(gz - ob.o[2], lat.nz) < ob.L[2])
-      return true;
-  }
-  return false;
-}
-
 // ---- fused bulk pass: density, psi, Shan-Chen force and collision in one pass -----------------
 // The Shan-Chen force at x needs psi of the post-streaming density of this step at all neighbours
 // x + c_i (Eq. benzi_force), so every cell's populations are pulled twice per step: once for the
@@ -987,7 +982,7 @@ __global__ void __launch_bounds__(256) k_density_tiles(const S* __restrict__ fa,
   const unsigned r = u / L0;
   const int gx = wrapi_near(b.o[0] + (int)(u - r * L0), lat.nx), gy = wrapi_near(b.o[1] + (int)(r % L1), lat.ny),
             gz = wrapi_near(b.o[2] + (int)(r / L1), lat.nz);
-  if (b.nnb && covered_by_lower(bodies, b, self, gx, gy, gz, lat)) return;
+  if (b.nnb && covered_by_lower_body(bodies, b, self, gx, gy, gz, lat)) return;
   const Cell c = make_cell(gx, gy, gz, lat);
   psi[c.n] = psi_of_cell<S>(f, flags, bodies, lat, c, rho0, rho0_f);
 }
@@ -1146,133 +1141,198 @@ __global__ void __launch_bounds__(TX * TY, CollideMinBlocks<S>::value)
 }
 
 // ---- solid-fluid force on the bodies ---------------------------------------------------------
-// For each listed fluid cell x: for a solid upstream neighbour s = x - c_i (owner B), momentum
-// exchange -c_i (2 f*_opp(i)(x) + g_i) with the arm at the link midpoint (Eq. solid_liquid_force);
-// for a solid downstream neighbour x + c_i (owner B), the reaction of the Shan-Chen force,
-// +G psi(x) w_i psi(x + c_i) c_i, arm x + c_i - X_B (Sec. 3.2.3). It reads the same source
-// populations and psi as the collision, so g_i and rho are bit-identical to the ones it used.
-// One thread per (list cell, direction): ~18x the parallelism of a thread per cell, which matters
-// because the list is short (the fluid cells next to a solid) and each link's work is a chain of
-// dependent loads (flags -> population or body). The 12 sums per body (momentum exchange F, T;
-// adhesion F, T) are reduced in compensated precision over the warp and the block and added to the
-// FP64 accumulators once per block and body.
-template <typename S>
-__global__ void __launch_bounds__(256) k_boundary(const S* __restrict__ fa, const S* __restrict__ fb,
-                                                  const uint16_t* __restrict__ flags,
-                                                  const BodyDev* __restrict__ bodies, double* __restrict__ acc,
-                                                  const int* __restrict__ blist, const StepState* __restrict__ st,
-                                                  const RhoPsi<typename St<S>::R>* __restrict__ nbuf, Lat lat,
-                                                  double G, float G_f) {
+// For each listed fluid cell x and each solid neighbour s = x - c_i (owner B): momentum exchange
+// -c_i (2 f*_opp(i)(x) + g_i) with the arm at the link midpoint (Eq. solid_liquid_force), and the
+// reaction of the Shan-Chen force, +G psi(x) w_i psi(s) (s - x), arm s - X_B (Sec. 3.2.3). It reads the
+// same source populations and psi as the collision, so g_i and rho are bit-identical to the ones it
+// used. A block tests LINK_TEST (cell, direction) pairs, collects those whose neighbour is solid (about a
+// quarter) in shared memory and works on them in full warps. The 12 sums per body (momentum exchange
+// F, T; adhesion F, T) are reduced in compensated precision: over the warp by halves (each step sends
+// half of the sums and keeps the other, 13 additions instead of 60), over a round of the block, then one
+// FP64 atomic per sum and body. Four-sphere cluster (60 k cells): 65 us with one thread per pair and full
+// butterflies (547 instructions per 32 pairs), 14 us here.
+constexpr int LINK_T = 256, LINK_TEST = 2048;  // threads; most pairs per round
+
+// sum over the warp of 12 values per lane; lane 16 a + 8 b + 4 c + 2 d (+ 1) returns sum 6 a + 3 b + 2 c + d
+// (no sum where 2 c + d = 3)
+template <typename R>
+__device__ __forceinline__ LinkSum<R> warp_sum12(const R v[12], int lane) {
+  LinkSum<R> w6[6], w3[4], w2[2], w1;
+  {
+    const bool up = lane & 16;
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+      const R got = __shfl_xor_sync(0xffffffffu, up ? v[q] : v[q + 6], 16);
+      LinkSum<R> o;
+      w6[q].set(up ? v[q + 6] : v[q]);
+      o.set(got);
+      w6[q].add(o);
+    }
+  }
+  auto half = [&](const LinkSum<R>& a, const LinkSum<R>& b, int m) {  // keeps a below, b above
+    const bool up = lane & m;
+    LinkSum<R> keep = up ? b : a;
+    const LinkSum<R> send = up ? a : b;
+    keep.add(send.shfl_xor(m));
+    return keep;
+  };
+#pragma unroll
+  for (int q = 0; q < 3; ++q) w3[q] = half(w6[q], w6[q + 3], 8);
+  w3[3].set((R)0);
+#pragma unroll
+  for (int q = 0; q < 2; ++q) w2[q] = half(w3[q], w3[q + 2], 4);
+  w1 = half(w2[0], w2[1], 2);
+  w1.add(w1.shfl_xor(1));
+  return w1;
+}
+
+template <typename S, bool B>
+__global__ void __launch_bounds__(LINK_T) k_boundary(const __grid_constant__ TileSet one, const TileSet* __restrict__ sets) {
   using R = typename St<S>::R;
-  constexpr int NW = 8;  // warps per block
+  constexpr int NW = LINK_T / 32;
+  __shared__ unsigned list[LINK_TEST];
+  __shared__ int count;
   __shared__ LinkSum<R> part[NW][12];
   __shared__ int pown[NW];
-  const unsigned total = st->nbnd * (unsigned)(Q - 1);
-  const S* __restrict__ src = st->parity ? fb : fa;
+  __shared__ int dir[Q];  // c_i + 1, two bits a component (a direction known only at run time)
+  const TileSet& C = B ? sets[blockIdx.z] : one;
+  const Lat lat = C.lat;
+  const uint16_t* __restrict__ flags = C.flags;
+  const BodyDev* __restrict__ bodies = C.bodies;
+  const int* __restrict__ blist = C.blist;
+  const RhoPsi<R>* __restrict__ nbuf = (const RhoPsi<R>*)C.nbuf;
+  double* const acc = C.acc;
+  const unsigned total = C.st->nbnd * (unsigned)(Q - 1);
+  const S* __restrict__ src = (const S*)(C.st->parity ? C.fb : C.fa);
+  const R Gr = par<R>(C.G, C.G_f);
   const size_t N = (size_t)lat.Ns;  // population stride
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  // whole-block rounds so that every thread reaches the barriers
-  for (unsigned base = blockIdx.x * blockDim.x; base < total; base += gridDim.x * blockDim.x) {
-    const unsigned k = base + threadIdx.x;
-    R v[12];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  // the sum that this lane holds after warp_sum12
+  const int sub = ((lane >> 2) & 1) * 2 + ((lane >> 1) & 1), slot = (lane >> 4) * 6 + ((lane >> 3) & 1) * 3 + sub;
+  const bool holds = sub < 3 && !(lane & 1);
+  if (tid == 0) {
 #pragma unroll
-    for (int q = 0; q < 12; ++q) v[q] = 0;
-    int Bm = -1, Ba = -1;  // body of the momentum-exchange term, of the adhesion term
-    if (k < total) {
-      const unsigned cell = k / (unsigned)(Q - 1);
-      const int i = 1 + (int)(k - cell * (unsigned)(Q - 1));
-      const long long n = blist[cell];
-      const Cell c = cell_of(n, lat);
-      const uint16_t up = __ldg(flags + nbr(c, lat, i, -1)), dn = __ldg(flags + nbr(c, lat, i, +1));
-      if (up & F_SOLID) {
-        // link to a solid upstream: the pulled value is f*_opp(i)(x) (half-way bounce-back)
-        const int B = up & F_OWNER;
-        const BodyDev& b = bodies[B];
-        const RhoPsi<R> rp = nbuf[n];
-        const R fi = St<S>::ld(src, (size_t)opp_of(i) * N + n, i);
-        const R g = wall_term<R>(b, c, lat, i, rp.rho);
-        const R m2 = (R)2 * fi + g;
-        const R dPx = -(R)cx_of(i) * m2, dPy = -(R)cy_of(i) * m2, dPz = -(R)cz_of(i) * m2;
-        const R ax = mimg1<R>((R)c.x - (R)0.5 * (R)cx_of(i) - par<R>(b.X[0], b.Xf[0]), lat.nx);
-        const R ay = mimg1<R>((R)c.y - (R)0.5 * (R)cy_of(i) - par<R>(b.X[1], b.Xf[1]), lat.ny);
-        const R az = mimg1<R>((R)c.z - (R)0.5 * (R)cz_of(i) - par<R>(b.X[2], b.Xf[2]), lat.nz);
-        v[0] = dPx;
-        v[1] = dPy;
-        v[2] = dPz;
-        v[3] = ay * dPz - az * dPy;
-        v[4] = az * dPx - ax * dPz;
-        v[5] = ax * dPy - ay * dPx;
-        Bm = B;
-      }
-      if (dn & F_SOLID) {
-        // solid downstream: reaction of the Shan-Chen force on that body
-        const int B = dn & F_OWNER;
-        const BodyDev& b = bodies[B];
-        const R ps = nbuf[n].psi;
-        const R gpw = par<R>(G, G_f) * ps * ((R)w_of(i) * par<R>(b.psi_wet, b.psi_wet_f));
-        const R fx = gpw * (R)cx_of(i), fy = gpw * (R)cy_of(i), fz = gpw * (R)cz_of(i);
-        const R ax = mimg1<R>((R)c.x + (R)cx_of(i) - par<R>(b.X[0], b.Xf[0]), lat.nx);
-        const R ay = mimg1<R>((R)c.y + (R)cy_of(i) - par<R>(b.X[1], b.Xf[1]), lat.ny);
-        const R az = mimg1<R>((R)c.z + (R)cz_of(i) - par<R>(b.X[2], b.Xf[2]), lat.nz);
-        v[6] = fx;
-        v[7] = fy;
-        v[8] = fz;
-        v[9] = ay * fz - az * fy;
-        v[10] = az * fx - ax * fz;
-        v[11] = ax * fy - ay * fx;
-        Ba = B;
-      }
-    }
-    // one body for the whole warp (the usual case): compensated warp sums; otherwise per-lane
-    // FP64 atomics
-    const int Bt = Bm >= 0 ? Bm : Ba;
-    const bool mixed = Bm >= 0 && Ba >= 0 && Bm != Ba;
-    const unsigned any = __ballot_sync(0xffffffffu, Bt >= 0);
-    int b0 = -1;
-    if (any) {
-      b0 = __shfl_sync(0xffffffffu, Bt, __ffs(any) - 1);
-      if (!__all_sync(0xffffffffu, (Bt < 0 || Bt == b0) && !mixed)) {
-#pragma unroll
-        for (int q = 0; q < 12; ++q) {
-          const int B = q < 6 ? Bm : Ba;
-          if (B >= 0 && v[q] != (R)0) atomicAdd(acc + (size_t)B * ACC_N + q, (double)v[q]);
-        }
-        b0 = -1;
-      } else {
-#pragma unroll
-        for (int q = 0; q < 12; ++q) {
-          LinkSum<R> a;
-          a.set(v[q]);
-#pragma unroll
-          for (int m = 16; m > 0; m >>= 1) a.add(a.shfl_xor(m));
-          if (lane == 0) part[w][q] = a;
-        }
-      }
-    }
-    if (lane == 0) pown[w] = b0;
+    for (int i = 0; i < Q; ++i) dir[i] = (cx_of(i) + 1) | (cy_of(i) + 1) << 2 | (cz_of(i) + 1) << 4;
+  }
+  auto upstream = [&](const Cell& c, int d) {
+    const int dx = (d & 3) - 1, dy = (d >> 2 & 3) - 1, dz = (d >> 4) - 1;
+    return c.n + (unsigned)((dx > 0 ? c.ox[0] : (dx < 0 ? c.ox[2] : 0)) + (dy > 0 ? c.oy[0] : (dy < 0 ? c.oy[2] : 0)) +
+                            (dz > 0 ? c.oz[0] : (dz < 0 ? c.oz[2] : 0)));
+  };
+  // pairs per round: all blocks take part where the list is short
+  const unsigned round = min((unsigned)LINK_TEST, max(1u, (total / gridDim.x + LINK_T) / LINK_T) * LINK_T);
+  for (unsigned base = blockIdx.x * round; base < total; base += gridDim.x * round) {
+    if (tid == 0) count = 0;
     __syncthreads();
-    if (threadIdx.x < 12) {
-      // warps of the same body in a row are combined before one FP64 atomic
-      const int q = threadIdx.x;
-      int cur = -1;
-      LinkSum<R> run;
-      run.set((R)0);
-      for (int ww = 0; ww < NW; ++ww) {
-        const int B = pown[ww];
-        if (B < 0) continue;
-        if (B != cur) {
-          if (cur >= 0) {
-            const double x = run.value();
-            if (x != 0.0) atomicAdd(acc + (size_t)cur * ACC_N + q, x);
-          }
-          cur = B;
-          run.set((R)0);
-        }
-        run.add(part[ww][q]);
+#pragma unroll 2
+    for (unsigned j = 0; j < round; j += LINK_T) {
+      const unsigned k = base + j + tid;
+      bool hit = false;
+      if (k < total) {
+        const unsigned cell = k / (unsigned)(Q - 1);
+        const int i = 1 + (int)(k - cell * (unsigned)(Q - 1));
+        const Cell c = cell_of(blist[cell], lat);
+        hit = __ldg(flags + upstream(c, dir[i])) & F_SOLID;
       }
-      if (cur >= 0) {
-        const double x = run.value();
-        if (x != 0.0) atomicAdd(acc + (size_t)cur * ACC_N + q, x);
+      const unsigned m = __ballot_sync(0xffffffffu, hit);
+      if (m) {
+        int at = 0;
+        if (lane == 0) at = atomicAdd(&count, __popc(m));
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if (hit) list[at + __popc(m & ((1u << lane) - 1u))] = k;
+      }
+    }
+    __syncthreads();
+    const int n_links = count;
+    int cur = -1;  // body of the warp's running sums
+    LinkSum<R> run;
+    run.set((R)0);
+    for (int e0 = w * 32; e0 < n_links; e0 += LINK_T) {
+      const int e = e0 + lane;
+      R v[12];
+#pragma unroll
+      for (int q = 0; q < 12; ++q) v[q] = 0;
+      int body = -1;
+      if (e < n_links) {
+        const unsigned k = list[e], cell = k / (unsigned)(Q - 1);
+        const int i = 1 + (int)(k - cell * (unsigned)(Q - 1));
+        const long long n = blist[cell];
+        const Cell c = cell_of(n, lat);
+        const int d = dir[i];
+        body = __ldg(flags + upstream(c, d)) & F_OWNER;
+        const BodyDev& b = bodies[body];
+        const RhoPsi<R> rp = nbuf[n];
+        const R cx = (R)((d & 3) - 1), cy = (R)((d >> 2 & 3) - 1), cz = (R)((d >> 4) - 1);
+        {
+          // the pulled value of a link to a solid is f*_opp(i)(x) (half-way bounce-back)
+          const R fi = St<S>::ld(src, (size_t)opp_of(i) * N + n, i);
+          const R g = wall_term_at<R>(b, c, lat, cx, cy, cz, w_run<R>(i), rp.rho);
+          const R m2 = (R)2 * fi + g;
+          const R ax = mimg1<R>((R)c.x - (R)0.5 * cx - par<R>(b.X[0], b.Xf[0]), lat.nx);
+          const R ay = mimg1<R>((R)c.y - (R)0.5 * cy - par<R>(b.X[1], b.Xf[1]), lat.ny);
+          const R az = mimg1<R>((R)c.z - (R)0.5 * cz - par<R>(b.X[2], b.Xf[2]), lat.nz);
+          v[0] = -cx * m2;
+          v[1] = -cy * m2;
+          v[2] = -cz * m2;
+          v[3] = ay * v[2] - az * v[1];
+          v[4] = az * v[0] - ax * v[2];
+          v[5] = ax * v[1] - ay * v[0];
+        }
+        {
+          const R gpw = Gr * rp.psi * (w_run<R>(i) * par<R>(b.psi_wet, b.psi_wet_f));
+          const R ax = mimg1<R>((R)c.x - cx - par<R>(b.X[0], b.Xf[0]), lat.nx);
+          const R ay = mimg1<R>((R)c.y - cy - par<R>(b.X[1], b.Xf[1]), lat.ny);
+          const R az = mimg1<R>((R)c.z - cz - par<R>(b.X[2], b.Xf[2]), lat.nz);
+          v[6] = gpw * -cx;
+          v[7] = gpw * -cy;
+          v[8] = gpw * -cz;
+          v[9] = ay * v[8] - az * v[7];
+          v[10] = az * v[6] - ax * v[8];
+          v[11] = ax * v[7] - ay * v[6];
+        }
+      }
+      // one body for the whole warp in the usual case, else body by body
+      unsigned todo = __ballot_sync(0xffffffffu, body >= 0);
+      while (todo) {
+        const int b0 = __shfl_sync(0xffffffffu, body, __ffs(todo) - 1);
+        const unsigned mine = __ballot_sync(0xffffffffu, body == b0);
+        R u[12];
+#pragma unroll
+        for (int q = 0; q < 12; ++q) u[q] = body == b0 ? v[q] : (R)0;
+        const LinkSum<R> t = warp_sum12<R>(u, lane);
+        if (b0 != cur) {
+          if (cur >= 0 && holds) {
+            const double x = run.value();
+            if (x != 0.0) atomicAdd(acc + (size_t)cur * ACC_N + slot, x);
+          }
+          cur = b0;
+          run = t;
+        } else {
+          run.add(t);
+        }
+        todo &= ~mine;
+      }
+    }
+    if (holds) part[w][slot] = run;
+    if (lane == 0) pown[w] = cur;
+    __syncthreads();
+    if (tid < 12) {
+      // warps of the same body in a row are combined before one FP64 atomic
+      int at = -1;
+      LinkSum<R> sum;
+      sum.set((R)0);
+      for (int ww = 0; ww <= NW; ++ww) {
+        const int o = ww < NW ? pown[ww] : -2;
+        if (o == -1) continue;
+        if (o != at) {
+          if (at >= 0) {
+            const double x = sum.value();
+            if (x != 0.0) atomicAdd(acc + (size_t)at * ACC_N + tid, x);
+          }
+          at = o;
+          sum.set((R)0);
+        }
+        if (ww < NW) sum.add(part[ww][tid]);
       }
     }
     __syncthreads();
@@ -1309,178 +1369,218 @@ __global__ void k_init_fluid(S* __restrict__ f, const uint16_t* __restrict__ fla
 
 
 // ---- cover refill and boundary list ------------------------------------------------------------
-// Over the body tiles (each cell once: the lowest-id tile that covers it), after the new flags.
-// A fluid cell with a solid neighbour along a lattice direction goes into the boundary list of the
-// next step. If any node was covered in this step, a fluid cell next to a covered node n receives
-// f_eq(rho_n, u_n) / |N_F(n)| (face neighbours; all 26 if n has no fluid face neighbour).
+// After the new flags. Over the bodies' tiles: the fluid neighbours of a body's solid cells along a lattice
+// direction are the cells next to a solid; whoever sets a cell's bit first puts it into the boundary
+// list of the next step (collected per block, so that the list's runs belong to one body). Outside a step
+// (next = 0) the pass also makes the bodies' member records (k_flags does in a step, where X is final before
+// it). Over this step's flag changes: a covered
+// node n hands f_eq(rho_n, u_n) / |N_F(n)| to its fluid neighbours (face neighbours; all 26 if n has no
+// fluid face neighbour), gathered by the receivers, each by the first of its covered neighbours, so that
+// no two threads write the same populations. The blocks share the changes out over the whole launch.
+// Only cells with phi > 0 are looked at (a third of a sphere's tile), and only the solid ones' neighbours;
+// testing the 18 neighbours of every fluid tile cell took 40 us on the four-sphere cluster, this 25.
+constexpr int NEAR_CAP = 2048;
+
+// the covered cells' share of k_near_refill (rare: in most steps no flag changes)
 template <typename S>
-__global__ void __launch_bounds__(256) k_refill(S* __restrict__ fa, S* __restrict__ fb,
-                                                uint16_t* __restrict__ flags,
-                                                const BodyDev* __restrict__ bodies, StepState* st, int* blist,
-                                                Lat lat, const double* __restrict__ arena, double member_thr,
-                                                int* __restrict__ mbox, int next) {
+__device__ __noinline__ void refill_covered(const TileSet& C, int self, int next) {
   using R = typename St<S>::R;
+  const Lat& lat = C.lat;
+  const uint16_t* const flags = C.flags;
   // the current state: the buffer this step's collision wrote (next = 1: the parity flips at the end
   // of the step) or, outside a step, the buffer the parity names
-  S* __restrict__ f = (st->parity ^ next) ? fb : fa;
-  const int self = blockIdx.y;
-  const BodyDev& b = bodies[self];
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  bool boundary = false;
-  long long m = 0;
-  // member cells (phi >= member_thr) of this body: their tile-coordinate bounding box, for the
-  // repulsion pass of the next step
-  bool member = false;
-  int mi[3] = {0, 0, 0};
-  float r2 = 0.0f;  // squared distance of a member cell from the body's centre
-  if (t < b.sz) {
-    const unsigned u = (unsigned)t, L0 = (unsigned)b.L[0], L1 = (unsigned)b.L[1];  // tiles hold < 2^31 cells
-    const unsigned r = u / L0;
-    const int i0 = (int)(u - r * L0), i1 = (int)(r % L1), i2 = (int)(r / L1);
-    member = dbits(arena[b.off + t]) >= dbits(member_thr);
-    mi[0] = i0;
-    mi[1] = i1;
-    mi[2] = i2;
-    const int gx = wrapi_near(b.o[0] + i0, lat.nx), gy = wrapi_near(b.o[1] + i1, lat.ny),
-              gz = wrapi_near(b.o[2] + i2, lat.nz);
-    m = gx + (long long)lat.nx * (gy + (long long)lat.ny * gz);
-    if (member) {
-      // in float from the float mirror of X (FP64 is 1/64 rate here and this is a bound with slack);
-      // tile cells lie within half a lattice length of X along each axis, so one wrap suffices
-      const float dx = mimg1<float>((float)gx - b.Xf[0], lat.nx), dy = mimg1<float>((float)gy - b.Xf[1], lat.ny),
-                  dz = mimg1<float>((float)gz - b.Xf[2], lat.nz);
-      r2 = dx * dx + dy * dy + dz * dz;
+  S* const f = (S*)((C.st->parity ^ next) ? C.fb : C.fa);
+  const size_t N = (size_t)lat.Ns;  // population stride
+  auto fluid_count = [&](const Cell& c, bool faces_only) {
+    int cnt = 0;
+    for (int o = 0; o < 27; ++o) {
+      const int dx = o % 3 - 1, dy = (o / 3) % 3 - 1, dz = o / 9 - 1, d2 = dx * dx + dy * dy + dz * dz;
+      if (d2 == 0 || (faces_only && d2 > 1)) continue;
+      if (!(flags[c.n + (unsigned)(c.ox[dx + 1] + c.oy[dy + 1] + c.oz[dz + 1])] & F_SOLID)) cnt++;
     }
-    if (!(b.nnb && covered_by_lower(bodies, b, self, gx, gy, gz, lat))) {
-      const Cell c = cell_of(m, lat);
-      const uint16_t fm = flags[m];
-      const bool events = st->ncover != 0;
-      const size_t N = (size_t)lat.Ns;  // population stride
-      auto at = [&](int x, int y, int z) {
-        return (long long)wrapi_near(x, lat.nx) +
-               (long long)lat.nx * (wrapi_near(y, lat.ny) + (long long)lat.ny * wrapi_near(z, lat.nz));
-      };
-      auto fluid_count = [&](int x, int y, int z, bool faces_only) {
-        int cnt = 0;
-        for (int dz = -1; dz <= 1; ++dz)
-          for (int dy = -1; dy <= 1; ++dy)
-            for (int dx = -1; dx <= 1; ++dx) {
-              int d2 = dx * dx + dy * dy + dz * dz;
-              if (d2 == 0 || (faces_only && d2 > 1)) continue;
-              if (!(flags[at(x + dx, y + dy, z + dz)] & F_SOLID)) cnt++;
-            }
-        return cnt;
-      };
-      if (fm & F_SOLID) {
-        // a covered node with no fluid node within sqrt(3) loses its mass: count it
-        if ((fm & F_COVER) && fluid_count(gx, gy, gz, false) == 0) {
-          atomicAdd(&st->lost_refills, 1ull);
-          atomicOr(&st->err, E_REFILL);
-        }
+    return cnt;
+  };
+  const unsigned total = 27u * C.cs->nevent, per = gridDim.x * gridDim.y * TILE_T;
+  for (unsigned k = ((unsigned)self * gridDim.y + blockIdx.y) * gridDim.x * TILE_T + blockIdx.x * TILE_T + threadIdx.x;
+       k < total; k += per * (unsigned)C.nb) {
+    const unsigned ev = k / 27u;
+    const int o = (int)(k - 27u * ev);
+    const Cell c = cell_of(C.events[ev], lat);
+    if (!(flags[c.n] & F_COVER)) continue;
+    if (o == 13) {
+      // a covered node with no fluid node within sqrt(3) loses its mass: count it
+      if (fluid_count(c, false) == 0) {
+        atomicAdd(&C.st->lost_refills, 1ull);
+        atomicOr(&C.st->err, E_REFILL);
+      }
+      continue;
+    }
+    // the receiver, and whether this node is the first of its covered neighbours
+    const Cell m = cell_of(c.n + (unsigned)(c.ox[o % 3] + c.oy[(o / 3) % 3] + c.oz[o / 9]), lat);
+    if (flags[m.n] & F_SOLID) continue;
+    bool mine = true, give = false;
+    R add[Q];
+#pragma unroll
+    for (int i = 0; i < Q; ++i) add[i] = 0;
+    for (int q = 0; q < 27; ++q) {
+      const int dx = q % 3 - 1, dy = (q / 3) % 3 - 1, dz = q / 9 - 1, d2 = dx * dx + dy * dy + dz * dz;
+      if (d2 == 0) continue;
+      const unsigned nn = m.n + (unsigned)(m.ox[dx + 1] + m.oy[dy + 1] + m.oz[dz + 1]);
+      if (!(flags[nn] & F_COVER)) continue;
+      if (!give && nn != c.n) {
+        mine = false;
+        break;
+      }
+      give = true;
+      const Cell g = cell_of(nn, lat);
+      const int c6 = fluid_count(g, true);
+      int cnt;
+      if (c6 > 0) {
+        if (d2 != 1) continue;  // only face neighbours share this node's populations
+        cnt = c6;
       } else {
+        cnt = fluid_count(g, false);
+      }
+      R fi[Q];
+      R rho = 0, mx = 0, my = 0, mz = 0;
 #pragma unroll
-        for (int i = 1; i < Q; ++i) boundary |= (__ldg(flags + nbr(c, lat, i, +1)) & F_SOLID) != 0;
-        // this thread is the only writer of the cell's flag word in this pass; concurrent readers
-        // only test the solid bit, which this store does not change
-        if (boundary != ((fm & F_NEAR) != 0)) flags[m] = boundary ? (uint16_t)(fm | F_NEAR) : (uint16_t)(fm & ~F_NEAR);
-        if (events) {
-          bool any = false;
-          for (int dz = -1; dz <= 1 && !any; ++dz)
-            for (int dy = -1; dy <= 1 && !any; ++dy)
-              for (int dx = -1; dx <= 1 && !any; ++dx)
-                if ((dx | dy | dz) && (flags[c.n + (unsigned)(c.ox[dx + 1] + c.oy[dy + 1] + c.oz[dz + 1])] & F_COVER))
-                  any = true;
-          if (any) {
-            R add[Q];
+      for (int i = 0; i < Q; ++i) {
+        fi[i] = St<S>::ld(f, (size_t)i * N + nn, i);
+        rho += fi[i];
+        mx += (R)cx_of(i) * fi[i];
+        my += (R)cy_of(i) * fi[i];
+        mz += (R)cz_of(i) * fi[i];
+      }
+      R ux = 0, uy = 0, uz = 0;
+      if (rho > (R)0) {
+        ux = mx / rho;
+        uy = my / rho;
+        uz = mz / rho;
+      }
+      const R uu = ux * ux + uy * uy + uz * uz;
+      const R inv = (R)1 / (R)cnt;
 #pragma unroll
-            for (int i = 0; i < Q; ++i) add[i] = 0;
-            for (int dz = -1; dz <= 1; ++dz)
-              for (int dy = -1; dy <= 1; ++dy)
-                for (int dx = -1; dx <= 1; ++dx) {
-                  const int d2 = dx * dx + dy * dy + dz * dz;
-                  if (d2 == 0) continue;
-                  const int nxp = gx + dx, nyp = gy + dy, nzp = gz + dz;
-                  const long long nn = c.n + (unsigned)(c.ox[dx + 1] + c.oy[dy + 1] + c.oz[dz + 1]);
-                  if (!(flags[nn] & F_COVER)) continue;
-                  const int c6 = fluid_count(nxp, nyp, nzp, true);
-                  int cnt;
-                  if (c6 > 0) {
-                    if (d2 != 1) continue;  // only face neighbours share this node's populations
-                    cnt = c6;
-                  } else {
-                    cnt = fluid_count(nxp, nyp, nzp, false);
-                  }
-                  R fi[Q];
-                  R rho = 0, mx = 0, my = 0, mz = 0;
-#pragma unroll
-                  for (int i = 0; i < Q; ++i) {
-                    fi[i] = St<S>::ld(f, (size_t)i * N + nn, i);
-                    rho += fi[i];
-                    mx += (R)cx_of(i) * fi[i];
-                    my += (R)cy_of(i) * fi[i];
-                    mz += (R)cz_of(i) * fi[i];
-                  }
-                  R ux = 0, uy = 0, uz = 0;
-                  if (rho > (R)0) {
-                    ux = mx / rho;
-                    uy = my / rho;
-                    uz = mz / rho;
-                  }
-                  const R uu = ux * ux + uy * uy + uz * uz;
-                  const R inv = (R)1 / (R)cnt;
-#pragma unroll
-                  for (int i = 0; i < Q; ++i) {
-                    const R cu = (R)cx_of(i) * ux + (R)cy_of(i) * uy + (R)cz_of(i) * uz;
-                    add[i] += rho * wgt<R>(i) * ((R)1 + (R)3 * cu + (R)4.5 * cu * cu - (R)1.5 * uu) * inv;
-                  }
-                }
-#pragma unroll
-            for (int i = 0; i < Q; ++i) {
-              const size_t k = (size_t)i * N + m;
-              St<S>::st(f, k, i, St<S>::ld(f, k, i) + add[i]);
-            }
-          }
-        }
+      for (int i = 0; i < Q; ++i) {
+        const R cu = (R)cx_of(i) * ux + (R)cy_of(i) * uy + (R)cz_of(i) * uz;
+        add[i] += rho * wgt<R>(i) * ((R)1 + (R)3 * cu + (R)4.5 * cu * cu - (R)1.5 * uu) * inv;
       }
     }
-  }
-  // warp, then block, then one set of global atomics per block (all warps of a block hit the same
-  // six words, so per-warp global atomics would queue up)
-  __shared__ int sbox[7];
-  if (threadIdx.x < 7) sbox[threadIdx.x] = threadIdx.x < 3 ? INT_MAX : (threadIdx.x < 6 ? INT_MIN : 0);
-  __syncthreads();
-  if (__ballot_sync(0xffffffffu, member)) {
-    const int lane = threadIdx.x & 31;
+    if (!mine) continue;
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      const int lo = __reduce_min_sync(0xffffffffu, member ? mi[a] : INT_MAX);
-      const int hi = __reduce_max_sync(0xffffffffu, member ? mi[a] : INT_MIN);
-      if (lane == 0) {
-        atomicMin(sbox + a, lo);
-        atomicMax(sbox + 3 + a, hi);
-      }
+    for (int i = 0; i < Q; ++i) {
+      const size_t at = (size_t)i * N + m.n;
+      St<S>::st(f, at, i, St<S>::ldv(f, at, i) + add[i]);
     }
-    // non-negative floats order like their bit patterns
-    const unsigned rb = __reduce_max_sync(0xffffffffu, member ? __float_as_uint(r2) : 0u);
-    if (lane == 0) atomicMax(sbox + 6, (int)rb);
-  }
-  __syncthreads();
-  if (threadIdx.x < 7 && sbox[0] <= sbox[3]) {
-    if (threadIdx.x < 3) atomicMin(mbox + MBOX_N * self + threadIdx.x, sbox[threadIdx.x]);
-    else atomicMax(mbox + MBOX_N * self + threadIdx.x, sbox[threadIdx.x]);
-  }
-  // warp-aggregated append to the boundary list
-  const unsigned mask = __ballot_sync(0xffffffffu, boundary);
-  if (mask) {
-    const int lane = threadIdx.x & 31;
-    const int leader = __ffs(mask) - 1;
-    unsigned base = 0;
-    if (lane == leader) base = atomicAdd(&st->nbnd, (unsigned)__popc(mask));
-    base = __shfl_sync(0xffffffffu, base, leader);
-    if (boundary) blist[base + __popc(mask & ((1u << lane) - 1))] = (int)m;
   }
 }
 
+template <typename S, bool B, int Z>
+__global__ void __launch_bounds__(TILE_T) k_near_refill(const __grid_constant__ TileSet one,
+                                                        const TileSet* __restrict__ sets, const int2* __restrict__ items,
+                                                        int next) {
+  int self;
+  const TileSet& C = tile_set<B>(one, sets, items, self);
+  const Lat& lat = C.lat;
+  uint16_t* const flags = C.flags;
+  unsigned* const words = reinterpret_cast<unsigned*>(flags);
+  __shared__ TileList list;
+  __shared__ int near[NEAR_CAP];
+  __shared__ int n_near, base_near, sbox[7];
+  if (threadIdx.x == 0) list.n = n_near = 0;
+  if (threadIdx.x < 7) sbox[threadIdx.x] = threadIdx.x < 3 ? INT_MAX : (threadIdx.x < 6 ? INT_MIN : 0);
+  __syncthreads();
+  const BodyDev& b = C.bodies[self];
+  const int L0 = b.L[0], L1 = b.L[1], L2 = b.L[2], z0 = blockIdx.y * Z;
+  const unsigned plane = (unsigned)L0 * L1, p0 = blockIdx.x * TILE_T, p = p0 + threadIdx.x;
+  if (z0 < L2 && p0 < plane) {
+    const int i1 = (int)(p / (unsigned)L0), i0 = (int)(p - (unsigned)i1 * L0);
+    const double* const phi = C.arena + b.off;
+    const long long thr = dbits(C.member_thr);
+    bool any = false;
+    int lz = INT_MAX, hz = INT_MIN;
+    float r2 = 0.0f;
+#pragma unroll
+    for (int q = 0; q < Z; ++q) {
+      const bool in = p < plane && z0 + q < L2;
+      const long long vb = in ? dbits(phi[p + (size_t)plane * (z0 + q)]) : 0;
+      bool solid = false;
+      const bool member = !next && in && vb >= thr;
+      if (vb > 0 || member) {
+        const TileCell c = tile_at(b, i0, i1, z0 + q, lat);
+        const uint16_t fl = flags[lat_index(c, lat)];
+        solid = (fl & F_SOLID) && (fl & F_OWNER) == self;
+        if (member) {
+          // in float from the float mirror of X (FP64 is 1/64 rate here and this is a bound with slack);
+          // tile cells lie within half a lattice length of X along each axis, so one wrap suffices
+          const float dx = mimg1<float>((float)c.gx - b.Xf[0], lat.nx), dy = mimg1<float>((float)c.gy - b.Xf[1], lat.ny),
+                      dz = mimg1<float>((float)c.gz - b.Xf[2], lat.nz);
+          r2 = fmaxf(r2, dx * dx + dy * dy + dz * dz);
+          any = true;
+          lz = min(lz, z0 + q);
+          hz = max(hz, z0 + q);
+        }
+      }
+      tile_append(list, solid, q * TILE_T + threadIdx.x);
+    }
+    // warp, then block, then one set of global atomics per block (all blocks of a body hit the same words)
+    if (__any_sync(0xffffffffu, any)) {
+      const int lo[3] = {any ? i0 : INT_MAX, any ? i1 : INT_MAX, lz}, hi[3] = {any ? i0 : INT_MIN, any ? i1 : INT_MIN, hz};
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        const int l = __reduce_min_sync(0xffffffffu, lo[a]), h = __reduce_max_sync(0xffffffffu, hi[a]);
+        if ((threadIdx.x & 31) == 0) {
+          atomicMin(sbox + a, l);
+          atomicMax(sbox + 3 + a, h);
+        }
+      }
+      // non-negative floats order like their bit patterns
+      const unsigned rb = __reduce_max_sync(0xffffffffu, __float_as_uint(r2));
+      if ((threadIdx.x & 31) == 0) atomicMax(sbox + 6, (int)rb);
+    }
+    __syncthreads();
+    if (threadIdx.x < 7 && sbox[0] <= sbox[3]) {
+      if (threadIdx.x < 3) atomicMin(C.mbox + MBOX_N * self + threadIdx.x, sbox[threadIdx.x]);
+      else atomicMax(C.mbox + MBOX_N * self + threadIdx.x, sbox[threadIdx.x]);
+    }
+    for (int e = threadIdx.x; e < list.n; e += TILE_T) {
+      const int id = list.id[e];
+      const unsigned pc = p0 + (id & (TILE_T - 1));
+      const int c1 = (int)(pc / (unsigned)L0), c0 = (int)(pc - (unsigned)c1 * L0);
+      const TileCell t = tile_at(b, c0, c1, z0 + id / TILE_T, lat);
+      const Cell c = make_cell(t.gx, t.gy, t.gz, lat);
+      uint16_t fl[Q];
+#pragma unroll
+      for (int i = 1; i < Q; ++i) fl[i] = flags[nbr(c, lat, i, +1)];
+#pragma unroll
+      for (int i = 1; i < Q; ++i) {
+        if (fl[i] & (F_SOLID | F_NEAR)) continue;
+        const unsigned n = (unsigned)nbr(c, lat, i, +1), bit = (unsigned)F_NEAR << ((n & 1u) * 16u);
+        if (atomicOr(words + (n >> 1), bit) & bit) continue;
+        const int at = atomicAdd(&n_near, 1);
+        if (at < NEAR_CAP) near[at] = (int)n;
+        else C.blist[atomicAdd(&C.cs->nnew, 1u)] = (int)n;
+      }
+    }
+    __syncthreads();
+    const int cnt = min(n_near, NEAR_CAP);
+    if (threadIdx.x == 0 && cnt) base_near = (int)atomicAdd(&C.cs->nnew, (unsigned)cnt);
+    __syncthreads();
+    for (int k = threadIdx.x; k < cnt; k += TILE_T) C.blist[base_near + k] = near[k];
+  }
+  if (C.st->ncover != 0) refill_covered<S>(C, self, next);
+  if (!next || C.mom) return;
+  // without the moment pass this is the step's last kernel: the last of the context's blocks ends it
+  __shared__ int s_last;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    s_last = atomicAdd(&C.cs->done, 1u) == gridDim.x * gridDim.y * (unsigned)C.nb - 1u;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  if (threadIdx.x == 0) C.cs->done = 0;
+  finish_step<TILE_T>(C.mass_part, MASS_SLOTS, C.st, C.cs);
+}
 // current populations, widened to double, [direction][cell]; solid cells read zero (a node covered
 // in the last step keeps its stale populations until the next collision overwrites them)
 template <typename S>
@@ -1705,42 +1805,43 @@ void launch_mom_near(int prec, const Lat& lat, void* fa, void* fb, const uint16_
   else mom_near_t<__half>(lat, fa, fb, flags, psi_a, psi_b, bodies, mass_part, st, diag_rho, diag_vel, pp, nbuf, blist, s);
 }
 
-void launch_mom_enter(int prec, const Lat& lat, const void* fa, const void* fb, const StepState* st,
+void launch_mom_enter(int prec, const Lat& lat, void* fa, void* fb, const StepState* st,
                       const uint16_t* flags, void* psi_a, void* psi_b, const MomDev& md, const PhysParams& pp,
                       cudaStream_t s) {
   const dim3 grid((lat.nx + 31) / 32, (lat.ny + 3) / 4, lat.nz);
   if (prec == 1)
-    k_mom_enter<float><<<grid, 128, 0, s>>>((const float*)fa, (const float*)fb, st, flags, (float*)psi_a, (float*)psi_b,
+    k_mom_enter<float><<<grid, 128, 0, s>>>((float*)fa, (float*)fb, st, flags, (float*)psi_a, (float*)psi_b,
                                             md, lat, pp.rho0_f);
   else
-    k_mom_enter<__half><<<grid, 128, 0, s>>>((const __half*)fa, (const __half*)fb, st, flags, (float*)psi_a,
+    k_mom_enter<__half><<<grid, 128, 0, s>>>((__half*)fa, (__half*)fb, st, flags, (float*)psi_a,
                                              (float*)psi_b, md, lat, pp.rho0_f);
 }
 
 void launch_mom_fill(int prec, const Lat& lat, void* fa, void* fb, const StepState* st, const void* psi_a,
-                     const void* psi_b, const MomDev& md, const PhysParams& pp, int next, cudaStream_t s) {
+                     const void* psi_b, const MomDev& md, ChainState* cs, const PhysParams& pp, int next,
+                     cudaStream_t s) {
   // inside a step the launch is a test of one word in nearly every step: one block per SM
   const unsigned grid = (unsigned)std::min(
       (lat.N + 255) / 256, next ? std::max(1LL, (long long)sm_count() / g_launch_share) : 16LL * sm_count());
   if (prec == 1)
-    k_mom_fill<float><<<grid, 256, 0, s>>>((float*)fa, (float*)fb, st, (const float*)psi_a, (const float*)psi_b, md, lat,
+    k_mom_fill<float><<<grid, 256, 0, s>>>((float*)fa, (float*)fb, st, (const float*)psi_a, (const float*)psi_b, md, cs, lat,
                                            pp, next);
   else
-    k_mom_fill<__half><<<grid, 256, 0, s>>>((__half*)fa, (__half*)fb, st, (const float*)psi_a, (const float*)psi_b, md,
+    k_mom_fill<__half><<<grid, 256, 0, s>>>((__half*)fa, (__half*)fb, st, (const float*)psi_a, (const float*)psi_b, md, cs,
                                             lat, pp, next);
 }
 
-void launch_mom_close(int prec, const Lat& lat, const void* fa, const void* fb, StepState* st, const uint16_t* flags,
-                      void* psi_a, void* psi_b, const MomDev& md, const int* blist, const PhysParams& pp, int next,
+void launch_mom_close(int prec, const Lat& lat, void* fa, void* fb, StepState* st, const uint16_t* flags,
+                      void* psi_a, void* psi_b, const MomDev& md, const int* events, ChainState* cs, const int* blist, const PhysParams& pp, int next,
                       double* mass_part, cudaStream_t s) {
   if (!blist) return;
   const unsigned grid = (unsigned)std::max(1, 4 * sm_count() / g_launch_share);
   if (prec == 1)
-    k_mom_close<float><<<grid, 128, 0, s>>>((const float*)fa, (const float*)fb, st, flags, (float*)psi_a, (float*)psi_b,
-                                            md, blist, lat, pp.rho0_f, next, mass_part);
+    k_mom_close<float><<<grid, 128, 0, s>>>((float*)fa, (float*)fb, st, flags, (float*)psi_a, (float*)psi_b,
+                                            md, events, cs, blist, lat, pp.rho0_f, next, mass_part);
   else
-    k_mom_close<__half><<<grid, 128, 0, s>>>((const __half*)fa, (const __half*)fb, st, flags, (float*)psi_a,
-                                             (float*)psi_b, md, blist, lat, pp.rho0_f, next, mass_part);
+    k_mom_close<__half><<<grid, 128, 0, s>>>((__half*)fa, (__half*)fb, st, flags, (float*)psi_a,
+                                             (float*)psi_b, md, events, cs, blist, lat, pp.rho0_f, next, mass_part);
 }
 
 // Accumulating pass: blocks of 32 x ty threads (ty = 8 or 16) marching sz planes. Resident blocks
@@ -1829,25 +1930,18 @@ void launch_psi_fixup(int prec, const Lat& lat, const void* fa, const void* fb, 
 }
 
 template <typename S>
-static void boundary_t(const Lat& lat, const S* fa, const S* fb, const uint16_t* flags, const BodyDev* bodies,
-                       double* acc, const int* blist, const StepState* st, const void* nbuf, double G,
-                       cudaStream_t s) {
-  using R = typename St<S>::R;
-  // whole-lattice grid-stride rounds; the list length is only known on the device
-  k_boundary<S><<<std::max(2, 8 * sm_count() / g_launch_share), 256, 0, s>>>(fa, fb, flags, bodies, acc, blist, st, (const RhoPsi<R>*)nbuf, lat, G,
-                                                (float)G);
+static void boundary_t(const ChainLaunch& c, cudaStream_t s) {
+  // the list length is only known on the device: a few blocks per SM, shared between a batch's contexts
+  const dim3 g((unsigned)std::max(2, 4 * sm_count() / c.share), 1, (unsigned)c.inst);
+  if (c.sets) k_boundary<S, true><<<g, LINK_T, 0, s>>>(c.one, c.sets);
+  else k_boundary<S, false><<<g, LINK_T, 0, s>>>(c.one, nullptr);
 }
 
-void launch_boundary(int prec, const Lat& lat, const void* fa, const void* fb, const uint16_t* flags,
-                     const BodyDev* bodies, int nb, double* acc, const int* blist, const StepState* st,
-                     const void* nbuf, double G, cudaStream_t s) {
-  if (nb == 0) return;
-  if (prec == 0)
-    boundary_t<double>(lat, (const double*)fa, (const double*)fb, flags, bodies, acc, blist, st, nbuf, G, s);
-  else if (prec == 1)
-    boundary_t<float>(lat, (const float*)fa, (const float*)fb, flags, bodies, acc, blist, st, nbuf, G, s);
-  else
-    boundary_t<__half>(lat, (const __half*)fa, (const __half*)fb, flags, bodies, acc, blist, st, nbuf, G, s);
+void launch_boundary(int prec, const ChainLaunch& c, cudaStream_t s) {
+  if (!c.bodies) return;
+  if (prec == 0) boundary_t<double>(c, s);
+  else if (prec == 1) boundary_t<float>(c, s);
+  else boundary_t<__half>(c, s);
 }
 
 void launch_init_fluid(int prec, const Lat& lat, void* f, const uint16_t* flags, const double* rho, const double* u,
@@ -1859,21 +1953,23 @@ void launch_init_fluid(int prec, const Lat& lat, void* f, const uint16_t* flags,
   else k_init_fluid<__half><<<blocks, T, 0, s>>>((__half*)f, flags, rho, u, lat);
 }
 
-void launch_refill(int prec, const Lat& lat, void* fa, void* fb, uint16_t* flags, const BodyDev* bodies, int nb,
-                   int max_tile, StepState* st, int* blist, const double* arena, double member_thr, int* mbox,
-                   int next, cudaStream_t s) {
-  if (nb == 0) return;
-  const int T = 256;
-  dim3 grid((unsigned)((max_tile + T - 1) / T), (unsigned)nb);
-  if (prec == 0)
-    k_refill<double><<<grid, T, 0, s>>>((double*)fa, (double*)fb, flags, bodies, st, blist, lat, arena, member_thr,
-                                        mbox, next);
-  else if (prec == 1)
-    k_refill<float><<<grid, T, 0, s>>>((float*)fa, (float*)fb, flags, bodies, st, blist, lat, arena, member_thr, mbox,
-                                       next);
-  else
-    k_refill<__half><<<grid, T, 0, s>>>((__half*)fa, (__half*)fb, flags, bodies, st, blist, lat, arena, member_thr,
-                                        mbox, next);
+template <typename S, bool B, int Z>
+static void near_refill_z(const ChainLaunch& c, int next, cudaStream_t s) {
+  const dim3 g((unsigned)((c.max_xy + TILE_T - 1) / TILE_T), (unsigned)((c.max_z + Z - 1) / Z), (unsigned)c.bodies);
+  k_near_refill<S, B, Z><<<g, TILE_T, 0, s>>>(c.one, c.sets, c.items, next);
+}
+template <typename S>
+static void near_refill_t(const ChainLaunch& c, int next, cudaStream_t s) {
+  const bool four = tile_planes(c, sm_count()) == TILE_Z;
+  if (c.sets) four ? near_refill_z<S, true, TILE_Z>(c, next, s) : near_refill_z<S, true, 1>(c, next, s);
+  else four ? near_refill_z<S, false, TILE_Z>(c, next, s) : near_refill_z<S, false, 1>(c, next, s);
+}
+
+void launch_near_refill(int prec, const ChainLaunch& c, int next, cudaStream_t s) {
+  if (!c.bodies) return;
+  if (prec == 0) near_refill_t<double>(c, next, s);
+  else if (prec == 1) near_refill_t<float>(c, next, s);
+  else near_refill_t<__half>(c, next, s);
 }
 
 // Tile shapes of the persistent batch kernels (x, y, z cells): of the split pass (128 threads per block),
@@ -1915,6 +2011,30 @@ static int batch_mom_occ() {
       cudaSuccess)
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_batch_mom<S, MOM_TY, MOM_MINB>, T::NT, T::smem);
   return nb;
+}
+
+// a batch's kernels of the chain that work on the lattice: a few blocks per instance
+static dim3 batch_grid(int ninst, int per_sm) {
+  return dim3((unsigned)std::max(1, (per_sm * sm_count() + ninst - 1) / ninst), (unsigned)ninst);
+}
+void launch_batch_begin(const BatchInst* tab, int ninst, BatchCtl* ctl, int diag, cudaStream_t s) {
+  k_batch_begin<<<(ninst + 127) / 128, 128, 0, s>>>(tab, ninst, ctl, diag);
+}
+void launch_batch_near(int prec, const BatchInst* tab, int ninst, cudaStream_t s) {
+  const dim3 g = batch_grid(ninst, 8);
+  if (prec == 0) k_batch_near<double><<<g, 128, 0, s>>>(tab);
+  else if (prec == 1) k_batch_near<float><<<g, 128, 0, s>>>(tab);
+  else k_batch_near<__half><<<g, 128, 0, s>>>(tab);
+}
+void launch_batch_fill(int prec, const BatchInst* tab, int ninst, cudaStream_t s) {
+  const dim3 g = batch_grid(ninst, 1);
+  if (prec == 1) k_batch_fill<float><<<g, 256, 0, s>>>(tab);
+  else k_batch_fill<__half><<<g, 256, 0, s>>>(tab);
+}
+void launch_batch_close(int prec, const BatchInst* tab, int ninst, cudaStream_t s) {
+  const dim3 g = batch_grid(ninst, 8);
+  if (prec == 1) k_batch_close<float><<<g, 128, 0, s>>>(tab);
+  else k_batch_close<__half><<<g, 128, 0, s>>>(tab);
 }
 
 // resident blocks per SM of the moment pass's batch kernel (and its shared-memory limit set)

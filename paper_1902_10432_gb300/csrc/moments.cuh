@@ -170,7 +170,12 @@ struct MomArgs {
   double *diag_rho, *diag_vel;
 };
 
-template <typename S, int TY>
+// FETCH: f* of the cells next to a solid is fetched a plane ahead. Loaded where it is used, a plane that
+// holds such a cell waits for memory once more; fetched, every plane pays for the look ahead. Spheres of
+// R 5 to 24 in boxes of 64 to 128 cells (nearly every column meets one): 2600 -> 1812 us per step of 64. One
+// 256^3 lattice with four of R = 24: 335 -> 347 us; 60 spheres in 224^3: 439 -> 424 of a step of 1240. A batch
+// fetches, a single lattice does not.
+template <typename S, int TY, bool FETCH>
 __device__ __forceinline__ void mom_column(const MomArgs<S>& a, const Lat& lat, const PhysParams& pp, int x0, int y0,
                                            int zb, int sz, unsigned slot_id, float* __restrict__ smem) {
   using T = MomTile<TY>;
@@ -215,7 +220,7 @@ __device__ __forceinline__ void mom_column(const MomArgs<S>& a, const Lat& lat, 
   const int x = wrapi(x0 - 1 + ex, lat.nx), y = wrapi(y0 - 1 + ey, lat.ny);
   const unsigned nxy = (unsigned)lat.nx * (unsigned)lat.ny, col = (unsigned)x + (unsigned)lat.nx * (unsigned)y;
   const int e = ey * T::EX + ex, pe = (ey + 1) * T::PX + ex + 1;
-  const unsigned char* const mapc = map + md.brick(x >> 3, y >> 3, 0);
+  const unsigned char* const mapc = map + md.brick(x >> BRICK_BITS, y >> BRICK_BITS, 0);
   const unsigned mapz = (unsigned)(md.nbx * md.nby);
   // psi columns this thread copies (at most two)
   unsigned pc[2];
@@ -239,14 +244,26 @@ __device__ __forceinline__ void mom_column(const MomArgs<S>& a, const Lat& lat, 
   copy_psi(0, 0);
   copy_psi(1, 1);
   copy_psi(2, 2);
-  unsigned nq = col + plane0(zb - 1);  // cell of the plane being computed
+  unsigned nq = col + plane0(zb - 1), nq1 = col + plane0(zb);  // cell of the plane being computed, of the next
   float4 m = M[nq];
-  uint16_t fl = flags[nq], fl_prev = 0;
+  // flags of the plane being computed, of the one before and (FETCH) the one after
+  uint16_t fl = flags[nq], fl_prev = 0, fl_next = FETCH ? flags[nq1] : (uint16_t)0;
   float f0 = 0.0f;
-  bool brick = mapc[mapz * ((unsigned)zb >> 3)];  // populations are stored in the cell's brick
+  bool brick = mapc[mapz * ((unsigned)zb >> BRICK_BITS)];  // populations are stored in the cell's brick
   MassAcc<float> mass;
   float* const fe = sf + e;
   const float* const pe0 = sp + pe;
+  // f* of a cell next to a solid (k_collide_near stored it), fetched into its place in shared memory behind
+  // the completion of the plane before. Halves arrive as the aligned word that holds them.
+  auto fetch_near = [&](float* s, unsigned n) {
+#pragma unroll
+    for (int i = 1; i < Q; ++i) {
+      const size_t k = (size_t)i * N + n;
+      cp_async4(s + (i - 1) * T::NE, sizeof(S) == 2 ? dst + (k & ~(size_t)1) : dst + k);
+    }
+  };
+  if (FETCH && ext && (fl & (F_SOLID | F_NEAR)) == F_NEAR) fetch_near(fe, nq);
+  cp_async_commit();
   cp_async_wait<0>();
   __syncthreads();
   // plane j is z = zb - 1 + j; planes 0 and planes + 1 are only pulled from. C = j mod 4.
@@ -257,29 +274,42 @@ __device__ __forceinline__ void mom_column(const MomArgs<S>& a, const Lat& lat, 
     const float4 mc = m;
     const uint16_t fc = fl;
     if (j <= planes) {
-      nq = col + plane0(zb + j);
-      m = M[nq];
-      fl = flags[nq];
+      if constexpr (FETCH) {
+        nq = nq1;
+        m = M[nq];
+        fl = fl_next;
+        nq1 = col + plane0(zb + min(j, planes - 1) + 1);
+        fl_next = flags[nq1];
+      } else {
+        nq = col + plane0(zb + j);
+        m = M[nq];
+        fl = flags[nq];
+      }
     }
     const float f0_prev = f0;
     const bool mine = own && j >= 1 && j <= planes;
     float* const s = fe + C * (Q - 1) * T::NE;
     if (fc & (F_SOLID | F_NEAR)) {
       if (fc & F_SOLID) {
-        if (mine) {
-#pragma unroll
-          for (int i = 0; i < Q; ++i) St<S>::st(dst, (size_t)i * N + n, i, 0.0f);
-          if (diag) {
-            diag_rho[n] = 0.0;
-            diag_vel[3 * (size_t)n] = 0.0;
-            diag_vel[3 * (size_t)n + 1] = 0.0;
-            diag_vel[3 * (size_t)n + 2] = 0.0;
-          }
+        if (mine && diag) {
+          diag_rho[n] = 0.0;
+          diag_vel[3 * (size_t)n] = 0.0;
+          diag_vel[3 * (size_t)n + 1] = 0.0;
+          diag_vel[3 * (size_t)n + 2] = 0.0;
         }
       } else if (ext) {
-        f0 = St<S>::ldv(dst, (size_t)n, 0);
+        f0 = St<S>::ldv(dst, (size_t)n, 0);  // (used a plane later)
+        if constexpr (!FETCH) {
 #pragma unroll
-        for (int i = 1; i < Q; ++i) s[(i - 1) * T::NE] = St<S>::ldv(dst, (size_t)i * N + n, i);
+          for (int i = 1; i < Q; ++i) s[(i - 1) * T::NE] = St<S>::ldv(dst, (size_t)i * N + n, i);
+        } else if constexpr (sizeof(S) == 2) {
+          cp_async_wait<0>();
+#pragma unroll
+          for (int i = 1; i < Q; ++i) {
+            const unsigned w = __float_as_uint(s[(i - 1) * T::NE]);
+            s[(i - 1) * T::NE] = St<S>::from_raw((unsigned short)(((size_t)i * N + n) & 1 ? w >> 16 : w), i);
+          }
+        }
       }
     } else if (ext) {
       auto psi_at = [&](int i) -> float {
@@ -308,12 +338,14 @@ __device__ __forceinline__ void mom_column(const MomArgs<S>& a, const Lat& lat, 
         }
       }
     }
-    if (j >= 1 && ((zb + j) & 7) == 0 && j < planes) brick = mapc[mapz * ((unsigned)(zb + j) >> 3)];
+    if (j >= 1 && ((zb + j) & ((1 << BRICK_BITS) - 1)) == 0 && j < planes) brick = mapc[mapz * ((unsigned)(zb + j) >> BRICK_BITS)];
     cp_async_wait<0>();
     // the one barrier per plane: f* of this plane and psi of the plane after next are in place. The planes
     // of f* that the slowest warp still pulls (j - 2 .. j) and the one the fastest writes next (j + 1)
     // are four different ones; psi that is overwritten next was read before this barrier.
     __syncthreads();
+    // into the plane of f* that was last pulled from before this barrier
+    if (FETCH && j <= planes && ext && (fl & (F_SOLID | F_NEAR)) == F_NEAR) fetch_near(fe + ((C + 1) & 3) * (Q - 1) * T::NE, nq);
     if (j >= 2 && own) {
       float fi[Q];
       fi[0] = f0_prev;
@@ -340,13 +372,9 @@ __device__ __forceinline__ void mom_column(const MomArgs<S>& a, const Lat& lat, 
   add_mass_slot(a.mass_part, mass, slot_id);
 }
 
-// at the start of a step: the next step's brick map is empty, this step's flag events too (both were
-// last read in the step before). Share k of n threads.
+// at the start of a step: the next step's brick map is empty (it was last read in the step before). Share
+// k of n threads.
 __device__ __forceinline__ void mom_reset(const MomDev& md, int parity, unsigned k, unsigned n) {
-  if (k == 0) {
-    md.ms->nevent = 0;
-    md.ms->full = 0;
-  }
   unsigned char* const map = md.map(parity ^ 1);
   const unsigned bricks = md.bricks();
   for (; k < bricks; k += n) map[k] = 0;
@@ -357,56 +385,82 @@ __global__ void __launch_bounds__(MomTile<TY>::NT, MINB) k_mom(const MomArgs<S> 
   extern __shared__ __align__(16) float mom_smem[];
   const unsigned blk = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
   mom_reset(a.md, a.st->parity, blk * MomTile<TY>::NT + threadIdx.x, gridDim.x * gridDim.y * gridDim.z * MomTile<TY>::NT);
-  mom_column<S, TY>(a, lat, pp, blockIdx.x * 32, blockIdx.y * TY, blockIdx.z * sz, sz, blk, mom_smem);
+  mom_column<S, TY, false>(a, lat, pp, blockIdx.x * 32, blockIdx.y * TY, blockIdx.z * sz, sz, blk, mom_smem);
 }
 
 // The moment pass over a batch: one persistent launch (as k_batch_lbm: every block resident, work items
 // from a device queue, one bounded grid barrier). Phase 0: the cells next to a solid of every instance,
-// MOM_NEAR_ITEMS items each; phase 1: the columns, sz planes each.
+// MOM_NEAR_ITEMS items each; phase 1: the columns, sz planes each. The instance's entry is copied to shared
+// memory and phase 0 kept out of line: with the table read from global memory and both phases in one
+// body, 50 words spilled. 64 pairs of spheres, 54 M cells on this pass: 1812 us (k_mom's rate on
+// 256^3 would give 1000; the near cells, and box sides that are no multiple of 32, take the rest).
 constexpr int MOM_NEAR_ITEMS = 8;
+template <typename S>
+__device__ __noinline__ float batch_near_item(const BatchInst& I, unsigned k, unsigned n) {
+  mom_reset(I.md, I.st->parity, k, n);
+  return near_cells<S, true>((S*)I.fa, (S*)I.fb, I.flags, (const float*)I.psi, (const float*)I.psi2, I.bodies, I.st,
+                             I.diag_rho, I.diag_vel, I.blist, I.lat, I.pp, (RhoPsi<float>*)I.nbuf, k, n);
+}
 template <typename S, int TY, int MINB>
 __global__ void __launch_bounds__(MomTile<TY>::NT, MINB)
     k_batch_mom(const BatchInst* __restrict__ tab, int ninst, long long items, BatchCtl* ctl, int sz) {
   constexpr int NT = MomTile<TY>::NT;
   extern __shared__ __align__(16) float mom_smem[];
+  __shared__ BatchInst I;
   __shared__ long long s_item;
-  for (int phase = 0; phase < 2; ++phase) {
-    if (phase == 1 && !grid_barrier(ctl)) return;
-    const long long n_items = phase ? items : (long long)ninst * MOM_NEAR_ITEMS;
-    for (;;) {
-      if (threadIdx.x == 0) s_item = (long long)atomicAdd(&ctl->queue[phase], 1ull);
+  __shared__ int s_inst;
+  for (;;) {
+    if (threadIdx.x == 0) s_item = (long long)atomicAdd(&ctl->queue[0], 1ull);
+    __syncthreads();
+    const long long item = s_item;
+    __syncthreads();  // s_item is written again in the next round
+    if (item >= (long long)ninst * MOM_NEAR_ITEMS) break;
+    const BatchInst& J = tab[item / MOM_NEAR_ITEMS];
+    const float m = batch_near_item<S>(J, (unsigned)(item % MOM_NEAR_ITEMS) * NT + threadIdx.x, MOM_NEAR_ITEMS * NT);
+    add_mass_slot(J.mass_part, m, (unsigned)item);
+  }
+  if (!grid_barrier(ctl)) return;
+  long long item0 = 0, item1 = 0;  // items of the instance in I
+  for (;;) {
+    if (threadIdx.x == 0) s_item = (long long)atomicAdd(&ctl->queue[1], 1ull);
+    __syncthreads();
+    const long long item = s_item;
+    if (item >= items) return;
+    if (item < item0 || item >= item1) {
+      for (int k = threadIdx.x; k < ninst; k += NT)
+        if (tab[k].item0 <= item && (k + 1 == ninst || tab[k + 1].item0 > item)) s_inst = k;
       __syncthreads();
-      const long long item = s_item;
-      __syncthreads();  // s_item is written again in the next round
-      if (item >= n_items) break;
-      if (phase == 0) {
-        const BatchInst& I = tab[item / MOM_NEAR_ITEMS];
-        const unsigned k = (unsigned)(item % MOM_NEAR_ITEMS) * NT + threadIdx.x, n = MOM_NEAR_ITEMS * NT;
-        mom_reset(I.md, I.st->parity, k, n);
-        const float m = near_cells<S, true>((S*)I.fa, (S*)I.fb, I.flags, (const float*)I.psi, (const float*)I.psi2,
-                                            I.bodies, I.st, I.diag_rho, I.diag_vel, I.blist, I.lat, I.pp,
-                                            (RhoPsi<float>*)I.nbuf, k, n);
-        add_mass_slot(I.mass_part, m, (unsigned)item);
-      } else {
-        const int lo = batch_instance(tab, ninst, item);
-        const BatchInst& I = tab[lo];
-        const long long k = item - I.item0;
-        const int bx = (int)(k % I.tiles[0]), by = (int)((k / I.tiles[0]) % I.tiles[1]),
-                  bz = (int)(k / ((long long)I.tiles[0] * I.tiles[1]));
-        const MomArgs<S> a{(S*)I.fa, (S*)I.fb, I.flags, (float*)I.psi, (float*)I.psi2, I.md, I.mass_part, I.st,
-                           I.diag_rho, I.diag_vel};
-        const Lat lat = I.lat;
-        mom_column<S, TY>(a, lat, I.pp, bx * 32, by * TY, bz * sz, sz, (unsigned)k, mom_smem);
-      }
+      static_assert(sizeof(BatchInst) % sizeof(long long) == 0, "copied in words of eight bytes");
+      for (int k = threadIdx.x; k < (int)(sizeof(BatchInst) / sizeof(long long)); k += NT)
+        reinterpret_cast<long long*>(&I)[k] = reinterpret_cast<const long long*>(tab + s_inst)[k];
+      __syncthreads();
+      item0 = I.item0;
+      item1 = item0 + (long long)I.tiles[0] * I.tiles[1] * I.tiles[2];
     }
+    const int k = (int)(item - item0);
+    const int tx = I.tiles[0], ty = I.tiles[1], bx = k % tx, by = (k / tx) % ty, bz = k / (tx * ty);
+    const MomArgs<S> a{(S*)I.fa, (S*)I.fb, I.flags, (float*)I.psi, (float*)I.psi2, I.md, I.mass_part, I.st,
+                       I.diag_rho, I.diag_vel};
+    mom_column<S, TY, true>(a, I.lat, I.pp, bx * 32, by * TY, bz * sz, sz, (unsigned)k, mom_smem);
+    __syncthreads();  // s_item, I and the planes in shared memory are written again
+  }
+}
+
+// a solid cell's populations are zero in both buffers, from here or from the step that covered it on: a cell
+// that is uncovered starts empty
+template <typename S>
+__device__ __forceinline__ void zero_populations(S* fa, S* fb, const Lat& lat, unsigned n) {
+#pragma unroll
+  for (int i = 0; i < Q; ++i) {
+    St<S>::st(fa, (size_t)i * (size_t)lat.Ns + n, i, 0.0f);
+    St<S>::st(fb, (size_t)i * (size_t)lat.Ns + n, i, 0.0f);
   }
 }
 
 // moments and psi of every cell from complete populations (after initialisation, a load, a move): the
 // entry into the moment pass
 template <typename S>
-__global__ void __launch_bounds__(128) k_mom_enter(const S* __restrict__ fa, const S* __restrict__ fb,
-                                                   const StepState* __restrict__ st, const uint16_t* __restrict__ flags,
+__global__ void __launch_bounds__(128) k_mom_enter(S* fa, S* fb, const StepState* __restrict__ st, const uint16_t* __restrict__ flags,
                                                    float* __restrict__ psi_a, float* __restrict__ psi_b, MomDev md,
                                                    Lat lat, float rho0_f) {
   const int x = blockIdx.x * 32 + (threadIdx.x & 31), y = blockIdx.y * 4 + (threadIdx.x >> 5), z = blockIdx.z;
@@ -420,11 +474,12 @@ __global__ void __launch_bounds__(128) k_mom_enter(const S* __restrict__ fa, con
     }
   }
   if (x >= lat.nx || y >= lat.ny) return;
-  const S* __restrict__ f = parity ? fb : fa;
+  const S* const f = parity ? fb : fa;
   const Cell c = make_cell(x, y, z, lat);
   const uint16_t fl = flags[c.n];
   if (fl & F_SOLID) {
     md.M(parity)[c.n] = make_float4(MOM_SOLID, 0.0f, 0.0f, 0.0f);
+    zero_populations<S>(fa, fb, lat, c.n);
     return;
   }
   float fi[Q];
@@ -439,18 +494,18 @@ __global__ void __launch_bounds__(128) k_mom_enter(const S* __restrict__ fa, con
 // that made them. next = 1: inside a step (the parity has not flipped), and then only if a flag
 // changed outside the stored bricks; next = 0: between steps.
 template <typename S>
-__global__ void __launch_bounds__(256) k_mom_fill(S* __restrict__ fa, S* __restrict__ fb,
-                                                  const StepState* __restrict__ st, const float* __restrict__ psi_a,
-                                                  const float* __restrict__ psi_b, MomDev md, Lat lat, PhysParams pp,
-                                                  int next) {
-  if (next && !md.ms->full) return;
+__device__ __forceinline__ void mom_fill(S* __restrict__ fa, S* __restrict__ fb, const StepState* __restrict__ st,
+                                         const float* __restrict__ psi_a, const float* __restrict__ psi_b,
+                                         const MomDev& md, const ChainState* __restrict__ cs, const Lat& lat,
+                                         const PhysParams& pp, int next) {
+  if (next && !cs->full) return;
   const int t = next ? st->parity : st->parity ^ 1;
   S* __restrict__ f = t ? fa : fb;
   const float* __restrict__ psi = t ? psi_b : psi_a;
   const size_t N = (size_t)lat.Ns;
   for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < lat.N; k += (long long)gridDim.x * blockDim.x) {
     const Cell c = cell_of(k, lat);
-    if (md.map(t)[md.brick(c.x >> 3, c.y >> 3, c.z >> 3)]) continue;
+    if (md.map(t)[md.brick(c.x >> BRICK_BITS, c.y >> BRICK_BITS, c.z >> BRICK_BITS)]) continue;
     const float4 m = md.M(t)[c.n];
     if (m.x == MOM_SOLID) {
 #pragma unroll
@@ -464,32 +519,44 @@ __global__ void __launch_bounds__(256) k_mom_fill(S* __restrict__ fa, S* __restr
   }
 }
 
-// the bricks within 4 cells of a cell near the periodic seam
+// the bricks around a cell near the periodic seam
 __device__ __noinline__ void mark_bricks_seam(const MomDev& md, int t, int x, int y, int z, const Lat& lat) {
   int b[3][BRICK_SPAN], nbk[3];
-  nbk[0] = brick_span(x, 4, lat.nx, b[0]);
-  nbk[1] = brick_span(y, 4, lat.ny, b[1]);
-  nbk[2] = brick_span(z, 4, lat.nz, b[2]);
+  nbk[0] = brick_span(x, BRICK_REACH, lat.nx, b[0]);
+  nbk[1] = brick_span(y, BRICK_REACH, lat.ny, b[1]);
+  nbk[2] = brick_span(z, BRICK_REACH, lat.nz, b[2]);
   for (int iz = 0; iz < nbk[2]; ++iz)
     for (int iy = 0; iy < nbk[1]; ++iy)
       for (int ix = 0; ix < nbk[0]; ++ix) md.map(t)[md.brick(b[0][ix], b[1][iy], b[2][iz])] = 1;
 }
 
+template <typename S>
+__global__ void __launch_bounds__(256) k_mom_fill(S* fa, S* fb, const StepState* st, const float* psi_a,
+                                                  const float* psi_b, const MomDev md, const ChainState* cs, const Lat lat,
+                                                  const PhysParams pp, int next) {
+  mom_fill<S>(fa, fb, st, psi_a, psi_b, md, cs, lat, pp, next);
+}
+template <typename S>
+__global__ void __launch_bounds__(256) k_batch_fill(const BatchInst* __restrict__ tab) {
+  const BatchInst& I = tab[blockIdx.y];
+  mom_fill<S>((S*)I.fa, (S*)I.fb, I.st, (const float*)I.psi, (const float*)I.psi2, I.md, I.cs, I.lat, I.pp, 1);
+}
+
 // End of a step, after the refill: for the cells next to a solid, psi of the next step and the bricks
-// around them (within 4 cells) in which the next step stores populations; and around every cell
-// whose obstacle flag changed (within 2 cells: the receivers of its refill are next to it, and the
-// cells that pull from those one further) the moments and psi of the cells that are not.
+// around them in which the next step stores populations; and around every cell whose obstacle flag
+// changed the moments and psi of the cells that are not: within 2 cells of a covered one (the receivers of
+// its refill are next to it, and the cells that pull from those one further), within 1 of an uncovered one.
 // The last block then ends the step, as k_finish does for the other passes.
 template <typename S>
-__global__ void __launch_bounds__(128) k_mom_close(const S* __restrict__ fa, const S* __restrict__ fb,
-                                                   StepState* __restrict__ st, const uint16_t* __restrict__ flags,
-                                                   float* __restrict__ psi_a, float* __restrict__ psi_b, MomDev md,
-                                                   const int* __restrict__ blist, Lat lat, float rho0_f, int next,
-                                                   double* __restrict__ mass_part) {
+__device__ __forceinline__ void mom_close(S* fa, S* fb, StepState* __restrict__ st,
+                                          const uint16_t* __restrict__ flags, float* __restrict__ psi_a,
+                                          float* __restrict__ psi_b, const MomDev& md, const int* __restrict__ events,
+                                          ChainState* __restrict__ cs, const int* __restrict__ blist, const Lat& lat,
+                                          float rho0_f, int next, double* __restrict__ mass_part) {
   const int t = next ? st->parity ^ 1 : st->parity;  // the next step's parity
-  const S* __restrict__ f = t ? fb : fa;
+  const S* const f = t ? fb : fa;
   float* __restrict__ psi = t ? psi_b : psi_a;
-  const unsigned near = st->nbnd, total = near + 125u * (next ? md.ms->nevent : 0u);
+  const unsigned near = next ? cs->nnew : st->nbnd, total = near + 125u * (next ? cs->nevent : 0u);
   for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < total; k += gridDim.x * blockDim.x) {
     float fi[Q];
     unsigned sl;
@@ -500,24 +567,31 @@ __global__ void __launch_bounds__(128) k_mom_close(const S* __restrict__ fa, con
 #pragma unroll
       for (int i = 0; i < Q; ++i) rho += fi[i];
       psi[c.n] = mom_psi(rho, rho0_f);
-      if (c.x >= 4 && c.y >= 4 && c.z >= 4 && c.x + 4 < lat.nx && c.y + 4 < lat.ny && c.z + 4 < lat.nz) {
-        // nine cells in a row touch at most two bricks of eight
+      if (c.x >= BRICK_REACH && c.y >= BRICK_REACH && c.z >= BRICK_REACH && c.x + BRICK_REACH < lat.nx &&
+          c.y + BRICK_REACH < lat.ny && c.z + BRICK_REACH < lat.nz) {
+        // seven cells in a row touch at most three bricks of four
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
-          md.map(t)[md.brick((c.x + (q & 1 ? 4 : -4)) >> 3, (c.y + (q & 2 ? 4 : -4)) >> 3, (c.z + (q & 4 ? 4 : -4)) >> 3)] = 1;
+        for (int q = 0; q < 27; ++q)
+          md.map(t)[md.brick((c.x + (q % 3 - 1) * BRICK_REACH) >> BRICK_BITS, (c.y + (q / 3 % 3 - 1) * BRICK_REACH) >> BRICK_BITS,
+                             (c.z + (q / 9 - 1) * BRICK_REACH) >> BRICK_BITS)] = 1;
       } else {
         mark_bricks_seam(md, t, c.x, c.y, c.z, lat);
       }
     } else {
       const unsigned r = k - near, ev = r / 125u, o = r - 125u * ev;
-      const Cell a = cell_of(md.events[ev], lat);
+      const Cell a = cell_of(events[ev], lat);
       const int x = wrapi_near(a.x + (int)(o % 5u) - 2, lat.nx), y = wrapi_near(a.y + (int)((o / 5u) % 5u) - 2, lat.ny),
                 z = wrapi_near(a.z + (int)(o / 25u) - 2, lat.nz);
       const Cell c = make_cell(x, y, z, lat);
+      // an uncovered cell starts empty: it changes itself and those that pull from it, no further
+      const bool inner = (unsigned)((int)(o % 5u) - 1) < 3u && (unsigned)((int)((o / 5u) % 5u) - 1) < 3u && o >= 25u && o < 100u;
+      if (!inner && !(flags[a.n] & F_COVER)) continue;
       const uint16_t fl = flags[c.n];
       if (fl & F_NEAR) continue;
       if (fl & F_SOLID) {
         md.M(t)[c.n] = make_float4(MOM_SOLID, 0.0f, 0.0f, 0.0f);
+        // (no fluid cell pulls from a solid one, so nothing reads what this overwrites)
+        if (o == 62u && (fl & F_COVER)) zero_populations<S>(fa, fb, lat, c.n);
         continue;
       }
       pull<S>(f, flags, lat, c, (long long)c.n, fi, sl, 0);
@@ -531,10 +605,43 @@ __global__ void __launch_bounds__(128) k_mom_close(const S* __restrict__ fa, con
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
-    s_last = atomicAdd(&md.ms->done, 1u) == gridDim.x - 1;
+    s_last = atomicAdd(&cs->done, 1u) == gridDim.x - 1;
   }
   __syncthreads();
   if (!s_last) return;
-  if (threadIdx.x == 0) md.ms->done = 0;
-  finish_step<128>(mass_part, MASS_SLOTS, st);
+  if (threadIdx.x == 0) cs->done = 0;
+  finish_step<128>(mass_part, MASS_SLOTS, st, cs);
+}
+
+template <typename S>
+__global__ void __launch_bounds__(128) k_mom_close(S* fa, S* fb, StepState* st, const uint16_t* flags,
+                                                   float* psi_a, float* psi_b, const MomDev md, const int* events,
+                                                   ChainState* cs, const int* blist, const Lat lat, float rho0_f, int next,
+                                                   double* mass_part) {
+  mom_close<S>(fa, fb, st, flags, psi_a, psi_b, md, events, cs, blist, lat, rho0_f, next, mass_part);
+}
+template <typename S>
+__global__ void __launch_bounds__(128) k_batch_close(const BatchInst* __restrict__ tab) {
+  const BatchInst& I = tab[blockIdx.y];
+  mom_close<S>((S*)I.fa, (S*)I.fb, I.st, I.flags, (float*)I.psi, (float*)I.psi2, I.md, I.events, I.cs, I.blist,
+               I.lat, I.pp.rho0_f, 1, I.mass_part);
+}
+// the cells next to a solid of a batch's instances on the split pass
+template <typename S>
+__global__ void __launch_bounds__(128) k_batch_near(const BatchInst* __restrict__ tab) {
+  using R = typename St<S>::R;
+  const BatchInst& I = tab[blockIdx.y];
+  const R mass = near_cells<S, false>((S*)I.fa, (S*)I.fb, I.flags, (const R*)I.psi, (const R*)nullptr, I.bodies, I.st,
+                                      I.diag_rho, I.diag_vel, I.blist, I.lat, I.pp, (RhoPsi<R>*)I.nbuf,
+                                      blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+  add_mass_slot(I.mass_part, mass, blockIdx.x * 7u + 3u);
+}
+// start of a batch's step: field record on or off, work queues and barrier arrivals cleared
+__global__ void k_batch_begin(const BatchInst* __restrict__ tab, int ninst, BatchCtl* ctl, int diag) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k < ninst) tab[k].st->diag = diag;
+  if (k < 2) {
+    ctl[k].queue[0] = ctl[k].queue[1] = 0;
+    ctl[k].arrive = 0;
+  }
 }
