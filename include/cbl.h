@@ -291,11 +291,10 @@ cbl_status cbl_get_option(cbl_ctx* ctx, const char* key, double* value);
  * caller's device buffers (19 * nx*ny*nz floats each, not overlapping); mass_out (device, may be
  * NULL) receives the fluid mass of the step. The library cannot check the buffers' sizes or where
  * they live: too small a buffer, or a host pointer, is a memory fault on the GPU (the Python binding
- * checks them before the call). Scratch (psi, flags, mass slots) is a fixed set of device arrays
+ * checks them before the call). Scratch (psi, mass slots) is a fixed set of device arrays
  * inside the library, sized for CBL_NOALLOC_MAX_CELLS cells and held on every GPU that loads the
- * library until the process exits; larger lattices return CBL_ERR_ARG. Each call looks up those
- * arrays with the calling device current and clears, on `stream`, the part it uses; the first call
- * on a device may load the library's device code, so make it before any stream capture. All calls
+ * library until the process exits; larger lattices return CBL_ERR_ARG. Each call uses those of the
+ * calling device and clears, on `stream`, the part it needs cleared; the first call on a device may load the library's device code, so make it before any stream capture. All calls
  * share the arrays: calls that overlap on the GPU (other streams, other threads) race. Work is
  * enqueued on `stream` (NULL = legacy default stream). Returns CBL_ERR_ARG for bad sizes,
  * non-finite parameters, NULL or overlapping buffers, CBL_ERR_CUDA if a CUDA call fails. */
