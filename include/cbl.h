@@ -294,8 +294,9 @@ cbl_status cbl_get_option(cbl_ctx* ctx, const char* key, double* value);
  * checks them before the call). Scratch (psi, mass slots) is a fixed set of device arrays
  * inside the library, sized for CBL_NOALLOC_MAX_CELLS cells and held on every GPU that loads the
  * library until the process exits; larger lattices return CBL_ERR_ARG. Each call uses those of the
- * calling device and clears, on `stream`, the part it needs cleared; the first call on a device may load the library's device code, so make it before any stream capture. All calls
- * share the arrays: calls that overlap on the GPU (other streams, other threads) race. Work is
+ * calling device and clears, on `stream`, the part it needs cleared; the first call on a device may
+ * load the library's device code, so make it before any stream capture. All calls share the arrays:
+ * calls that overlap on the GPU (other streams, other threads) race. Work is
  * enqueued on `stream` (NULL = legacy default stream). Returns CBL_ERR_ARG for bad sizes,
  * non-finite parameters, NULL or overlapping buffers, CBL_ERR_CUDA if a CUDA call fails. */
 #define CBL_NOALLOC_MAX_CELLS (1 << 20)

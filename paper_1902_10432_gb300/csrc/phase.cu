@@ -20,9 +20,10 @@ namespace cbl {
 
 constexpr double PI = 3.14159265358979323846;
 constexpr int MAXOFF = 512;
-__constant__ int c_off[3 * MAXOFF];
-__constant__ double c_offf[3 * MAXOFF];  // force on the first point of a pair at offset d: f(d)
-__constant__ int c_noff;
+// (in global memory: lanes read different entries)
+__device__ int c_off[3 * MAXOFF];
+__device__ double c_offf[3 * MAXOFF];  // force on the first point of a pair at offset d: f(d)
+__device__ int c_noff;
 
 // Offsets d with 0 < |d| < r_c and the pair force e0 (n / r_c) |(|d| - r_c) / r_c|^(n-1) (-d/|d|)
 // (Eq. solid_solid_force) that a point feels from a point at x + d.
@@ -427,9 +428,13 @@ __global__ void k_body_props_finish(BodyDev* bodies, int nb, const double* scrat
 // ---- solid-solid repulsion ---------------------------------------------------------------------
 // For a point x of body A (phi_A >= the membership threshold) and every body B whose tile overlaps
 // A's: sum the table forces f(d) over the points x + d of B; torque (x - X_A) x (sum f).
+// The points in reach of a contact are few and close together: blocks take chunks of them, a warp a point, a
+// lane a few of its offsets. Two touching spheres of R = 20: 51 us with a point per thread (its
+// hundred offsets one after the other, all in a few blocks), 27 to 34 here; four at R = 24, 65 and 28. None in range: 4.
+constexpr unsigned REP_T = 256;
 
 template <bool B>
-__global__ void __launch_bounds__(256) k_repulsion(const __grid_constant__ TileSet one, const TileSet* __restrict__ sets,
+__global__ void __launch_bounds__(REP_T) k_repulsion(const __grid_constant__ TileSet one, const TileSet* __restrict__ sets,
                                                    const int2* __restrict__ items) {
   int self;
   const TileSet& S = tile_set<B>(one, sets, items, self);
@@ -494,54 +499,74 @@ __global__ void __launch_bounds__(256) k_repulsion(const __grid_constant__ TileS
   if (w0 <= 0 || w1 <= 0 || w2 <= 0) return;
   const unsigned cells = (unsigned)w0 * (unsigned)w1 * (unsigned)w2, w01 = (unsigned)w0 * (unsigned)w1;
   const long long tb = dbits(thr);
-  // grid-stride over the hull: a grid of a few waves, so that the common case (no pair in range,
-  // every block leaves after the cull above) costs one short launch
-  for (unsigned base = blockIdx.x * blockDim.x; base < cells; base += gridDim.x * blockDim.x) {
+  // chunks of the hull, of 32 to 256 cells, so that few cells still reach many SMs
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const unsigned share = (cells + gridDim.x - 1) / gridDim.x, chunk = min(REP_T, (share + 31u) & ~31u);
+  __shared__ unsigned list[REP_T], reached[REP_T];
+  static_assert(MAXNB <= 32, "a bit per neighbour");
+  __shared__ int n_list;
+  double F[3] = {0, 0, 0}, T[3] = {0, 0, 0};
+  bool has = false;
+  for (unsigned base = blockIdx.x * chunk; base < cells; base += gridDim.x * chunk) {
+    if (threadIdx.x == 0) n_list = 0;
+    __syncthreads();
     const unsigned k = base + threadIdx.x;
-    double F[3] = {0, 0, 0};
-    bool has = false;
-    TileCell c;
-    const int l2 = (int)(k / w01), l1 = (int)((k - (unsigned)l2 * w01) / (unsigned)w0), l0 = (int)(k - (unsigned)l2 * w01) - l1 * w0;
-    if (k < cells &&
-        dbits(arena[a.off + h0 + l0 + (long long)a.L[0] * (h1 + l1 + (long long)a.L[1] * (h2 + l2))]) >= tb) {
-      c = tile_at(a, h0 + l0, h1 + l1, h2 + l2, lat);
-      const int g[3] = {c.gx, c.gy, c.gz};
-      const int nn[3] = {lat.nx, lat.ny, lat.nz};
-      for (int k = 0; k < a.nnb; ++k) {
-        const BodyDev& b = bodies[a.nbl[k]];
-        // this point's coordinates in the other body's tile, wrapped to [0, n); skip unless the point
-        // lies within rc of that tile
-        // tile coordinates of the other body's member cells (phi >= thr) lie in its box mbox (built by
-        // the refill pass after the last flag update); the offsets reach Rc cells per axis, so a point
-        // outside the box grown by Rc (periodically) finds no partner
-        const int* bx = mbox + MBOX_N * a.nbl[k];
-        int l[3];
-        bool near = true;
-        for (int d = 0; d < 3; ++d) {
-          l[d] = wrapi_near(g[d] - b.o[d], nn[d]);
-          const int lo = bx[d] - Rc, hi = bx[3 + d] + Rc;
-          const bool in = (l[d] >= lo && l[d] <= hi) || (l[d] - nn[d] >= lo && l[d] - nn[d] <= hi) ||
-                          (l[d] + nn[d] >= lo && l[d] + nn[d] <= hi);
-          if (bx[d] > bx[3 + d] || !in) near = false;  // an empty box has no members
-        }
-        if (!near) continue;
-        {
+    if (threadIdx.x < chunk && k < cells) {
+      const int l2 = (int)(k / w01), r = (int)(k - (unsigned)l2 * w01), l1 = r / w0, l0 = r - l1 * w0;
+      unsigned reach = 0;  // neighbours that the point may reach
+      if (dbits(arena[a.off + h0 + l0 + (long long)a.L[0] * (h1 + l1 + (long long)a.L[1] * (h2 + l2))]) >= tb) {
+        const TileCell c = tile_at(a, h0 + l0, h1 + l1, h2 + l2, lat);
+        const int g[3] = {c.gx, c.gy, c.gz}, nn[3] = {lat.nx, lat.ny, lat.nz};
+        for (int kb = 0; kb < a.nnb; ++kb) {
+          // tile coordinates of the other body's member cells (phi >= thr) lie in its box mbox (built by the
+          // flag pass); the offsets reach Rc cells per axis, so a point outside the box grown by Rc
+          // (periodically) finds no partner
+          const BodyDev& b = bodies[a.nbl[kb]];
+          const int* bx = mbox + MBOX_N * a.nbl[kb];
+          bool near = true;
+          for (int d = 0; d < 3; ++d) {
+            const int l = wrapi_near(g[d] - b.o[d], nn[d]), lo = bx[d] - Rc, hi = bx[3 + d] + Rc;
+            const bool in = (l >= lo && l <= hi) || (l - nn[d] >= lo && l - nn[d] <= hi) ||
+                            (l + nn[d] >= lo && l + nn[d] <= hi);
+            if (bx[d] > bx[3 + d] || !in) near = false;  // an empty box has no members
+          }
+          if (!near) continue;
           // and within B's member radius (plus rc and a cell) of B's centre
           float dx = (float)c.gx - b.Xf[0], dy = (float)c.gy - b.Xf[1], dz = (float)c.gz - b.Xf[2];
           dx -= (float)lat.nx * rintf(dx / (float)lat.nx);
           dy -= (float)lat.ny * rintf(dy / (float)lat.ny);
           dz -= (float)lat.nz * rintf(dz / (float)lat.nz);
           const float lim = sqrtf(__int_as_float(bx[MBOX_R2])) + (float)rc + 1.0f;
-          if (dx * dx + dy * dy + dz * dz > lim * lim) continue;
+          if (!(dx * dx + dy * dy + dz * dz > lim * lim)) reach |= 1u << kb;
         }
+      }
+      if (reach) {
+        const int at = atomicAdd(&n_list, 1);
+        list[at] = k;
+        reached[at] = reach;
+      }
+    }
+    __syncthreads();
+    const int n = n_list;
+    for (int e = warp; e < n; e += REP_T / 32) {
+      const unsigned q0 = list[e];
+      const int l2 = (int)(q0 / w01), r = (int)(q0 - (unsigned)l2 * w01), l1 = r / w0, l0 = r - l1 * w0;
+      const TileCell c = tile_at(a, h0 + l0, h1 + l1, h2 + l2, lat);
+      const int g[3] = {c.gx, c.gy, c.gz};
+      const int nn[3] = {lat.nx, lat.ny, lat.nz};
+      double f[3] = {0, 0, 0};
+      bool hit = false;
+      for (unsigned todo = reached[e]; todo; todo &= todo - 1) {
+        const BodyDev& b = bodies[a.nbl[__ffs(todo) - 1]];
+        int l[3];  // the point's coordinates in the other body's tile, wrapped to [0, n)
+        for (int d = 0; d < 3; ++d) l[d] = wrapi_near(g[d] - b.o[d], nn[d]);
         const double* bb = arena + b.off;
-        // offsets in groups of 8: the group's loads are issued before any of them is tested (a
-        // test per load would wait for each load in turn); contributions are added in offset order
-        for (int j0 = 0; j0 < c_noff; j0 += 8) {
-          double v[8];
-  #pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            const int j = j0 + u;
+        // a lane per offset; four loads are issued before any of them is tested
+        for (int j0 = 0; j0 < c_noff; j0 += 128) {
+          double v[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int j = j0 + 32 * u + lane;
             long long q = -1;
             if (j < c_noff) {
               int m[3];
@@ -556,31 +581,51 @@ __global__ void __launch_bounds__(256) k_repulsion(const __grid_constant__ TileS
             }
             v[u] = q >= 0 ? __ldg(bb + q) : 0.0;
           }
-  #pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            const int j = j0 + u;
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int j = j0 + 32 * u + lane;
             if (j >= c_noff || dbits(v[u]) < tb) continue;
-            F[0] += c_offf[3 * j];
-            F[1] += c_offf[3 * j + 1];
-            F[2] += c_offf[3 * j + 2];
-            has = true;
+            f[0] += c_offf[3 * j];
+            f[1] += c_offf[3 * j + 1];
+            f[2] += c_offf[3 * j + 2];
+            hit = true;
           }
         }
       }
-    }
-    if (__ballot_sync(0xffffffffu, has) == 0) continue;
-    double T[3] = {0, 0, 0};
-    if (has) {
-      const double arm[3] = {mimg(c.gx - a.X[0], lat.nx), mimg(c.gy - a.X[1], lat.ny), mimg(c.gz - a.X[2], lat.nz)};
-      xcross(arm, F, T);
-    }
-    for (int p = 0; p < 3; ++p) {
-      double sf = dwarp_sum(F[p]), st = dwarp_sum(T[p]);
-      if ((threadIdx.x & 31) == 0) {
-        if (sf != 0.0) atomicAdd(acc + (size_t)self * ACC_N + ACC_REP_F + p, sf);
-        if (st != 0.0) atomicAdd(acc + (size_t)self * ACC_N + ACC_REP_T + p, st);
+      if (!__any_sync(0xffffffffu, hit)) continue;
+      // the arm, an axis per lane
+      const int ax = min(lane, 2);
+      const double arm1 = mimg((double)g[ax] - a.X[ax], nn[ax]);
+      const double arm[3] = {__shfl_sync(0xffffffffu, arm1, 0), __shfl_sync(0xffffffffu, arm1, 1),
+                             __shfl_sync(0xffffffffu, arm1, 2)};
+      if (hit) {
+        double t[3];
+        xcross(arm, f, t);
+        for (int p = 0; p < 3; ++p) {
+          F[p] += f[p];
+          T[p] += t[p];
+        }
+        has = true;
       }
     }
+    __syncthreads();  // the list is written again
+  }
+  // block totals, then one atomic per component
+  if (!__syncthreads_or(has)) return;
+  __shared__ double sum[REP_T / 32][6];
+  for (int p = 0; p < 3; ++p) {
+    const double sf = dwarp_sum(F[p]), st = dwarp_sum(T[p]);
+    if (lane == 0) {
+      sum[warp][p] = sf;
+      sum[warp][3 + p] = st;
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < 6) {
+    double t = 0.0;
+    for (int w = 0; w < REP_T / 32; ++w) t += sum[w][threadIdx.x];
+    const int slot = threadIdx.x < 3 ? ACC_REP_F + threadIdx.x : ACC_REP_T + threadIdx.x - 3;
+    if (t != 0.0) atomicAdd(acc + (size_t)self * ACC_N + slot, t);
   }
 }
 
@@ -1369,8 +1414,8 @@ void launch_repulsion(const ChainLaunch& c, cudaStream_t s) {
   // a few waves in all. Only the points near a contact have work, and every block repeats the cull, so many
   // bodies get few blocks each (128 bodies of a batch: 140 us with a block for four chunks of the tile, 12 now)
   const dim3 g(std::min(tile, (unsigned)std::max(8, 4 * nsm / c.bodies)), 1, (unsigned)c.bodies);
-  if (c.sets) k_repulsion<true><<<g, 256, 0, s>>>(c.one, c.sets, c.items);
-  else k_repulsion<false><<<g, 256, 0, s>>>(c.one, nullptr, nullptr);
+  if (c.sets) k_repulsion<true><<<g, REP_T, 0, s>>>(c.one, c.sets, c.items);
+  else k_repulsion<false><<<g, REP_T, 0, s>>>(c.one, nullptr, nullptr);
 }
 void launch_bodies(const ChainLaunch& c, cudaStream_t s) {
   if (!c.bodies) return;

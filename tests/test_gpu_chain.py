@@ -61,6 +61,21 @@ def test_chain_follows_the_oracle(many, mpf, solid, member, still):
     assert g.info()["device_error"] & ~1 == 0
 
 
+@pytest.mark.parametrize("n,gap,member,rc", [(2, -1.0, 0.5, 3.0), (12, -3.0, 0.5, 3.0), (12, -3.0, 0.2, 4.5), (9, 0.5, 0.9, 2.0)])
+def test_repulsion_of_touching_spheres(n, gap, member, rc):
+    # pairs in reach of a contact, several neighbours at once, tables of one to four offsets per lane
+    w, _, _ = workloads.packing(seed=4, n_spheres=n, L=41, Rmin=5.0, Rmax=8.0, min_gap=gap, prec="fp64")
+    g, o = make_pair(w, options=dict(tile_tail=30.0), member_threshold=member, rc=rc)
+    for _ in range(2):
+        g.step(1)
+        o.step(1)
+        rep_g, rep_o = g.body_forces()[2][:, 2, :], o.body_forces()[2][:, 2, :]
+        scale = max(np.abs(rep_o).max(), 1e-300)
+        assert np.abs(rep_g - rep_o).max() < 1e-9 * scale
+        assert compare(g, o)["force"] < 1e-8
+    assert gap > 0 or np.abs(rep_o).max() > 0
+
+
 def _unlike():
     ws = [workloads.small_spheres(prec="fp32", nx=41, ny=37, nz=59, R=7.0),
           workloads.spheres2(seed=2, prec="fp32", nx=64, ny=64, nz=128, R=14.0),  # 2^19 cells: moment pass
