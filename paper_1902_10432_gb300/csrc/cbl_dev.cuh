@@ -160,6 +160,8 @@ struct PhysParams {
   // FP32 copies for the FP32 kernels, rounded once on the host (fill_float_params): a per-thread
   // double-to-float conversion is an FP64-pipe instruction, and GB300 issues FP64 at 1/64 rate
   float tau_f, G_f, rho0_f, ext_f[3];
+  double itau;   // 1 / tau, divided once on the host (the division is correctly rounded on both sides)
+  float itau_f;
 };
 
 // End of a step, by one block of T threads: the fluid mass (fixed-order sum of the collision's partials,
@@ -194,6 +196,8 @@ __device__ __forceinline__ void finish_step(double* mass_part, unsigned n_mass_p
 
 inline void fill_float_params(PhysParams& p) {
   p.tau_f = (float)p.tau;
+  p.itau = 1.0 / p.tau;
+  p.itau_f = 1.0f / p.tau_f;
   p.G_f = (float)p.G;
   p.rho0_f = (float)p.rho0;
   for (int k = 0; k < 3; ++k) p.ext_f[k] = (float)p.ext[k];

@@ -187,27 +187,46 @@ __device__ __forceinline__ R wgt(int i) {
   }
 }
 
+// c_i . (x, y, z): components -1, 0, 1 cost additions only (a product with a zero component is not removed
+// by the compiler, which has to keep 0 * inf)
+template <typename R>
+__device__ __forceinline__ R cdot(int i, R x, R y, R z) {
+  const int c[3] = {cx_of(i), cy_of(i), cz_of(i)};
+  const R v[3] = {x, y, z};
+  R r = 0;
+  bool set = false;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    if (!c[a]) continue;
+    const R t = c[a] > 0 ? v[a] : -v[a];
+    r = set ? r + t : t;
+    set = true;
+  }
+  return r;
+}
+
+// The even part is w_i (b + (c.v)(c.g)) with g = 4.5 (rho / tau) v + 9 (1 - 1/2tau) F and
+// b = (rho / tau)(1 - 1.5 v.v) - 3 (1 - 1/2tau) v.F, the odd part w_i c.p with p = 3 ((rho / tau) v + (1 - 1/2tau) F):
+// six to nine operations per pair of directions instead of 19. With the class sums of sc_force, one step (us,
+// split pass, tau = 1.1): FP64 128^3 1136 -> 973, D3Q27 1546 -> 1333; FP32 200^3 372 -> 368, D3Q27 537 -> 522;
+// binary16 353 -> 341, 488 -> 468.
 template <typename R, typename Sink>
-__device__ __forceinline__ void bgk_values(const R fi[Q], R rho, R vx, R vy, R vz, R Fx, R Fy, R Fz, R tau,
+__device__ __forceinline__ void bgk_values(const R fi[Q], R rho, R vx, R vy, R vz, R Fx, R Fy, R Fz, R itau,
                                            const Sink& sink) {
-  const R itau = (R)1 / tau;
   const R keep = (R)1 - itau;
   const R pref = (R)1 - (R)0.5 * itau;
   const R ro = rho * itau;
-  const R uu = vx * vx + vy * vy + vz * vz;
-  const R vF = vx * Fx + vy * Fy + vz * Fz;
-  const R base = (R)1 - (R)1.5 * uu;   // even part without (c.v)^2
-  const R fv = -(R)3 * pref * vF;       // even forcing part without (c.v)(c.F)
-  sink(0, keep * fi[0] + wgt<R>(0) * (ro * base + fv));
+  const R qx = ro * vx, qy = ro * vy, qz = ro * vz, hx = pref * Fx, hy = pref * Fy, hz = pref * Fz;
+  const R b = ro - ((R)1.5 * (vx * qx + vy * qy + vz * qz) + (R)3 * (vx * hx + vy * hy + vz * hz));
+  const R gx = (R)4.5 * qx + (R)9 * hx, gy = (R)4.5 * qy + (R)9 * hy, gz = (R)4.5 * qz + (R)9 * hz;
+  const R px = (R)3 * (qx + hx), py = (R)3 * (qy + hy), pz = (R)3 * (qz + hz);
+  sink(0, keep * fi[0] + wgt<R>(0) * b);
 #pragma unroll
   for (int i = 1; i < Q; i += 2) {
-    const R cu = (R)cx_of(i) * vx + (R)cy_of(i) * vy + (R)cz_of(i) * vz;
-    const R cF = (R)cx_of(i) * Fx + (R)cy_of(i) * Fy + (R)cz_of(i) * Fz;
-    const R w = wgt<R>(i);
-    const R sym = w * (ro * (base + (R)4.5 * cu * cu) + fv + (R)9 * pref * cu * cF);
-    const R anti = (R)3 * w * (ro * cu + pref * cF);
-    sink(i, keep * fi[i] + sym + anti);
-    sink(i + 1, keep * fi[i + 1] + sym - anti);
+    const R w = wgt<R>(i), wp = w * cdot<R>(i, px, py, pz);
+    const R sym = w * (b + cdot<R>(i, vx, vy, vz) * cdot<R>(i, gx, gy, gz));
+    sink(i, keep * fi[i] + sym + wp);
+    sink(i + 1, keep * fi[i + 1] + sym - wp);
   }
 }
 
@@ -218,15 +237,31 @@ __device__ __forceinline__ void collide_store(S* __restrict__ dst, size_t N, lon
                                               const typename St<S>::R fi[Q], typename St<S>::R rho,
                                               typename St<S>::R vx, typename St<S>::R vy, typename St<S>::R vz,
                                               typename St<S>::R Fx, typename St<S>::R Fy, typename St<S>::R Fz,
-                                              typename St<S>::R tau, typename St<S>::R* fo = nullptr) {
+                                              typename St<S>::R itau, typename St<S>::R* fo = nullptr) {
   using R = typename St<S>::R;
-  bgk_values<R>(fi, rho, vx, vy, vz, Fx, Fy, Fz, tau, [&](int i, R v) {
+  bgk_values<R>(fi, rho, vx, vy, vz, Fx, Fy, Fz, itau, [&](int i, R v) {
     St<S>::st(dst, (size_t)i * N + (size_t)n, i, v);
     if constexpr (OUT) fo[i] = St<S>::rt(v, i);
   });
 }
 
-template <typename S>
+// Cell of a thread of the kernels that take a plane of the lattice per blockIdx.z: blocks are tiles of the plane, or
+// (FLAT, gridDim.y = 1) 128 cells of it in a row.
+template <bool FLAT>
+__device__ __forceinline__ bool plane_cell(const Lat& lat, int& x, int& y) {
+  if constexpr (FLAT) {
+    const unsigned p = blockIdx.x * 128u + threadIdx.x;
+    y = (int)(p / (unsigned)lat.nx);
+    x = (int)(p - (unsigned)y * (unsigned)lat.nx);
+    return y < lat.ny;
+  } else {
+    x = blockIdx.x * blockDim.x + threadIdx.x;
+    y = blockIdx.y * blockDim.y + threadIdx.y;
+    return x < lat.nx && y < lat.ny;
+  }
+}
+
+template <typename S, bool FLAT = false>
 __global__ void __launch_bounds__(128) k_density(const S* __restrict__ fa, const S* __restrict__ fb,
                                                  const StepState* __restrict__ st,
                                                  const uint16_t* __restrict__ flags,
@@ -238,8 +273,9 @@ __global__ void __launch_bounds__(128) k_density(const S* __restrict__ fa, const
   const S* __restrict__ f = st->parity ? fb : fa;
   // two psi buffers (accumulating pass): the current step's is the one the parity names
   R* __restrict__ psi = (psi_b && st->parity) ? psi_b : psi_a;
-  const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y, z = blockIdx.z;
-  if (x >= lat.nx || y >= lat.ny) return;
+  int x, y;
+  const int z = blockIdx.z;
+  if (!plane_cell<FLAT>(lat, x, y)) return;
   const Cell c = make_cell(x, y, z, lat);
   const long long n = c.n;
   const uint16_t fl = flags[n];
@@ -354,14 +390,39 @@ struct CollideMinBlocks<__half> {
 template <typename R, typename PsiAt>
 __device__ __forceinline__ void sc_force(const PsiAt& psi_at, const PhysParams& pp, R& ps, R& Fx, R& Fy, R& Fz) {
   ps = psi_at(0);
-  R sx = 0, sy = 0, sz = 0;
+  R s3[3] = {0, 0, 0};
+  if constexpr (sizeof(R) == 8) {
+    // FP64: the weight of a class of directions (faces, edges, corners) multiplies the sum of its
+    // differences. FP32 is bound by its registers there, and keeps three sums only (with six, a step of
+    // 200^3 took 383 us instead of 368).
+    R f[3], e[3], k[3];
 #pragma unroll
-  for (int i = 1; i < Q; i += 2) {
-    const R wd = (R)w_of(i) * (psi_at(i) - psi_at(i + 1));
-    if (cx_of(i)) sx += wd * (R)cx_of(i);
-    if (cy_of(i)) sy += wd * (R)cy_of(i);
-    if (cz_of(i)) sz += wd * (R)cz_of(i);
+    for (int i = 1; i < Q; i += 2) {
+      const R d = psi_at(i) - psi_at(i + 1);
+      const int c[3] = {cx_of(i), cy_of(i), cz_of(i)};
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        R& s = i <= 6 ? f[a] : (i <= 18 ? e[a] : k[a]);
+        const bool first = i <= 6 || i == (a == 2 ? 11 : 7) || i == 19;  // of the class along this axis
+        if (c[a] > 0) s = first ? d : s + d;
+        if (c[a] < 0) s = first ? -d : s - d;
+      }
+    }
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      s3[a] = (R)w_of(1) * f[a] + (R)w_of(7) * e[a];
+      if constexpr (Q == 27) s3[a] += (R)w_of(Q - 1) * k[a];
+    }
+  } else {
+#pragma unroll
+    for (int i = 1; i < Q; i += 2) {
+      const R wd = (R)w_of(i) * (psi_at(i) - psi_at(i + 1));
+      if (cx_of(i)) s3[0] += wd * (R)cx_of(i);
+      if (cy_of(i)) s3[1] += wd * (R)cy_of(i);
+      if (cz_of(i)) s3[2] += wd * (R)cz_of(i);
+    }
   }
+  const R sx = s3[0], sy = s3[1], sz = s3[2];
   const R mG = -par<R>(pp.G, pp.G_f) * ps;
   Fx = mG * sx + par<R>(pp.ext[0], pp.ext_f[0]);
   Fy = mG * sy + par<R>(pp.ext[1], pp.ext_f[1]);
@@ -432,7 +493,7 @@ __device__ __forceinline__ typename St<S>::R collide_fluid(const S* __restrict__
     }
     R vx, vy, vz;
     fluid_velocity<R>(fi, rho, Fx, Fy, Fz, vx, vy, vz);
-    collide_store<S, OUT>(dst, N, n, fi, rho, vx, vy, vz, Fx, Fy, Fz, par<R>(pp.tau, pp.tau_f), fo);
+    collide_store<S, OUT>(dst, N, n, fi, rho, vx, vy, vz, Fx, Fy, Fz, par<R>(pp.itau, pp.itau_f), fo);
     if (diag) {
       diag_rho[n] = (double)rho;
       diag_vel[3 * n] = (double)vx;
@@ -527,7 +588,7 @@ __device__ __forceinline__ void add_mass_slot(double* __restrict__ mass_part, co
 
 // Bulk collision: solid cells store zeros, fluid cells without a solid neighbour collide; fluid cells
 // next to a solid are left to k_collide_near.
-template <typename S>
+template <typename S, bool FLAT = false>
 __global__ void __launch_bounds__(128, CollideMinBlocks<S>::value) k_collide(S* __restrict__ fa, S* __restrict__ fb,
                                                  const uint16_t* __restrict__ flags,
                                                  const typename St<S>::R* __restrict__ psi,
@@ -541,8 +602,9 @@ __global__ void __launch_bounds__(128, CollideMinBlocks<S>::value) k_collide(S* 
   const int diag = st->diag;
   const S* __restrict__ src = st->parity ? fb : fa;
   S* __restrict__ dst = st->parity ? fa : fb;
-  const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y, z = blockIdx.z;
-  const bool valid = x < lat.nx && y < lat.ny;
+  int x, y;
+  const int z = blockIdx.z;
+  const bool valid = plane_cell<FLAT>(lat, x, y);
   const Cell c = make_cell(valid ? x : 0, valid ? y : 0, z, lat);
   const long long n = c.n;
   R my_mass = 0;
@@ -1716,11 +1778,23 @@ static void lbm_step_t(const Lat& lat, S* fa, S* fb, const uint16_t* flags, void
   const int bx = blocks == 64 || blocks == 128 ? (int)blocks : 32, by = 128 / bx;
   const dim3 blk(bx, by, 1);
   const dim3 grid((lat.nx + bx - 1) / bx, (lat.ny + by - 1) / by, lat.nz);
-  if (phases & 1)
-    k_density<S><<<grid, blk, 0, s>>>(fa, fb, st, flags, bodies, (R*)psi, (R*)psi_b, lat, pp.rho0, pp.rho0_f);
-  if (phases & 2)
-    k_collide<S><<<grid, blk, 0, s>>>(fa, fb, flags, (const R*)psi, bodies, mass_part, st, diag_rho, diag_vel, lat,
-                                      pp, (RhoPsi<R>*)nbuf);
+  // Tiles that reach beyond the lattice leave lanes of their warps idle: from an eighth of them on, blocks take
+  // 128 cells of the plane in a row. us per step, tiles and rows: FP32 72^3 (33 % idle) 27 and 23, 100^3 (28 %)
+  // 62 and 54, 136^3 (18 %) 131 and 126; FP64 100^3 597 and 477. (90^3, 9 %: 39 with tiles.)
+  const bool flat = bx == 32 && 8LL * grid.x * bx * grid.y * by > 9LL * lat.nx * lat.ny;
+  const dim3 row((unsigned)(((long long)lat.nx * lat.ny + 127) / 128), 1, lat.nz);
+  if (phases & 1) {
+    if (flat) k_density<S, true><<<row, 128, 0, s>>>(fa, fb, st, flags, bodies, (R*)psi, (R*)psi_b, lat, pp.rho0, pp.rho0_f);
+    else k_density<S><<<grid, blk, 0, s>>>(fa, fb, st, flags, bodies, (R*)psi, (R*)psi_b, lat, pp.rho0, pp.rho0_f);
+  }
+  if (phases & 2) {
+    if (flat)
+      k_collide<S, true><<<row, 128, 0, s>>>(fa, fb, flags, (const R*)psi, bodies, mass_part, st, diag_rho, diag_vel, lat,
+                                             pp, (RhoPsi<R>*)nbuf);
+    else
+      k_collide<S><<<grid, blk, 0, s>>>(fa, fb, flags, (const R*)psi, bodies, mass_part, st, diag_rho, diag_vel, lat,
+                                        pp, (RhoPsi<R>*)nbuf);
+  }
   if ((phases & 4) && blist)
     k_collide_near<S><<<std::max(1, 2 * sm_count() / g_launch_share), 128, 0, s>>>(
         fa, fb, flags, (const R*)psi, (const R*)psi_b, bodies, mass_part, st, diag_rho, diag_vel, blist, lat, pp,
