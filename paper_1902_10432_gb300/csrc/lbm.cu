@@ -18,9 +18,10 @@
 //               the reaction of the Shan-Chen force (Sec. 3.2.3), summed in FP64.
 //  k_batch_lbm : the density and bulk collision of every instance of a batch in one persistent
 //               launch (work queue, bounded grid barrier).
-//  k_refill   : cover refill of nodes that became solid (Sec. 3.2.2), as a gather over each
-//               fluid node's 26 neighbours so that no two threads write the same populations; the
-//               same scan rebuilds the boundary-cell list for the next step.
+//  k_near_refill : boundary-cell list of the next step from the bodies' solid cells, and the cover refill
+//               of nodes that became solid (Sec. 3.2.2), each receiver written by one thread; it ends
+//               the step where no moment pass does.
+//  moments.cuh : the moment pass (tau = 1): the bulk fluid carried as density and momentum.
 //
 // Populations are SoA, f[i * N + n], in FP64, FP32 or binary16 deviations from the weights.
 //
@@ -205,28 +206,45 @@ __device__ __forceinline__ R cdot(int i, R x, R y, R z) {
   return r;
 }
 
-// The even part is w_i (b + (c.v)(c.g)) with g = 4.5 (rho / tau) v + 9 (1 - 1/2tau) F and
+// FP64 (bound by its pipe): the even part is w_i (b + (c.v)(c.g)) with g = 4.5 (rho / tau) v + 9 (1 - 1/2tau) F and
 // b = (rho / tau)(1 - 1.5 v.v) - 3 (1 - 1/2tau) v.F, the odd part w_i c.p with p = 3 ((rho / tau) v + (1 - 1/2tau) F):
-// six to nine operations per pair of directions instead of 19. With the class sums of sc_force, one step (us,
-// split pass, tau = 1.1): FP64 128^3 1136 -> 973, D3Q27 1546 -> 1333; FP32 200^3 372 -> 368, D3Q27 537 -> 522;
-// binary16 353 -> 341, 488 -> 468.
+// six to nine operations per pair of directions instead of 19. With the class sums of sc_force, one step at
+// tau = 1.1 (us, split pass): 128^3 1136 -> 973, D3Q27 1546 -> 1333. FP32 gains 1 to 3 % from it, but rounds
+// otherwise than the other FP32 passes and before; it keeps its terms.
 template <typename R, typename Sink>
 __device__ __forceinline__ void bgk_values(const R fi[Q], R rho, R vx, R vy, R vz, R Fx, R Fy, R Fz, R itau,
                                            const Sink& sink) {
   const R keep = (R)1 - itau;
   const R pref = (R)1 - (R)0.5 * itau;
   const R ro = rho * itau;
-  const R qx = ro * vx, qy = ro * vy, qz = ro * vz, hx = pref * Fx, hy = pref * Fy, hz = pref * Fz;
-  const R b = ro - ((R)1.5 * (vx * qx + vy * qy + vz * qz) + (R)3 * (vx * hx + vy * hy + vz * hz));
-  const R gx = (R)4.5 * qx + (R)9 * hx, gy = (R)4.5 * qy + (R)9 * hy, gz = (R)4.5 * qz + (R)9 * hz;
-  const R px = (R)3 * (qx + hx), py = (R)3 * (qy + hy), pz = (R)3 * (qz + hz);
-  sink(0, keep * fi[0] + wgt<R>(0) * b);
+  if constexpr (sizeof(R) == 8) {
+    const R qx = ro * vx, qy = ro * vy, qz = ro * vz, hx = pref * Fx, hy = pref * Fy, hz = pref * Fz;
+    const R b = ro - ((R)1.5 * (vx * qx + vy * qy + vz * qz) + (R)3 * (vx * hx + vy * hy + vz * hz));
+    const R gx = (R)4.5 * qx + (R)9 * hx, gy = (R)4.5 * qy + (R)9 * hy, gz = (R)4.5 * qz + (R)9 * hz;
+    const R px = (R)3 * (qx + hx), py = (R)3 * (qy + hy), pz = (R)3 * (qz + hz);
+    sink(0, keep * fi[0] + wgt<R>(0) * b);
 #pragma unroll
-  for (int i = 1; i < Q; i += 2) {
-    const R w = wgt<R>(i), wp = w * cdot<R>(i, px, py, pz);
-    const R sym = w * (b + cdot<R>(i, vx, vy, vz) * cdot<R>(i, gx, gy, gz));
-    sink(i, keep * fi[i] + sym + wp);
-    sink(i + 1, keep * fi[i + 1] + sym - wp);
+    for (int i = 1; i < Q; i += 2) {
+      const R w = wgt<R>(i), wp = w * cdot<R>(i, px, py, pz);
+      const R sym = w * (b + cdot<R>(i, vx, vy, vz) * cdot<R>(i, gx, gy, gz));
+      sink(i, keep * fi[i] + sym + wp);
+      sink(i + 1, keep * fi[i + 1] + sym - wp);
+    }
+  } else {
+    const R uu = vx * vx + vy * vy + vz * vz;
+    const R vF = vx * Fx + vy * Fy + vz * Fz;
+    const R base = (R)1 - (R)1.5 * uu;  // even part without (c.v)^2
+    const R fv = -(R)3 * pref * vF;     // even forcing part without (c.v)(c.F)
+    sink(0, keep * fi[0] + wgt<R>(0) * (ro * base + fv));
+#pragma unroll
+    for (int i = 1; i < Q; i += 2) {
+      const R cu = cdot<R>(i, vx, vy, vz), cF = cdot<R>(i, Fx, Fy, Fz);
+      const R w = wgt<R>(i);
+      const R sym = w * (ro * (base + (R)4.5 * cu * cu) + fv + (R)9 * pref * cu * cF);
+      const R anti = (R)3 * w * (ro * cu + pref * cF);
+      sink(i, keep * fi[i] + sym + anti);
+      sink(i + 1, keep * fi[i + 1] + sym - anti);
+    }
   }
 }
 
