@@ -59,11 +59,10 @@ def batch_kernels_per_step(variants):
 # ncu captures (gpu__time_duration, dram__bytes_read/write only), valid only for the source they were
 # taken on (source_hash of the lattice-Boltzmann sources); None otherwise
 PROFILED = {
-    ("tetra4", "fp32", 19, "e464e6a96e81"): 2722.1e6,      # k_collide<float>, mean of 15 launches
-    ("tetra4", "fp16dev", 19, "e464e6a96e81"): 1452.5e6,   # k_collide<__half>, mean of 10 launches
+    ("tetra4", "fp32", 19, "c13c15c92306"): 729.4e6,       # k_mom<float>, mean of 2 launches
 }
 PROFILED_STEP = {
-    ("tetra4", "fp32", 19, "e464e6a96e81"): 4199.6e6,      # every kernel of one step
+    ("tetra4", "fp32", 19, "c13c15c92306"): 867.7e6,       # every kernel of one step
 }
 
 

@@ -1485,10 +1485,36 @@ struct cbl_batch {
   ChainLaunch chain;
 };
 
+// The kernels of instance k on its own stream while they are captured; the batch's choice of pass holds.
+struct BatchBranch {
+  cbl_ctx* c;
+  cudaStream_t keep;
+  int keep_acc;
+  bool keep_mom;
+  BatchBranch(cbl_batch* b, size_t k) : c(b->ctxs[k]), keep(c->s), keep_acc(c->acc_pass), keep_mom(c->mom) {
+    c->s = b->branches[k];
+    c->acc_pass = 0;  // a batch runs these instances with the split pass (one psi buffer)
+    c->mom = b->mom[k];
+    cudaStreamWaitEvent(c->s, b->events[0], 0);
+  }
+  void join(cbl_batch* b, size_t k) {
+    cudaEventRecord(b->events[k + 1], c->s);
+    cudaStreamWaitEvent(b->s, b->events[k + 1], 0);
+  }
+  ~BatchBranch() {
+    c->s = keep;
+    c->acc_pass = keep_acc;
+    c->mom = keep_mom;
+  }
+};
+
 // Persistent mode: the bulk pass of every instance in one launch (or two, split and moment pass), then the
-// bodies' chain of every instance with one launch per kernel: a batch of 64 pairs of spheres has 13 launches
-// per step instead of 750 on 64 branches (7.5 ms per step; each is too short to fill the GPU and waits
-// for its turn).
+// bodies' chain. From BATCH_CHAIN_MIN instances on one launch per kernel serves all of them: a batch of 64
+// pairs of spheres has 14 launches per step instead of 750 on 64 branches (7.5 ms per step; each is too short to
+// fill the GPU and waits for its turn). Fewer instances do not fill the launches, whose latencies add up:
+// their chains run side by side on branches (us per step, one launch and branches: 4 pairs 571 and 505,
+// 6 pairs 790 and 759, 10 pairs 1093 and 1173).
+constexpr int BATCH_CHAIN_MIN = 8;
 static cudaError_t batch_enqueue(cbl_batch* b, int diag) {
   cbl_ctx* c0 = b->ctxs[0];
   const LbmOps& ops = c0->ops;
@@ -1503,7 +1529,18 @@ static cudaError_t batch_enqueue(cbl_batch* b, int diag) {
     if (e != cudaSuccess) return e;
   }
   const ChainLaunch& c = b->chain;
-  if (c.bodies) {
+  if (c.bodies && c.inst < BATCH_CHAIN_MIN) {
+    LaunchShare share(c.inst);
+    cudaEventRecord(b->events[0], s);
+    for (size_t k = 0; k < b->ctxs.size(); ++k) {
+      if (b->ctxs[k]->hb.empty()) continue;
+      BatchBranch br(b, k);
+      if (!br.c->mom) enqueue_lbm(br.c, 4, br.c->s);
+      enqueue_bodies(br.c, br.c->s);
+      enqueue_flags_refill(br.c, br.c->s);
+      br.join(b, k);
+    }
+  } else if (c.bodies) {
     if (b->n[0]) ops.batch_near(c0->prec, b->tab, b->n[0], s);
     ops.boundary(c0->prec, c, s);
     launch_repulsion(c, s);
@@ -1531,22 +1568,10 @@ static cudaError_t batch_capture(cbl_batch* b, int diag, cudaGraph_t* g) {
     LaunchShare share((int)std::min<size_t>(b->ctxs.size(), 64));
     cudaEventRecord(b->events[0], b->s);
     for (size_t k = 0; k < b->ctxs.size(); ++k) {
-      cbl_ctx* c = b->ctxs[k];
-      cudaStream_t br = b->branches[k];
-      cudaStreamWaitEvent(br, b->events[0], 0);
-      cudaStream_t keep = c->s;
-      const int keep_acc = c->acc_pass;
-      const bool keep_mom = c->mom;
-      c->s = br;
-      c->acc_pass = 0;  // a batch runs these instances with the split pass (one psi buffer)
-      c->mom = b->mom[k];
-      cudaMemsetAsync(&c->st->diag, diag, sizeof(int), br);
-      enqueue_step(c);
-      c->s = keep;
-      c->acc_pass = keep_acc;
-      c->mom = keep_mom;
-      cudaEventRecord(b->events[k + 1], br);
-      cudaStreamWaitEvent(b->s, b->events[k + 1], 0);
+      BatchBranch br(b, k);
+      cudaMemsetAsync(&br.c->st->diag, diag, sizeof(int), br.c->s);
+      enqueue_step(br.c);
+      br.join(b, k);
     }
   }
   cudaError_t e1 = cudaGetLastError();
@@ -1590,6 +1615,29 @@ static cbl_status batch_states(cbl_batch* b) {
   return CBL_OK;
 }
 
+// Planes per work item of the moment pass, at most the tile's: an item computes two more than it completes, the
+// blocks share them all out, and the last ones end half an item apart on average (as mom_sz). With 32 planes
+// whatever the batch, a step of two pairs took 442 us, of four 536; 266 and 410 so.
+static int batch_planes(const cbl_batch* b, const int tile[3]) {
+  int best = tile[2];
+  double best_cost = 1e300;
+  for (int sz = tile[2]; sz >= 4; --sz) {
+    double planes = 0;
+    for (size_t k = 0; k < b->ctxs.size(); ++k) {
+      if (!b->mom[k]) continue;
+      const Lat& l = b->ctxs[k]->lat;
+      const double cols = (double)((l.nx + tile[0] - 1) / tile[0]) * ((l.ny + tile[1] - 1) / tile[1]);
+      planes += cols * (l.nz + 2.0 * ((l.nz + sz - 1) / sz));
+    }
+    const double cost = planes / b->grid[1] + 0.5 * (sz + 2);
+    if (cost < best_cost) {
+      best_cost = cost;
+      best = sz;
+    }
+  }
+  return best;
+}
+
 // (re)build the instance table and both step graphs for the batch's mode and tile shape
 static cudaError_t batch_build(cbl_batch* b) {
   batch_drop_graphs(b);
@@ -1598,10 +1646,17 @@ static cudaError_t batch_build(cbl_batch* b) {
   if (b->mode == 1) {
     cbl_ctx* c0 = b->ctxs[0];
     std::vector<BatchInst> h;
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     for (int kind = 0; kind < 2; ++kind) {
       int t[3];
       c0->ops.batch_tile(b->tile_cfg, kind, t);
-      if (kind) b->sz = t[2];
+      b->grid[kind] = 0;
+      if (std::none_of(b->mom.begin(), b->mom.end(), [&](char m) { return (m != 0) == (kind == 1); })) continue;
+      b->grid[kind] = sms * (kind ? c0->ops.batch_mom_blocks_per_sm(c0->prec) : c0->ops.batch_blocks_per_sm(c0->prec, b->tile_cfg));
+      if (b->grid[kind] <= 0) return cudaErrorInvalidConfiguration;
+      if (kind) b->sz = t[2] = batch_planes(b, t);
       long long items = 0;
       for (size_t k = 0; k < b->ctxs.size(); ++k) {
         const cbl_ctx* c = b->ctxs[k];
@@ -1655,14 +1710,6 @@ static cudaError_t batch_build(cbl_batch* b) {
     if (e == cudaSuccess && ch.bodies)
       e = cudaMemcpy(b->items, items.data(), sizeof(int2) * items.size(), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return e;
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    for (int kind = 0; kind < 2; ++kind) {
-      if (!b->n[kind]) continue;
-      b->grid[kind] = sms * (kind ? c0->ops.batch_mom_blocks_per_sm(c0->prec) : c0->ops.batch_blocks_per_sm(c0->prec, b->tile_cfg));
-      if (b->grid[kind] <= 0) return cudaErrorInvalidConfiguration;
-    }
     BatchCtl ctl[2];
     std::memset(ctl, 0, sizeof(ctl));
     ctl[0].spin_limit = ctl[1].spin_limit = b->spin_limit;

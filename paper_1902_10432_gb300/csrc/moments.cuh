@@ -9,8 +9,8 @@
 // pulls 19 populations twice and stores them once.
 //
 // Where populations are still stored: the fluid cells next to a solid (F_NEAR: bounce-back, wall
-// terms, collided by k_collide_near before this pass) and every cell of the bricks (8 x 8 x 8 cells)
-// within 4 cells of one, which this pass stores beside the moments. k_mom_close pulls them at the end
+// terms, collided by k_collide_near before this pass) and every cell of the bricks (4 x 4 x 4 cells)
+// within 3 cells of one, which this pass stores beside the moments. k_mom_close pulls them at the end
 // of the step: psi of the next step's near cells, and the moments around every cell whose obstacle
 // flag changed (the refill rewrites populations there). A flag that changes where populations are
 // not stored (a body moving by cells in one step) makes k_mom_fill write all of them first; the same
@@ -390,11 +390,10 @@ __global__ void __launch_bounds__(MomTile<TY>::NT, MINB) k_mom(const MomArgs<S> 
 
 // The moment pass over a batch: one persistent launch (as k_batch_lbm: every block resident, work items
 // from a device queue, one bounded grid barrier). Phase 0: the cells next to a solid of every instance,
-// MOM_NEAR_ITEMS items each; phase 1: the columns, sz planes each. The instance's entry is copied to shared
+// near_items each; phase 1: the columns, sz planes each. The instance's entry is copied to shared
 // memory and phase 0 kept out of line: with the table read from global memory and both phases in one
 // body, 50 words spilled. 64 pairs of spheres, 54 M cells on this pass: 1812 us (k_mom's rate on
 // 256^3 would give 1000; the near cells, and box sides that are no multiple of 32, take the rest).
-constexpr int MOM_NEAR_ITEMS = 8;
 template <typename S>
 __device__ __noinline__ float batch_near_item(const BatchInst& I, unsigned k, unsigned n) {
   mom_reset(I.md, I.st->parity, k, n);
@@ -409,14 +408,16 @@ __global__ void __launch_bounds__(MomTile<TY>::NT, MINB)
   __shared__ BatchInst I;
   __shared__ long long s_item;
   __shared__ int s_inst;
+  // enough for the few thousand cells next to a pair of spheres, more where there are blocks to spare
+  const int near_items = min(max(8, (int)gridDim.x / ninst), 32);
   for (;;) {
     if (threadIdx.x == 0) s_item = (long long)atomicAdd(&ctl->queue[0], 1ull);
     __syncthreads();
     const long long item = s_item;
     __syncthreads();  // s_item is written again in the next round
-    if (item >= (long long)ninst * MOM_NEAR_ITEMS) break;
-    const BatchInst& J = tab[item / MOM_NEAR_ITEMS];
-    const float m = batch_near_item<S>(J, (unsigned)(item % MOM_NEAR_ITEMS) * NT + threadIdx.x, MOM_NEAR_ITEMS * NT);
+    if (item >= (long long)ninst * near_items) break;
+    const BatchInst& J = tab[item / near_items];
+    const float m = batch_near_item<S>(J, (unsigned)(item % near_items) * NT + threadIdx.x, near_items * NT);
     add_mass_slot(J.mass_part, m, (unsigned)item);
   }
   if (!grid_barrier(ctl)) return;
