@@ -59,10 +59,10 @@ def batch_kernels_per_step(variants):
 # ncu captures (gpu__time_duration, dram__bytes_read/write only), valid only for the source they were
 # taken on (source_hash of the lattice-Boltzmann sources); None otherwise
 PROFILED = {
-    ("tetra4", "fp32", 19, "c13c15c92306"): 729.4e6,       # k_mom<float>, mean of 2 launches
+    ("tetra4", "fp32", 19, "f516674d3bf5"): 729.4e6,       # k_mom<float>, mean of 2 launches
 }
 PROFILED_STEP = {
-    ("tetra4", "fp32", 19, "c13c15c92306"): 867.7e6,       # every kernel of one step
+    ("tetra4", "fp32", 19, "f516674d3bf5"): 867.7e6,       # every kernel of one step
 }
 
 

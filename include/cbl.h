@@ -316,7 +316,8 @@ cbl_status cbl_lbm_step_noalloc(const float* f_in, float* f_out, int nx, int ny,
  * cycles, default ~2 s): a block that waits longer sets an error word and returns, and
  * cbl_batch_sync then returns CBL_ERR_TIMEOUT (that step's results are not valid; the contexts stay
  * usable). The remaining work (the cells next to a solid, the bodies, the phase fields, flags and
- * refill) follows with one launch per kernel over all instances and bodies. Mode 0: one fork/join branch per instance with
+ * refill) follows with one launch per kernel over all instances and bodies; of fewer than eight
+ * instances, on a graph branch each. Mode 0: one fork/join branch per instance with
  * its whole step. The contexts must be initialised (cbl_init_fluid), live on the current device
  * and outlive the batch; while in a batch they must not be stepped on their own. `stream` (may be
  * NULL: the library creates one) orders the batch's work. The batch itself allocates its instance
@@ -330,7 +331,7 @@ cbl_status cbl_batch_step(cbl_batch* batch, int nsteps);
 cbl_status cbl_batch_sync(cbl_batch* batch);
 /* Batch options (synchronises, rebuilds the graphs): "mode" 0 or 1; "tile" 0..3, the persistent
  * kernel's tile of x * y * z cells: 32*4*1, 32*4*4 (default), 32*4*8, 64*2*4 (moment pass: columns of
- * 16, 32, 64 or 24 planes); "spin_limit" the
+ * at most 16, 32, 64 or 24 planes); "spin_limit" the
  * barrier wait limit in clock64 cycles (0 makes every wait run out at once: a test of the timeout
  * path). CBL_ERR_UNSUPPORTED for mode 1 over mixed precisions or velocity sets. */
 cbl_status cbl_batch_set_option(cbl_batch* batch, const char* key, double value);

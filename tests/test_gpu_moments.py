@@ -5,7 +5,7 @@ as density and momentum, their populations formed where they are pulled) against
 Both evaluate the same post-collision values from the same density, momentum and force, in another
 association, so they agree to rounding: FP32 within 2e-5 of the largest density and 20 times that of
 the largest velocity (the bounds of the accumulating pass), binary16 storage within its own rounding.
-Sides smaller than a block's column, sides that are no multiple of it or of the 8-cell bricks, and both
+Sides smaller than a block's column, sides that are no multiple of it or of the bricks, and both
 velocity sets cover the edges; free, held and thrown spheres the cells where populations are stored.
 """
 import os
