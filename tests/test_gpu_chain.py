@@ -88,17 +88,18 @@ def _unlike():
     return ws
 
 
-def test_unlike_instances_of_a_batch_step_as_alone():
+@pytest.mark.parametrize("copies", [1, 2])  # chains on branches (below eight instances), one launch per kernel
+def test_unlike_instances_of_a_batch_step_as_alone(copies):
     def sims():
         out = []
-        for w in _unlike():
+        for w in _unlike() * copies:
             s = cbl.Sim(w.nx, w.ny, w.nz, **w.params)
             workloads.build(s, w)
             out.append(s)
         return out
 
     alone, many = sims(), sims()
-    assert [s.get_option("lbm_variant") == 3 for s in alone] == [False, True, False, False, True]
+    assert [s.get_option("lbm_variant") == 3 for s in alone] == [False, True, False, False, True] * copies
     b = cbl.Batch(many)
     b.step(20)
     b.sync()
