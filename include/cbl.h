@@ -248,13 +248,14 @@ cbl_status cbl_kernel_times(cbl_ctx* ctx, int max, float* ms, int* count);
  *                  regions' edge cells from the populations of their outside sources and of the
  *                  bodies' tiles from the populations. Each step pulls the populations once. A
  *                  batch (cbl_batch_*) runs such instances with the split pass;
- *                  3 = moment pass (default at tau = 1 with FP32 or binary16 storage on 2^19 cells or
- *                  more; CBL_ERR_UNSUPPORTED at another tau or in FP64): at tau = 1 the post-collision
+ *                  3 = moment pass (default at tau = 1 with FP32 storage on 2^19 cells or more; also for
+ *                  binary16 storage; CBL_ERR_UNSUPPORTED at another tau or in FP64): at tau = 1 the post-collision
  *                  populations are functions of density, momentum and force, so the cells away from a
  *                  solid carry density and momentum (16 + 4 bytes per cell, two buffers, allocated at
  *                  the first step; without room for them the split pass runs) and populations are
  *                  stored next to the solids only. cbl_read_populations, cbl_save, cbl_move_bodies
- *                  write out all populations first; binary16 storage rounds as before;
+ *                  write out all populations first. In binary16 storage the variants 0 to 2 give the
+ *                  same bits and this one another sequence of roundings, as far from FP64 as theirs;
  *   "fused_ty"     y extent of a fused block's consumer tile: 4 or 8 (default);
  *   "fused_tz"     z extent of a fused block (0 = derived from the SM count);
  *   "acc_ty"       y extent of an accumulating region: 8 (default) or 16;

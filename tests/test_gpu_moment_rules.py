@@ -1,0 +1,44 @@
+"""Where the moment pass runs by default, and what a state on it gives to its readers right after a step."""
+import numpy as np
+import pytest
+
+from paper_1902_10432_gb300 import autotune, cbl, workloads
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import __graft_entry__
+    import torch
+
+    __graft_entry__.build()
+    assert torch.cuda.is_available()
+
+
+def _sim(w, variant=None, **kw):
+    s = cbl.Sim(w.nx, w.ny, w.nz, **dict(w.params, **kw))
+    if variant is not None:
+        s.set_option("lbm_variant", variant)
+    workloads.build(s, w)
+    return s
+
+
+def test_binary16_default_gives_the_bits_of_the_other_passes():
+    # 2^19 cells, held bodies (no order of FP64 sums in the result); the first rounding that differs is carried on
+    # by the flow, so 60 steps and equality
+    w = workloads.spheres2(seed=2, prec="fp16dev", nx=64, ny=64, nz=128, R=14.0)
+    for b in w.bodies:
+        b["fixed"] = True
+    a, b = _sim(w), _sim(w, 0)
+    assert a.get_option("lbm_variant") == 0
+    batch = cbl.Batch([_sim(w) for _ in range(2)])
+    for s in (a, b, batch):
+        s.step(60)
+    batch.sync()
+    for s in [a] + batch.sims:
+        assert np.array_equal(s.populations(), b.populations())
+        assert np.array_equal(s.fields()[1], b.fields()[1])
+    batch.close()
+    assert all(c["lbm_variant"] != 3 for c in autotune.candidates("fp16dev"))
+    assert _sim(workloads.spheres2(seed=2, prec="fp32", nx=64, ny=64, nz=128, R=14.0)).get_option("lbm_variant") == 3
