@@ -1533,6 +1533,7 @@ static cudaError_t batch_enqueue(cbl_batch* b, int diag) {
     if (e != cudaSuccess) return e;
   }
   const ChainLaunch& c = b->chain;
+  bool closed = false;  // k_batch_close ends the step of every instance on the moment pass, with bodies or without
   if (c.bodies && c.inst < BATCH_CHAIN_MIN) {
     LaunchShare share(c.inst);
     cudaEventRecord(b->events[0], s);
@@ -1555,9 +1556,12 @@ static cudaError_t batch_enqueue(cbl_batch* b, int diag) {
     if (b->n[1]) ops.batch_fill(c0->prec, mom, b->n[1], s);
     ops.near_refill(c0->prec, c, 1, s);
     if (b->n[1]) ops.batch_close(c0->prec, mom, b->n[1], s);
+    closed = true;
   }
-  for (size_t k = 0; k < b->ctxs.size(); ++k)
-    if (b->ctxs[k]->hb.empty()) launch_finish(b->ctxs[k]->mass_part, b->ctxs[k]->n_mass_part, b->ctxs[k]->st, b->ctxs[k]->cs, s);
+  for (size_t k = 0; k < b->ctxs.size(); ++k) {
+    cbl_ctx* x = b->ctxs[k];
+    if (x->hb.empty() && !(closed && b->mom[k])) launch_finish(x->mass_part, x->n_mass_part, x->st, x->cs, s);
+  }
   return cudaSuccess;
 }
 

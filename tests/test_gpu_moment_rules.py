@@ -42,3 +42,33 @@ def test_binary16_default_gives_the_bits_of_the_other_passes():
     batch.close()
     assert all(c["lbm_variant"] != 3 for c in autotune.candidates("fp16dev"))
     assert _sim(workloads.spheres2(seed=2, prec="fp32", nx=64, ny=64, nz=128, R=14.0)).get_option("lbm_variant") == 3
+
+
+@pytest.mark.parametrize("copies", [1, 3])  # chains on branches (below eight instances), one launch per kernel
+def test_instances_without_bodies_beside_those_with(copies):
+    # a fluid without bodies on each pass beside pairs of spheres: every instance ends its step once
+    def sims():
+        ws = []
+        for k in range(copies):
+            ws += [workloads.spheres2(seed=2, prec="fp32", nx=64, ny=64, nz=128, R=14.0),
+                   workloads.spheres2(seed=3, prec="fp32", nx=64, ny=64, nz=128, R=14.0),
+                   workloads.small_spheres(prec="fp32")]
+            ws[-2].bodies = []
+            if k == 1:
+                ws[-1].bodies = []
+        return [_sim(w) for w in ws]
+
+    alone, many = sims(), sims()
+    assert {(s.nb == 0, s.get_option("lbm_variant")) for s in alone} >= {(True, 3), (False, 3), (False, 0)}
+    b = cbl.Batch(many)
+    b.step(7)
+    b.step(4)
+    b.sync()
+    for a, m in zip(alone, many):
+        a.step(11)
+        # the same kernels: equal up to the order of FP64 sums (the bounds of the batch of unlike instances)
+        for x, y in zip(a.fields()[:2], m.fields()[:2]):
+            assert np.abs(x - y).max() < 4e-4 * np.abs(x).max()
+        assert np.abs(a.populations() - m.populations()).max() < 2e-5 * np.abs(a.populations()).max()
+        assert abs(a.total_mass() - m.total_mass()) < 1e-6 * a.total_mass()
+    b.close()
