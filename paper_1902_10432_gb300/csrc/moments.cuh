@@ -602,6 +602,13 @@ __device__ __forceinline__ void mom_close(S* fa, S* fb, StepState* __restrict__ 
     }
   }
   if (!next) return;
+  // After a fill in this step every population of it is stored, and what the refill added and what was zeroed above
+  // is in the populations alone: a fill between steps must leave them. (Nothing reads this map any more but
+  // such a fill; the next step's start empties it.)
+  if (cs->full) {
+    unsigned char* const map = md.map(t ^ 1);
+    for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < md.bricks(); k += gridDim.x * blockDim.x) map[k] = 1;
+  }
   __shared__ int s_last;
   __syncthreads();
   if (threadIdx.x == 0) {
