@@ -1451,12 +1451,13 @@ __global__ void k_init_fluid(S* __restrict__ f, const uint16_t* __restrict__ fla
 // ---- cover refill and boundary list ------------------------------------------------------------
 // After the new flags. Over the bodies' tiles: the fluid neighbours of a body's solid cells along a lattice
 // direction are the cells next to a solid; whoever sets a cell's bit first puts it into the boundary
-// list of the next step (collected per block, so that the list's runs belong to one body). Outside a step
-// (next = 0) the pass also makes the bodies' member records (k_flags does in a step, where X is final before
-// it). Over this step's flag changes: a covered
-// node n hands f_eq(rho_n, u_n) / |N_F(n)| to its fluid neighbours (face neighbours; all 26 if n has no
-// fluid face neighbour), gathered by the receivers, each by the first of its covered neighbours, so that
-// no two threads write the same populations. The blocks share the changes out over the whole launch.
+// list of the next step (collected per block, so that the list's runs belong to one body). What the clamp
+// of the phase field sets to 0 is set here, each body's own (k_flags, whose blocks look at all fields, leaves
+// it). Outside a step (next = 0) the pass also makes the bodies' member records (k_flags does in a step, where
+// X is final before it). Over this step's flag changes: a covered node n hands f_eq(rho_n, u_n) / |N_F(n)| to
+// its fluid neighbours (face neighbours; all 26 if n has no fluid face neighbour), gathered by the receivers,
+// each by the first of its covered neighbours, so that no two threads write the same populations. The blocks
+// share the changes out over the whole launch.
 // Only cells with phi > 0 are looked at (a third of a sphere's tile), and only the solid ones' neighbours;
 // testing the 18 neighbours of every fluid tile cell took 40 us on the four-sphere cluster, this 25.
 constexpr int NEAR_CAP = 2048;
@@ -1574,7 +1575,7 @@ __global__ void __launch_bounds__(TILE_T) k_near_refill(const __grid_constant__ 
   const unsigned plane = (unsigned)L0 * L1, p0 = blockIdx.x * TILE_T, p = p0 + threadIdx.x;
   if (z0 < L2 && p0 < plane) {
     const int i1 = (int)(p / (unsigned)L0), i0 = (int)(p - (unsigned)i1 * L0);
-    const double* const phi = C.arena + b.off;
+    double* const phi = C.arena + b.off;
     const long long thr = dbits(C.member_thr);
     bool any = false;
     int lz = INT_MAX, hz = INT_MIN;
@@ -1582,7 +1583,11 @@ __global__ void __launch_bounds__(TILE_T) k_near_refill(const __grid_constant__ 
 #pragma unroll
     for (int q = 0; q < Z; ++q) {
       const bool in = p < plane && z0 + q < L2;
-      const long long vb = in ? dbits(phi[p + (size_t)plane * (z0 + q)]) : 0;
+      long long vb = in ? dbits(phi[p + (size_t)plane * (z0 + q)]) : 0;
+      if (vb != 0 && phi_clamp(vb) == 0) {  // (k_flags leaves these)
+        phi[p + (size_t)plane * (z0 + q)] = 0.0;
+        vb = 0;
+      }
       bool solid = false;
       const bool member = !next && in && vb >= thr;
       if (vb > 0 || member) {

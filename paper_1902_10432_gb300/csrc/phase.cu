@@ -97,7 +97,7 @@ __global__ void k_rasterize(BodyDev* bodies, double* arena, Lat lat, double eta)
   double d = body_sdf(b, r);
   double v = d <= -0.5 * eta ? 1.0 : (d >= 0.5 * eta ? 0.0 : 0.5 - 0.5 * sin(PI * d / eta));
   double* buf = arena + b.off;
-  buf[t] = v;
+  buf[t] = __longlong_as_double(phi_clamp(dbits(v)));
   buf[b.sz + t] = 0.0;
   buf[2 * b.sz + t] = 0.0;
 }
@@ -150,10 +150,9 @@ __device__ __noinline__ void flag_event(const TileSet& S, const TileCell& c, lon
   if (!all) S.cs->full = 1;
 }
 
-// New obstacle flag of a cell; the near-solid bit is rebuilt by the pass that follows. Two bodies may both
-// take a cell for theirs to write where one flushes a vanishing phase while the other looks (below);
-// they decide alike, and the exchange lets only one of them count the cell as covered. The cover bit
-// stays until the body update of the next step clears it (its users come after this pass).
+// New obstacle flag of a cell; the near-solid bit is rebuilt by the pass that follows (the exchange keeps the
+// solid cell's word whole while another block clears that bit). The cover bit stays until the body update of
+// the next step clears it (its users come after this pass).
 __device__ __forceinline__ void set_flag(const TileSet& S, const TileCell& c, bool solid, int owner, int init) {
   const long long n = lat_index(c, S.lat);
   uint16_t old = S.flags[n];
@@ -178,12 +177,15 @@ __device__ __forceinline__ void set_flag(const TileSet& S, const TileCell& c, bo
 
 // Clamp to [0, 1], renormalise the solid sum, obstacle flag (fluid phase below the threshold, Sec. 3.2.2) and
 // owner (the largest phase, ties to the lower id), cover events. A cell is written by one body: the one
-// whose phase field is not zero there, the lowest of them where several are not. A cell whose field
-// has gone to zero under its owner in this step (a body moving by cells) is written by the owner, or
-// by any body whose tile holds it if the owner's has left it. The cells with phi >= the membership threshold
-// make up the body's member record (tile-coordinate box and largest squared distance from X, a bound: the
-// fields may still be rescaled) for the repulsion of the next step. The blocks also clear the near-solid bits
-// of the old boundary list (atomically: a neighbouring half word may be written meanwhile).
+// whose phase field is not zero there, the lowest of them where several are not. All bodies' blocks run at
+// once and look at each other's fields, so this kernel makes no value zero: what the clamp sets to 0 counts
+// as 0 here and is set by the pass that follows (k_near_refill), each body's own. (What is rescaled to a
+// sum of 1 stays above 1e-14.) A cell whose field has gone to zero under its owner in this step (a body
+// moving by cells) is written by the owner, or by any body whose tile holds it if the owner's has left it,
+// by all alike. The cells with phi >= the membership threshold make up the body's member record (tile-coordinate
+// box and largest squared distance from X, a bound: the fields may still be rescaled) for the repulsion of
+// the next step. The blocks also clear the near-solid bits of the old boundary list (atomically: a
+// neighbouring half word may be written meanwhile).
 template <bool B, int Z>
 __global__ void __launch_bounds__(TILE_T) k_flags(const __grid_constant__ TileSet one, const TileSet* __restrict__ sets,
                                                   const int2* __restrict__ items, int init) {
@@ -286,19 +288,17 @@ __global__ void __launch_bounds__(TILE_T) k_flags(const __grid_constant__ TileSe
     if (thr > 1.0 && dbits(*p0) == 0 && (m > 1 || covered_by_lower_body(S.bodies, b, self, c.gx, c.gy, c.gz, lat))) continue;
     double S1 = 0.0;
     for (int k = 0; k < m; ++k) {
-      // the clamp on bit patterns (a NaN goes to 0, as by fmax)
-      const long long old = dbits(*ptr[k]), inf = 0x7FF0000000000000LL;
-      long long vb = old;
-      if (old < dbits(PHI_EPS) || old > inf) vb = 0;
-      else if (old > dbits(1.0 - PHI_EPS)) vb = dbits(1.0);
+      const long long old = dbits(*ptr[k]), vb = phi_clamp(old);
       const double v = __longlong_as_double(vb);
-      if (vb != old) *ptr[k] = v;
+      if (vb != old && vb != 0) *ptr[k] = v;  // 1
       S1 = k ? S1 + v : v;
     }
     if (m > 1 && S1 > 1.0) {
       double S2 = 0.0;
       for (int k = 0; k < m; ++k) {
-        const double v = *ptr[k] / S1;
+        const long long vb = phi_clamp(dbits(*ptr[k]));
+        if (vb == 0) continue;
+        const double v = __longlong_as_double(vb) / S1;
         *ptr[k] = v;
         S2 += v;
       }
@@ -311,7 +311,7 @@ __global__ void __launch_bounds__(TILE_T) k_flags(const __grid_constant__ TileSe
     else solid = 1.0 - S1 < thr;
     int best = ids[0];
     if (solid && m > 1) {
-      double bv = *ptr[0];
+      double bv = __longlong_as_double(phi_clamp(dbits(*ptr[0])));
       for (int k = 1; k < m; ++k)
         if (*ptr[k] > bv) {
           bv = *ptr[k];

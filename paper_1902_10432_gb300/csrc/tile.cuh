@@ -11,6 +11,12 @@ namespace cbl {
 // last bit of a rounding, and keeps the support of a moving field compact.
 constexpr double PHI_EPS = 1e-12;
 
+// the clamp, on bit patterns (a NaN goes to 0, as by fmax)
+__device__ __forceinline__ long long phi_clamp(long long b) {
+  if (b < dbits(PHI_EPS) || b > 0x7FF0000000000000LL) return 0;
+  return b > dbits(1.0 - PHI_EPS) ? dbits(1.0) : b;
+}
+
 // Launch geometry of the tile kernels: block (x, y, z) takes cells [256 x, 256 x + 256) of the tile's
 // planes Z y .. Z y + Z - 1 of body z. One division per thread gives its column (a flat cell index needs
 // three), and what depends on the column is computed once for Z cells. Most cells of a tile need nothing
