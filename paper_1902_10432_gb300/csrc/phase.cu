@@ -902,7 +902,7 @@ __global__ void __launch_bounds__(TILE_T) k_sweep(const __grid_constant__ TileSe
     }
     still &= sh[a] == 0 && (dbits(b.V[a]) << 1) == 0 && (dbits(b.W[a]) << 1) == 0;
   }
-  if (still && !(D == 0 && S.mpf)) return;
+  if (still && D != 0) return;
   __shared__ TileList list;
   if (threadIdx.x == 0) list.n = 0;
   __syncthreads();
@@ -917,6 +917,10 @@ __global__ void __launch_bounds__(TILE_T) k_sweep(const __grid_constant__ TileSe
   long long frac = 0;
   int ones = 0, shell = 0;
   bool halo = false;
+  auto outer = [&](int c0, int c1, int c2) {
+    return (L0 < nn[0] && (c0 < 2 || c0 >= L0 - 2)) || (L1 < nn[1] && (c1 < 2 || c1 >= L1 - 2)) ||
+           (L2 < nn[2] && (c2 < 2 || c2 >= L2 - 2));
+  };
   auto tally = [&](double v, int c0, int c1, int c2) {
     const long long vb = dbits(v);
     if ((vb << 1) == 0) return;
@@ -936,17 +940,17 @@ __global__ void __launch_bounds__(TILE_T) k_sweep(const __grid_constant__ TileSe
     // the outer two layers must stay empty (they are the stencil halo); a moving body's upwind
     // scheme leaves a geometrically decaying tail ahead of its front, and the tile drops what
     // reaches past it, so values of at most PHI_EPS there are tolerated
-    if (LAST && (vb << 1) > (dbits(PHI_EPS) << 1))
-      halo |= (L0 < nn[0] && (c0 < 2 || c0 >= L0 - 2)) || (L1 < nn[1] && (c1 < 2 || c1 >= L1 - 2)) ||
-              (L2 < nn[2] && (c2 < 2 || c2 >= L2 - 2));
+    if ((vb << 1) > (dbits(PHI_EPS) << 1))
+      halo |= outer(c0, c1, c2);
   };
   if (still) {
+    // (without kinetics only the halo is looked at: a field that a move or a turn has put there)
 #pragma unroll
     for (int q = 0; q < Z; ++q)
-      if (pt < plane && z0 + q < L2) {
+      if (pt < plane && z0 + q < L2 && (S.mpf || outer(i0, i1, z0 + q))) {
         const size_t t = pt + (size_t)plane * (z0 + q);
         const double v = in[t];
-        out[t] = v;
+        if (S.mpf) out[t] = v;
         tally(v, i0, i1, z0 + q);
       }
   } else {
