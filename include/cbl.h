@@ -318,7 +318,7 @@ cbl_status cbl_lbm_step_noalloc(const float* f_in, float* f_out, int nx, int ny,
  * cbl_batch_sync then returns CBL_ERR_TIMEOUT (that step's results are not valid; the contexts stay
  * usable). The remaining work (the cells next to a solid, the bodies, the phase fields, flags and
  * refill) follows with one launch per kernel over all instances and bodies; of fewer than eight
- * instances, on a graph branch each. Mode 0: one fork/join branch per instance with
+ * instances, or with more than 65535 bodies in all, on a graph branch each. Mode 0: one fork/join branch per instance with
  * its whole step. The contexts must be initialised (cbl_init_fluid), live on the current device
  * and outlive the batch; while in a batch they must not be stepped on their own. `stream` (may be
  * NULL: the library creates one) orders the batch's work. The batch itself allocates its instance

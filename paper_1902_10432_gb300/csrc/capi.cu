@@ -1518,7 +1518,8 @@ struct BatchBranch {
 // fill the GPU and waits for its turn). Fewer instances do not fill the launches, whose latencies add up:
 // their chains run side by side on branches (us per step, one launch and branches: 4 pairs 571 and 505,
 // 6 pairs 790 and 759, 10 pairs 1093 and 1173).
-constexpr int BATCH_CHAIN_MIN = 8;
+// So do more bodies than a launch's grid numbers in z.
+constexpr int BATCH_CHAIN_MIN = 8, BATCH_CHAIN_BODIES = 65535;
 static cudaError_t batch_enqueue(cbl_batch* b, int diag) {
   cbl_ctx* c0 = b->ctxs[0];
   const LbmOps& ops = c0->ops;
@@ -1534,7 +1535,7 @@ static cudaError_t batch_enqueue(cbl_batch* b, int diag) {
   }
   const ChainLaunch& c = b->chain;
   bool closed = false;  // k_batch_close ends the step of every instance on the moment pass, with bodies or without
-  if (c.bodies && c.inst < BATCH_CHAIN_MIN) {
+  if (c.bodies && (c.inst < BATCH_CHAIN_MIN || c.bodies > BATCH_CHAIN_BODIES)) {
     LaunchShare share(c.inst);
     cudaEventRecord(b->events[0], s);
     for (size_t k = 0; k < b->ctxs.size(); ++k) {
