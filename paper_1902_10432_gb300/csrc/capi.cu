@@ -1662,6 +1662,7 @@ static cudaError_t batch_build(cbl_batch* b) {
       int t[3];
       c0->ops.batch_tile(b->tile_cfg, kind, t);
       b->grid[kind] = 0;
+      b->items_n[kind] = 0;
       if (std::none_of(b->mom.begin(), b->mom.end(), [&](char m) { return (m != 0) == (kind == 1); })) continue;
       b->grid[kind] = sms * (kind ? c0->ops.batch_mom_blocks_per_sm(c0->prec) : c0->ops.batch_blocks_per_sm(c0->prec, b->tile_cfg));
       if (b->grid[kind] <= 0) return cudaErrorInvalidConfiguration;

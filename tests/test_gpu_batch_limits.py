@@ -41,3 +41,27 @@ def test_more_bodies_than_a_grid_numbers():
         assert np.allclose(s.body_forces()[0], F, rtol=1e-9, atol=1e-12)
         assert np.abs(s.fields()[0] - alone.fields()[0]).max() < 2e-5
     b.close()
+
+
+def test_work_items_follow_the_passes():
+    # the instances change from the moment to the split pass: the items are those of the split pass alone
+    def sims(variant):
+        out = []
+        for _ in range(2):
+            s = cbl.Sim(96, 64, 96, prec="fp32")
+            s.set_option("lbm_variant", variant)
+            s.init_fluid(1.9, 0.12)
+            out.append(s)
+        return out
+
+    split, mom = cbl.Batch(sims(0)), sims(3)
+    changed = cbl.Batch(mom)
+    assert changed.info() != split.info()
+    for s in mom:
+        s.set_option("lbm_variant", 0)
+    changed.set_option("tile", 1)
+    assert changed.info() == split.info()
+    changed.step(3)
+    changed.sync()
+    for b in (changed, split):
+        b.close()
