@@ -252,7 +252,9 @@ cbl_status cbl_kernel_times(cbl_ctx* ctx, int max, float* ms, int* count);
  *                  binary16 storage; CBL_ERR_UNSUPPORTED at another tau or in FP64): at tau = 1 the post-collision
  *                  populations are functions of density, momentum and force, so the cells away from a
  *                  solid carry density and momentum (16 + 4 bytes per cell, two buffers, allocated at
- *                  the first step; without room for them the split pass runs) and populations are
+ *                  the first step; without room for them the split pass runs, and they are asked for again
+ *                  after some calls; setting another variant gives them back, unless a batch holds
+ *                  the context) and populations are
  *                  stored next to the solids only. cbl_read_populations, cbl_save, cbl_move_bodies
  *                  write out all populations first. In binary16 storage the variants 0 to 2 give the
  *                  same bits and this one another sequence of roundings, as far from FP64 as theirs;

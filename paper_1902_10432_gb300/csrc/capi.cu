@@ -6,6 +6,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -72,6 +73,9 @@ struct cbl_ctx {
   bool mom = false;        // the step graph runs the moment pass
   bool mom_state = false;  // the state is in moments (populations complete only after mom_leave)
   int mom_sz = 0;          // planes per block
+  int mom_wait = 0, mom_skip = 0;  // no room for its buffers: calls until they are asked for again, and those left
+  // batches that hold this context: their graphs use its buffers (shared with them, as a context may go first)
+  std::shared_ptr<int> batches = std::make_shared<int>(0);
   MomDev md = {};
   ChainState* cs = nullptr;
   int* events = nullptr;  // cells whose obstacle flag changed in a flag update (capacity: the tiles)
@@ -698,10 +702,37 @@ static void drop_graph(cbl_ctx* ctx) {
   ctx->graph = nullptr;
 }
 
-// Before a step: the moment pass's buffers (without room for them the step stays with the split pass)
-// and, where the state is in populations, the moments.
+// The moment pass's buffers given back, the state in populations. A batch's graphs keep theirs.
+static cbl_status mom_free(cbl_ctx* ctx) {
+  if (!ctx->md.M0 || *ctx->batches) return CBL_OK;
+  const cbl_status st = mom_leave(ctx, false);
+  if (st != CBL_OK) return st;
+  drop_graph(ctx);
+  CK(cudaStreamSynchronize(ctx->s));
+  // (psi2 belongs to the accumulating pass too)
+  void* const own[] = {ctx->md.M0, ctx->md.M1, ctx->md.map0, ctx->rhop ? nullptr : ctx->psi2};
+  for (void* p : own) {
+    const auto at = std::find(ctx->allocs.begin(), ctx->allocs.end(), p);
+    if (!p || at == ctx->allocs.end()) continue;
+    if (ctx->user_alloc) ctx->alloc.free(p, ctx->alloc.user);
+    else cudaFree(p);
+    ctx->allocs.erase(at);
+  }
+  if (!ctx->rhop) ctx->psi2 = nullptr;
+  ctx->md = MomDev{};
+  ctx->mom = false;
+  return CBL_OK;
+}
+
+// Before a step: the moment pass's buffers (without room for them the step stays with the split pass, and
+// they are asked for again after 16 calls, then 32, up to 1024) and, where the state is in populations,
+// the moments.
 static cbl_status mom_prepare(cbl_ctx* ctx) {
   bool use = mom_rule(ctx);
+  if (use && !ctx->md.M0 && ctx->mom_skip > 0) {
+    --ctx->mom_skip;
+    use = false;
+  }
   if (use && !ctx->md.M0) {
     const size_t N = (size_t)ctx->lat.N;
     MomDev& d = ctx->md;
@@ -725,11 +756,12 @@ static cbl_status mom_prepare(cbl_ctx* ctx) {
       ctx->allocs.resize(mark);
       cudaGetLastError();
       d = MomDev{};
-      ctx->mom_req = 0;
+      ctx->mom_skip = ctx->mom_wait = std::min(1024, std::max(16, 2 * ctx->mom_wait));
       use = false;
     } else {
       d.map0 = small;
       d.map1 = d.map0 + bricks;
+      ctx->mom_wait = 0;
       ctx->mom_sz = ctx->ops.mom_sz(ctx->lat, 1);
       CK(ctx->ops.mom(ctx->prec, ctx->lat, ctx->fa, ctx->fb, ctx->flags, ctx->psi, ctx->psi2, d, ctx->mass_part, ctx->st,
                       ctx->diag_rho, ctx->diag_vel, ctx->pp, 0, ctx->s));
@@ -1378,7 +1410,7 @@ cbl_status cbl_info(cbl_ctx* ctx, int* nbodies, int64_t* ncells, int* device_err
 cbl_status cbl_get_option(cbl_ctx* ctx, const char* key, double* value) {
   if (!ctx || !key || !value) return fail(ctx, CBL_ERR_ARG, "NULL argument");
   const std::string k(key);
-  if (k == "lbm_variant") *value = ctx->acc_pass ? 2 : (ctx->fused_tz ? 1 : (mom_rule(ctx) ? 3 : 0));
+  if (k == "lbm_variant") *value = ctx->acc_pass ? 2 : (ctx->fused_tz ? 1 : (mom_rule(ctx) && (ctx->md.M0 || !ctx->mom_wait) ? 3 : 0));
   else if (k == "acc_ty") *value = ctx->acc_ty;
   else if (k == "acc_sz") *value = ctx->acc_sz_req > 0 ? ctx->acc_sz_req : ctx->ops.acc_sz(ctx->lat, ctx->prec, ctx->acc_ty, 2);
   else if (k == "fused_ty") *value = ctx->fused_ty;
@@ -1405,9 +1437,14 @@ cbl_status cbl_set_option(cbl_ctx* ctx, const char* key, double value) {
     if (v < 0 || v > 3) return fail(ctx, CBL_ERR_ARG, "lbm_variant must be 0, 1, 2 or 3");
     if (v == 3 && (ctx->prec == 0 || ctx->p.tau != 1.0))
       return fail(ctx, CBL_ERR_UNSUPPORTED, "the moment pass needs tau = 1 and FP32 or binary16 storage");
+    if (v != 3) {
+      const cbl_status sm = mom_free(ctx);
+      if (sm != CBL_OK) return sm;
+    }
     ctx->fused_tz = v == 1 ? fused_tz_of(ctx) : 0;
     ctx->acc_pass = v == 2;
     ctx->mom_req = v == 3;
+    ctx->mom_wait = ctx->mom_skip = 0;
   } else if (k == "acc_ty") {
     const int v = (int)value;
     if (v != 8 && v != 16) return fail(ctx, CBL_ERR_ARG, "acc_ty must be 8 or 16");
@@ -1464,6 +1501,7 @@ cbl_status cbl_set_option(cbl_ctx* ctx, const char* key, double value) {
 
 struct cbl_batch {
   std::vector<cbl_ctx*> ctxs;
+  std::vector<std::shared_ptr<int>> held;  // the contexts' counts of batches
   std::vector<cudaStream_t> branches;
   std::vector<cudaEvent_t> events;  // [0] fork, [1..n] joins
   cudaStream_t s = nullptr;
@@ -1748,6 +1786,10 @@ cbl_status cbl_batch_create(cbl_ctx* const* ctxs, int n, void* stream, cbl_batch
   }
   cbl_batch* b = new cbl_batch();
   b->ctxs.assign(ctxs, ctxs + n);
+  for (cbl_ctx* c : b->ctxs) {
+    b->held.push_back(c->batches);
+    ++*c->batches;
+  }
   // the persistent launch serves instances of one precision and velocity set on the split pass
   bool uniform = true;
   for (int k = 0; k < n; ++k)
@@ -1757,7 +1799,7 @@ cbl_status cbl_batch_create(cbl_ctx* const* ctxs, int n, void* stream, cbl_batch
     b->s = (cudaStream_t)stream;
   } else {
     if (cudaStreamCreateWithFlags(&b->s, cudaStreamNonBlocking) != cudaSuccess) {
-      delete b;
+      cbl_batch_destroy(b);
       return fail(nullptr, CBL_ERR_CUDA, "stream");
     }
     b->own_stream = true;
@@ -1860,6 +1902,7 @@ cbl_status cbl_batch_destroy(cbl_batch* b) {
   if (!b) return CBL_OK;
   if (b->s) cudaStreamSynchronize(b->s);
   batch_drop_graphs(b);
+  for (const std::shared_ptr<int>& h : b->held) --*h;
   for (cudaStream_t br : b->branches)
     if (br) cudaStreamDestroy(br);
   for (cudaEvent_t e : b->events)
