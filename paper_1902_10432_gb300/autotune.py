@@ -7,13 +7,15 @@ FP32 at tau = 1 the moment pass. For a batch (tune_batch): the persistent kernel
 shapes 32x4x1, 32x4x4, 32x4x8 and 64x2x4 cells. Each candidate is timed on the simulation it will run
 (three warm-up steps, then CUDA events around a few steps on the simulation's stream; the state
 advances, which does not matter for the choice); the fastest is applied and cached in a JSON file
-keyed by lattice shape, precision, whether bodies are present and the GPU name.
+keyed by lattice shape, precision, velocity set, relaxation time, whether bodies are present and the GPU name.
 """
 from __future__ import annotations
 
 import json
 import os
 import threading
+
+from .cbl import CBL_FP32
 
 CACHE = os.environ.get("CBL_TUNE_CACHE",
                        os.path.join(os.path.dirname(os.path.abspath(__file__)), "_tune_cache.json"))
@@ -24,7 +26,7 @@ def candidates(prec):
     c = [dict(lbm_variant=0, lbm_block_x=bx) for bx in (32, 64, 128)]
     c.append(dict(lbm_variant=1, lbm_block_x=32))
     c += [dict(lbm_variant=2, lbm_block_x=32, acc_ty=ty) for ty in (8, 16)]
-    if prec == "fp32":  # (in binary16 the passes above give the same bits, the moment pass others)
+    if prec in ("fp32", CBL_FP32):  # (in binary16 the passes above give the same bits, the moment pass others)
         c.append(dict(lbm_variant=3, lbm_block_x=32))  # only at tau = 1: left out elsewhere by tune()
     return c
 
@@ -35,8 +37,8 @@ def _key(sim):
     nx = sim.shape[2]
     ny = sim.shape[1]
     nz = sim.shape[0]
-    return "%dx%dx%d/%s/tau%g/%s/%s" % (nx, ny, nz, sim.params["prec"], sim.params["tau"],
-                                        "bodies" if sim.nb else "fluid", torch.cuda.get_device_name())
+    return "%dx%dx%d/%s/q%d/tau%r/%s/%s" % (nx, ny, nz, sim.params["prec"], sim.q, float(sim.params["tau"]),
+                                            "bodies" if sim.nb else "fluid", torch.cuda.get_device_name())
 
 
 def _load():
