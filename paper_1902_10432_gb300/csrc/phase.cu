@@ -868,6 +868,19 @@ __device__ void build_list(BodyDev* bodies, int self, int nb, const Lat& lat, St
   }
 }
 
+// A body at rest without kinetics has nothing to copy: the halo check alone (a move or a turn may have put the
+// field there), on the halo's cells alone: Z planes from z0 on of column t of its tile. (Not inlined: rare.)
+__device__ __noinline__ void resting_halo(const TileSet& S, const BodyDev& b, unsigned t, int z0, int Z) {
+  const int nn[3] = {S.lat.nx, S.lat.ny, S.lat.nz}, L0 = b.L[0], i1 = (int)(t / (unsigned)L0), i0 = (int)(t - (unsigned)i1 * L0);
+  if (i1 >= b.L[1]) return;
+  const size_t plane = (size_t)L0 * b.L[1];
+  const double* const phi = S.arena + b.off + t;
+  bool halo = false;
+  for (int z = z0; z < min(z0 + Z, b.L[2]); ++z)
+    if (tile_halo(b, nn, i0, i1, z)) halo |= (dbits(phi[plane * z]) << 1) > (dbits(PHI_EPS) << 1);
+  if (halo) atomicOr(&S.st->err, E_TILE);
+}
+
 // Cells with a flat stencil keep their value (both face fluxes are u p with the same u, so the update is
 // exactly zero); the others, the interface shell, are collected and updated in full warps. A body at rest
 // changes nothing: its sweeps end at once, but for one copy of the field to where the kinetics reads it.
@@ -903,6 +916,10 @@ __global__ void __launch_bounds__(TILE_T) k_sweep(const __grid_constant__ TileSe
     still &= sh[a] == 0 && (dbits(b.V[a]) << 1) == 0 && (dbits(b.W[a]) << 1) == 0;
   }
   if (still && D != 0) return;
+  if (D == 0 && still && !S.mpf) {
+    resting_halo(S, b, blockIdx.x * TILE_T + threadIdx.x, z0, Z);
+    return;
+  }
   __shared__ TileList list;
   if (threadIdx.x == 0) list.n = 0;
   __syncthreads();
@@ -917,10 +934,6 @@ __global__ void __launch_bounds__(TILE_T) k_sweep(const __grid_constant__ TileSe
   long long frac = 0;
   int ones = 0, shell = 0;
   bool halo = false;
-  auto outer = [&](int c0, int c1, int c2) {
-    return (L0 < nn[0] && (c0 < 2 || c0 >= L0 - 2)) || (L1 < nn[1] && (c1 < 2 || c1 >= L1 - 2)) ||
-           (L2 < nn[2] && (c2 < 2 || c2 >= L2 - 2));
-  };
   auto tally = [&](double v, int c0, int c1, int c2) {
     const long long vb = dbits(v);
     if ((vb << 1) == 0) return;
@@ -941,16 +954,15 @@ __global__ void __launch_bounds__(TILE_T) k_sweep(const __grid_constant__ TileSe
     // scheme leaves a geometrically decaying tail ahead of its front, and the tile drops what
     // reaches past it, so values of at most PHI_EPS there are tolerated
     if ((vb << 1) > (dbits(PHI_EPS) << 1))
-      halo |= outer(c0, c1, c2);
+      halo |= tile_halo(b, nn, c0, c1, c2);
   };
   if (still) {
-    // (without kinetics only the halo is looked at: a field that a move or a turn has put there)
 #pragma unroll
     for (int q = 0; q < Z; ++q)
-      if (pt < plane && z0 + q < L2 && (S.mpf || outer(i0, i1, z0 + q))) {
+      if (pt < plane && z0 + q < L2) {
         const size_t t = pt + (size_t)plane * (z0 + q);
         const double v = in[t];
-        if (S.mpf) out[t] = v;
+        out[t] = v;
         tally(v, i0, i1, z0 + q);
       }
   } else {

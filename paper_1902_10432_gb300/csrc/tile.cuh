@@ -88,6 +88,12 @@ __device__ __forceinline__ long long lat_index(const TileCell& c, const Lat& lat
   return c.gx + (long long)lat.nx * (c.gy + (long long)lat.ny * c.gz);
 }
 
+// the outer two layers of a tile, its stencils' halo (none along an axis that the tile spans)
+__device__ __forceinline__ bool tile_halo(const BodyDev& b, const int nn[3], int i0, int i1, int i2) {
+  return (b.L[0] < nn[0] && (i0 < 2 || i0 >= b.L[0] - 2)) || (b.L[1] < nn[1] && (i1 < 2 || i1 >= b.L[1] - 2)) ||
+         (b.L[2] < nn[2] && (i2 < 2 || i2 >= b.L[2] - 2));
+}
+
 // local index of global cell g in a tile with origin o, or -1 if outside
 __device__ __forceinline__ long long tile_index(const int o[3], const int L[3], int gx, int gy, int gz, const Lat& lat) {
   int a = wrapi_near(gx - o[0], lat.nx), b = wrapi_near(gy - o[1], lat.ny), c = wrapi_near(gz - o[2], lat.nz);
