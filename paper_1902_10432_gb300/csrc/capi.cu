@@ -1790,7 +1790,8 @@ cbl_status cbl_batch_create(cbl_ctx* const* ctxs, int n, void* stream, cbl_batch
     b->held.push_back(c->batches);
     ++*c->batches;
   }
-  // the persistent launch serves instances of one precision and velocity set on the split pass
+  // the persistent launches (one for the instances on the split pass, one for those on the moment pass) serve
+  // one precision and velocity set
   bool uniform = true;
   for (int k = 0; k < n; ++k)
     uniform &= ctxs[k]->prec == ctxs[0]->prec && ctxs[k]->ops.q == ctxs[0]->ops.q && ctxs[k]->fused_tz == 0;
@@ -1842,7 +1843,7 @@ cbl_status cbl_batch_set_option(cbl_batch* b, const char* key, double value) {
     if (v == 1) {
       for (cbl_ctx* c : b->ctxs)
         if (c->prec != b->ctxs[0]->prec || c->ops.q != b->ctxs[0]->ops.q || c->fused_tz)
-          return fail(nullptr, CBL_ERR_UNSUPPORTED, "persistent mode needs one precision and velocity set, split pass");
+          return fail(nullptr, CBL_ERR_UNSUPPORTED, "persistent mode needs one precision and velocity set, split or moment pass");
     }
     b->mode = v;
   } else if (k == "tile") {

@@ -67,13 +67,13 @@ constexpr uint16_t F_OWNER = 0x1FFF;
 constexpr int MAX_BODIES = 0x1FFF;
 constexpr uint16_t F_STALE = 0x1FFF;  // owner id of a cell solid before a body move (never a body)
 constexpr int MAXNB = 24;  // neighbour-list capacity per body (tiles that overlap)
-// Per-body member record (rebuilt by the refill pass from the cells with phi >= the membership
-// threshold): tile-coordinate box lo[3], hi[3], then the bit pattern of the largest squared distance
+// Per-body member record (rebuilt by the flag pass in a step, by the refill pass outside one, from the cells
+// with phi >= the membership threshold): tile-coordinate box lo[3], hi[3], then the bit pattern of the largest squared distance
 // of a member cell from the body's centre X (a non-negative float: its bits order like the value),
 // and one unused word.
 constexpr int MBOX_N = 8, MBOX_R2 = 6;
 
-// Fluid-mass accumulation slots written by the collision kernel and summed by the body kernel.
+// Fluid-mass accumulation slots written by the collision kernels and summed at the end of the step (finish_step).
 constexpr int MASS_SLOTS = 256;
 
 // Device error word bits.

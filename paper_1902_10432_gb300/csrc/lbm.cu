@@ -523,7 +523,7 @@ __device__ __forceinline__ typename St<S>::R collide_fluid(const S* __restrict__
 }
 
 // Block sum of the cells' densities, added into one of MASS_SLOTS slots (spreads the atomics); the
-// body kernel adds the slots in a fixed order and clears them. FP64 values are summed in FP64; FP32
+// step's last kernel adds the slots in a fixed order and clears them (finish_step). FP64 values are summed in FP64; FP32
 // values in compensated float pairs (exact to about 2^-48) up to one FP64 conversion per block
 // (GB300 issues FP64 at 1/64 of the FP32 rate).
 __device__ __forceinline__ void add_mass_slot(double* __restrict__ mass_part, double v, unsigned slot) {
