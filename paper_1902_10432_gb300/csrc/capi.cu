@@ -328,7 +328,8 @@ cbl_status cbl_add_body(cbl_ctx* ctx, const cbl_body* body, int* body_id) {
       L = n[a];
       b.o[a] = 0;
     } else {
-      b.o[a] = (int)std::floor(b.c0[a] + 0.5) - L / 2;
+      // (from the periodic image in the lattice: the kernels wrap a tile's cells by at most two lengths)
+      b.o[a] = (int)std::floor(wrapd(b.c0[a], n[a]) + 0.5) - L / 2;
     }
     b.o_prev[a] = b.o[a];
     b.L[a] = L;
