@@ -665,7 +665,10 @@ static cbl_status acc_prepare(cbl_ctx* ctx) {
 // storage only where it is asked for: the other passes give the same bits there, and this one's FP32 rounding
 // (its velocity starts from the summed momentum, theirs from half the force) crosses binary16 rounding
 // points now and then. The error against FP64 is the same, but the flow carries the differences on: 2e-3 of
-// the velocity's 2-norm after 20 steps of a four-sphere cluster, 2e-2 after 60. It would be 1.3 times as fast.
+// the velocity's 2-norm after 20 steps of a four-sphere cluster, 2e-2 after 60. On 256^3 it would take 11.9 ms
+// for 20 steps instead of 16.8.
+// The line of the cells, with two spheres (us per step, split and moment pass): 0.33 M cells 80 and 88, 0.52 M 95 and
+// 95, 0.64 M 105 and 103, 1.0 M 122 and 116, 2.1 M 182 and 166.
 constexpr long long MOM_MIN_CELLS = 1LL << 19;
 static bool mom_rule(const cbl_ctx* ctx) {
   if (ctx->fused_tz || ctx->acc_pass || ctx->mom_req == 0) return false;
@@ -1555,9 +1558,9 @@ struct BatchBranch {
 // bodies' chain. From BATCH_CHAIN_MIN instances on one launch per kernel serves all of them: a batch of 64
 // pairs of spheres has 14 launches per step instead of 750 on 64 branches (7.5 ms per step; each is too short to
 // fill the GPU and waits for its turn). Fewer instances do not fill the launches, whose latencies add up:
-// their chains run side by side on branches (us per step, one launch and branches: 4 pairs 571 and 505,
-// 6 pairs 790 and 759, 10 pairs 1093 and 1173).
-// So do more bodies than a launch's grid numbers in z.
+// their chains run side by side on branches (us per step, one launch and branches: 2 pairs 331 and 270,
+// 4 pairs 469 and 407, 6 pairs 624 and 628, 8 pairs 815 and 845, 10 pairs 896 and 1002). So do more bodies than
+// a launch's grid numbers in z.
 constexpr int BATCH_CHAIN_MIN = 8, BATCH_CHAIN_BODIES = 65535;
 static cudaError_t batch_enqueue(cbl_batch* b, int diag) {
   cbl_ctx* c0 = b->ctxs[0];
@@ -1665,7 +1668,7 @@ static cbl_status batch_states(cbl_batch* b) {
 
 // Planes per work item of the moment pass, at most the tile's: an item computes two more than it completes, the
 // blocks share them all out, and the last ones end half an item apart on average (as mom_sz). With 32 planes
-// whatever the batch, a step of two pairs took 442 us, of four 536; 266 and 410 so.
+// whatever the batch, a step of two pairs takes 315 us, of four 421; 271 and 412 so.
 static int batch_planes(const cbl_batch* b, const int tile[3]) {
   int best = tile[2];
   double best_cost = 1e300;
