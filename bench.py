@@ -59,10 +59,12 @@ def batch_kernels_per_step(variants):
 # ncu captures (gpu__time_duration, dram__bytes_read/write only), valid only for the source they were
 # taken on (source_hash of the lattice-Boltzmann sources); None otherwise
 PROFILED = {
-    ("tetra4", "fp32", 19, "f516674d3bf5"): 729.4e6,       # k_mom<float>, mean of 2 launches
+    ("tetra4", "fp32", 19, "8f9a0455b1fe"): 730.3e6,       # k_mom<float>, mean of 2 launches
+    ("tetra4", "fp16dev", 19, "8f9a0455b1fe"): 1347.9e6,   # k_collide<__half>, mean of 2 launches
 }
 PROFILED_STEP = {
-    ("tetra4", "fp32", 19, "f516674d3bf5"): 867.7e6,       # every kernel of one step
+    ("tetra4", "fp32", 19, "8f9a0455b1fe"): 868.6e6,       # every kernel of one step
+    ("tetra4", "fp16dev", 19, "8f9a0455b1fe"): 2177.4e6,
 }
 
 
